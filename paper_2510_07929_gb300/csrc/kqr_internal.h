@@ -251,6 +251,8 @@ kqr_status precond_update(Handle* h, const double* Lpre, double gam, double rtol
 cudaError_t precond_apply(Handle* h, const double* Ldiag, const double* r, double* out, double* rz_out,
                           cudaStream_t st);
 kqr_status rpcholesky_setup(Handle* h, const double* uniforms);
+// Inverse of an SPD matrix over all SMs (spd_inverse.cu): G overwritten, W scratch, all N x N.
+cudaError_t spd_inverse(Handle* h, double* G, double* W, double* Ginv, int N, int* info, cudaStream_t st);
 
 // ---- solver (solver.cu) --------------------------------------------------------
 kqr_status solve(Handle* h, double tau, double lam, double tol, kqr_info* info);

@@ -99,64 +99,6 @@ __global__ void add_diag_kernel(double* G, int N, double v, double last) {
   GRID_LOOP(i, N) G[i * N + i] += (i == N - 1) ? last : v;
 }
 
-// In-place lower Cholesky of the N x N row-major matrix (single CTA).
-// info[0] = 0 on success, j + 1 if pivot j was not positive.
-__global__ void __launch_bounds__(1024) cholesky_kernel(double* G, int N, int* info) {
-  __shared__ double piv;
-  __shared__ int bad;
-  if (threadIdx.x == 0) bad = 0;
-  __syncthreads();
-  for (int j = 0; j < N; ++j) {
-    if (threadIdx.x == 0) {
-      const double d = G[(size_t)j * N + j];
-      if (!(d > 0.0)) {
-        bad = j + 1;
-        piv = 1.0;
-      } else {
-        piv = sqrt(d);
-      }
-      G[(size_t)j * N + j] = piv;
-    }
-    __syncthreads();
-    if (bad) break;
-    const double inv = 1.0 / piv;
-    for (int i = j + 1 + threadIdx.x; i < N; i += blockDim.x) G[(size_t)i * N + j] *= inv;
-    __syncthreads();
-    // trailing update of the lower triangle, one warp per row
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int i = j + 1 + (int)(threadIdx.x >> 5); i < N; i += nw) {
-      const double gij = G[(size_t)i * N + j];
-      for (int k = j + 1 + lane; k <= i; k += 32) G[(size_t)i * N + k] -= gij * G[(size_t)k * N + j];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *info = bad;
-}
-
-// W = L^{-1} (lower) from the Cholesky factor stored in the lower triangle of G;
-// one thread per column of W (single CTA).  W is written to Winv.
-__global__ void __launch_bounds__(1024) tri_inverse_kernel(const double* G, int N, double* W) {
-  for (int c = threadIdx.x; c < N; c += blockDim.x) {
-    for (int i = 0; i < c; ++i) W[(size_t)i * N + c] = 0.0;
-    for (int i = c; i < N; ++i) {
-      double s = (i == c) ? 1.0 : 0.0;
-      for (int k = c; k < i; ++k) s -= G[(size_t)i * N + k] * W[(size_t)k * N + c];
-      W[(size_t)i * N + c] = s / G[(size_t)i * N + i];
-    }
-  }
-}
-
-// Ginv = W^T W (symmetric), one output entry per thread.
-__global__ void wtw_kernel(const double* W, int N, double* Ginv) {
-  GRID_LOOP(e, (int64_t)N * N) {
-    const int a = (int)(e / N), b = (int)(e % N);
-    const int i0 = a > b ? a : b;
-    double s = 0.0;
-    for (int i = i0; i < N; ++i) s += W[(size_t)i * N + a] * W[(size_t)i * N + b];
-    Ginv[e] = s;
-  }
-}
-
 __global__ void recip_kernel(double* out, const double* L, int64_t n) { GRID_LOOP(i, n) out[i] = 1.0 / L[i]; }
 
 // t[a] += sum_i U_ai (Linv_i r_i) over a chunk of 2048 rows and 8 columns of U = [F 1].
@@ -310,19 +252,12 @@ kqr_status precond_build(Handle* h, const double* Lpre, double gam, cudaStream_t
   add_diag_kernel<<<grid_for(N), 256, 0, st>>>(G, N, 1.0, 1.0 / gam);
   h->launches++;
   int* info = reinterpret_cast<int*>(h->scal + S_COUNT - 1);
-  cholesky_kernel<<<1, 1024, 0, st>>>(G, N, info);
-  h->launches++;
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(h, e, "cholesky");
+  if ((e = spd_inverse(h, G, W, Ginv, N, info, st)) != cudaSuccess) return cuda_fail(h, e, "core inverse");
   int hinfo = 0;
   if ((e = cudaMemcpyAsync(&hinfo, info, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
       (e = cudaStreamSynchronize(st)) != cudaSuccess)
-    return cuda_fail(h, e, "cholesky info");
+    return cuda_fail(h, e, "core inverse info");
   if (hinfo != 0) return fail(h, KQR_BREAKDOWN, "Woodbury core not positive definite at pivot " + std::to_string(hinfo - 1));
-  tri_inverse_kernel<<<1, 1024, 0, st>>>(G, N, W);
-  h->launches++;
-  wtw_kernel<<<grid_for((int64_t)N * N), 256, 0, st>>>(W, N, Ginv);
-  h->launches++;
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(h, e, "core inverse");
   h->core_valid = true;
   return KQR_OK;
 }

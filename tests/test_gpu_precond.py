@@ -1,0 +1,48 @@
+"""The Woodbury core's blocked inverse through kqr_precond_apply_dev (Lemma 1), at ranks around
+the edges of its 32 x 32 blocks and of its doubling steps, against the FP64 oracle."""
+import numpy as np
+import pytest
+
+from oracle import kqr_oracle as O
+from paper_2510_07929_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def K_():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_07929_gb300 import build
+
+    build.build()
+    from paper_2510_07929_gb300 import kqr
+
+    return kqr
+
+
+def woodbury_error(K_, n, rank, L, gam, seed):
+    import torch
+
+    wl = W.lap_large(n=n, p=20, seed=seed)
+    with K_.Problem(wl.X, wl.y, wl.kind, wl.gamma, rank0=rank, adaptive_rank=0,
+                    pivot_uniforms=W.pivot_uniforms(max(rank, 2))) as prob:
+        F, _, r, _ = prob.factor()
+        assert r == rank
+        rv = np.random.default_rng(seed).standard_normal(n)
+        out = torch.empty(n, dtype=torch.float64, device="cuda")
+        prob.precond_apply_dev(torch.from_numpy(L).cuda(), gam, torch.from_numpy(rv).cuda(), out)
+    ref = O.woodbury_apply(F.astype(np.float64), L, gam, rv)
+    return np.max(np.abs(out.cpu().numpy() - ref)) / np.max(np.abs(ref))
+
+
+# The core is I + U^T L^{-1} U with L in [0.5, 1.5]: condition at most ~4 n (the constant mode), so
+# both sides' FP64 errors stay below 4 n N 2^-53 = 4e-10 at n = 1200, N = 700.
+@pytest.mark.parametrize("rank", [1, 2, 30, 31, 32, 33, 62, 63, 64, 95, 96, 130, 255, 256, 700])
+def test_core_inverse_at_block_edges(K_, rank):
+    n = 1200
+    L = np.random.default_rng(rank).uniform(0.5, 1.5, n)
+    assert woodbury_error(K_, n, rank, L, 0.3, seed=rank) <= 4e-10
+
