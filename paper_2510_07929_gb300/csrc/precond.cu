@@ -26,71 +26,180 @@ namespace kqr {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n); i += (int64_t)gridDim.x * blockDim.x)
 
 // ---- weighted Gram of the columns of U = [F, 1] (optional ones column) -----------
-// G[a][b] += sum_{i in chunk} U_ai U_bi w_i for a 32 x 32 tile pair (ta <= tb).
-constexpr int kCT = 32;    // core tile
-constexpr int kCR = 32;    // rows per shared-memory step
-constexpr int kChunk = 4096;
+// G[a][b] = sum_i U_ai (w_i U_bi), FP64-class on the FP32 pipe.
+//
+// On the FP64 pipe (2 FMAs per clock and SM) the r^2 n / 2 products of a core cost 21 ms at
+// n = 20011, r = 1024, and a conversion of F besides.  Here a product is an FP32 factor (F
+// itself, exact) times a double-float (w U, or F of the set-up, as hi + lo): 11 FP32 pipe
+// operations with the TwoSum accumulation, 128 lanes per clock and SM instead of 2.  The
+// double-float sums run over kCgRows rows only and are then added to FP64 sums: their rounding
+// error grows with the square of the rows summed, and at 32 rows it is below that of the long
+// FP64 sum it replaces (64 rows: 6.6 instead of 7.2 ms, but a larger error).  w is scaled by the power of two that
+// brings its maximum to [1, 2), so that hi and lo stay inside the FP32 range.
+//
+// Tile: 64 x 64 entries per CTA of 128 threads, 4 x 8 per thread (32 independent chains; the
+// operands of a row are 20 shared-memory words for 352 FP32 operations).  The rows are cut into
+// chunks so that about two waves of CTAs exist at every (n, r): with a fixed chunk of 4096 rows
+// a rank-45 core at n = 2000 ran on 3 CTAs (707 us, now 26).  n = 20011, r = 1024: 21.1 ms
+// before, 7.2 ms now; the FP32 pipe alone would take 3.4 ms, the rest is the operand split and
+// the FP64 additions.
+constexpr int kCT = 64;      // core tile
+constexpr int kCR = 16;      // rows per shared-memory step
+constexpr int kCgRows = 32;  // rows per double-float sum
+constexpr int kCgThreads = 128;
 
+__device__ __forceinline__ void df_split(double x, float& hi, float& lo) {
+  hi = (float)x;
+  lo = (float)(x - (double)hi);
+}
+
+// T: float (the FP32 factor, weights w; both triangles of G are written) or double (the set-up's FP64 factor, no weights).
 template <typename T>
-__global__ void __launch_bounds__(256) core_gram_kernel(const T* __restrict__ F, int rr, int ncols, int64_t n,
-                                                        const double* __restrict__ w, double* __restrict__ G,
-                                                        int ntile) {
+__global__ void __launch_bounds__(kCgThreads, 3)
+    core_gram_kernel(const T* __restrict__ F, int rr, int ncols, int64_t n, const double* __restrict__ w,
+                     const unsigned long long* __restrict__ wmax, double* __restrict__ G, int ntile,
+                     int64_t chunk) {
+  constexpr bool kPair = sizeof(T) == 8;   // the left operand needs its low part too
   // blockIdx.x enumerates tile pairs (ta <= tb), blockIdx.y row chunks.
   int pair = blockIdx.x, ta = 0;
   while (pair >= ntile - ta) { pair -= ntile - ta; ++ta; }
   const int tb = ta + pair;
-  __shared__ double Ua[kCR][kCT + 1];
-  __shared__ double Ub[kCR][kCT + 1];
+  __shared__ __align__(16) float Ah[kCR][kCT + 4];
+  __shared__ __align__(16) float Al[kPair ? kCR : 1][kCT + 4];
+  __shared__ __align__(16) float Bh[kCR][kCT + 4];
+  __shared__ __align__(16) float Bl[kCR][kCT + 4];
   const int tid = threadIdx.x;
-  const int la = tid / 8;          // 0..31: row of the 32x32 output tile
-  const int lb0 = (tid % 8) * 4;   // 4 consecutive columns
-  double acc[4] = {0, 0, 0, 0};
-  const int64_t i0 = (int64_t)blockIdx.y * kChunk;
-  const int64_t i1 = min(n, i0 + kChunk);
-  for (int64_t ib = i0; ib < i1; ib += kCR) {
-    __syncthreads();
-    for (int e = tid; e < kCR * kCT; e += 256) {
-      const int rrow = e / kCT, c = e % kCT;
-      const int64_t i = ib + rrow;
-      const int ca = ta * kCT + c, cb = tb * kCT + c;
-      double ua = 0.0, ub = 0.0;
-      if (i < i1) {
-        const double wi = w ? w[i] : 1.0;
-        ua = ca < rr ? (double)F[(size_t)ca * n + i] : (ca < ncols ? 1.0 : 0.0);
-        ub = cb < rr ? (double)F[(size_t)cb * n + i] : (cb < ncols ? 1.0 : 0.0);
-        ua *= wi;
+  const int la = (tid >> 3) * 4;   // 4 rows of the tile
+  const int lb = (tid & 7) * 4;    // columns lb .. lb + 3 and 32 + lb ..
+  double scale = 1.0, unscale = 1.0;
+  if (wmax) {
+    const int ex = (int)((*wmax >> 52) & 0x7ff);   // biased exponent of max w
+    if (ex > 0 && ex < 2046) {
+      scale = __longlong_as_double((long long)(2046 - ex) << 52);   // 2^(1023 - ex)
+      unscale = __longlong_as_double((long long)ex << 52);
+    }
+  }
+  __shared__ float2 wsplit[kCgRows];   // w_i scaled, as hi + lo (float T)
+  double tot[4][8];
+  float sl[4][8];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      tot[a][b] = 0.0;
+      sl[a][b] = 0.f;
+    }
+  const int64_t i0 = (int64_t)blockIdx.y * chunk;
+  const int64_t i1 = min(n, i0 + chunk);
+  for (int64_t ig = i0; ig < i1; ig += kCgRows) {
+    float sh[4][8];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 8; ++b) sh[a][b] = 0.f;
+    if (!kPair) {
+      __syncthreads();
+      if (tid < kCgRows) {
+        const double wi = ig + tid < i1 ? (w ? w[ig + tid] * scale : 1.0) : 0.0;
+        float hi, lo;
+        df_split(wi, hi, lo);
+        wsplit[tid] = make_float2(hi, lo);
       }
-      Ua[rrow][c] = ua;
-      Ub[rrow][c] = ub;
     }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < kCR; ++k) {
-      const double a = Ua[k][la];
+    for (int64_t ib = ig; ib < min(i1, ig + kCgRows); ib += kCR) {
+      __syncthreads();
+      // lanes along the rows of a column (F is column-major): 16 rows x 2 columns per warp load
+      for (int e = tid; e < kCR * kCT; e += kCgThreads) {
+        const int k = e % kCR, c = e / kCR;
+        const int64_t i = ib + k;
+        const int ca = ta * kCT + c, cb = tb * kCT + c;
+        T ua = 0, ub = 0;
+        if (i < i1) {
+          ua = ca < rr ? F[(size_t)ca * n + i] : (T)(ca < ncols ? 1 : 0);
+          ub = cb < rr ? F[(size_t)cb * n + i] : (T)(cb < ncols ? 1 : 0);
+        }
+        if (kPair) {
+          df_split((double)ua, Ah[k][c], Al[kPair ? k : 0][c]);
+          df_split((double)ub, Bh[k][c], Bl[k][c]);
+        } else {
+          const float2 wi = wsplit[(int)(ib - ig) + k];
+          const float u = (float)ub, bh = __fmul_rn(wi.x, u);
+          Ah[k][c] = (float)ua;
+          Bh[k][c] = bh;
+          Bl[k][c] = fmaf(wi.y, u, fmaf(wi.x, u, -bh));
+        }
+      }
+      __syncthreads();
+#pragma unroll 2
+      for (int k = 0; k < kCR; ++k) {
+        const float4 a4 = *reinterpret_cast<const float4*>(&Ah[k][la]);
+        const float4 h0 = *reinterpret_cast<const float4*>(&Bh[k][lb]);
+        const float4 h1 = *reinterpret_cast<const float4*>(&Bh[k][32 + lb]);
+        const float4 l0 = *reinterpret_cast<const float4*>(&Bl[k][lb]);
+        const float4 l1 = *reinterpret_cast<const float4*>(&Bl[k][32 + lb]);
+        const float xa[4] = {a4.x, a4.y, a4.z, a4.w};
+        float xl[4] = {0.f, 0.f, 0.f, 0.f};
+        if (kPair) {
+          const float4 q = *reinterpret_cast<const float4*>(&Al[kPair ? k : 0][la]);
+          xl[0] = q.x; xl[1] = q.y; xl[2] = q.z; xl[3] = q.w;
+        }
+        const float yh[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+        const float yl[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fma(a, Ub[k][lb0 + q], acc[q]);
-    }
-  }
-  const int a = ta * kCT + la;
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int b = tb * kCT + lb0 + q;
-    if (a < ncols && b < ncols) {
-      atomicAdd(&G[(size_t)a * ncols + b], acc[q]);
-      if (ta != tb) atomicAdd(&G[(size_t)b * ncols + a], acc[q]);
+          for (int b = 0; b < 8; ++b) {
+            const float p = __fmul_rn(xa[a], yh[b]);
+            float e = fmaf(xa[a], yh[b], -p);
+            e = fmaf(xa[a], yl[b], e);
+            if (kPair) e = fmaf(xl[a], yh[b], e);
+            // TwoSum
+            const float s = __fadd_rn(sh[a][b], p);
+            const float bb = __fsub_rn(s, sh[a][b]);
+            const float er = __fadd_rn(__fsub_rn(sh[a][b], __fsub_rn(s, bb)), __fsub_rn(p, bb));
+            sh[a][b] = s;
+            sl[a][b] = __fadd_rn(sl[a][b], __fadd_rn(er, e));
+          }
+      }
     }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        // renormalise, so that one FP64 addition takes all but a remainder below half an ulp of it
+        const float v = __fadd_rn(sh[a][b], sl[a][b]);
+        sl[a][b] = __fsub_rn(sl[a][b], __fsub_rn(v, sh[a][b]));
+        tot[a][b] += (double)v;
+      }
   }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const int ra = ta * kCT + la + a, cb = tb * kCT + (b < 4 ? lb + b : 28 + lb + b);
+      if (ra < ncols && cb < ncols) {
+        const double v = (tot[a][b] + (double)sl[a][b]) * unscale;
+        atomicAdd(&G[(size_t)ra * ncols + cb], v);
+        if (ta != tb) atomicAdd(&G[(size_t)cb * ncols + ra], v);
+      }
+    }
 }
 
+// wmax (device, nullable): max_i w_i, for the scaling of the weights.
 template <typename T>
-static cudaError_t core_gram(Handle* h, const T* F, int rr, bool ones, const double* w, double* G, cudaStream_t st) {
+static cudaError_t core_gram(Handle* h, const T* F, int rr, bool ones, const double* w,
+                             const unsigned long long* wmax, double* G, cudaStream_t st) {
   const int ncols = rr + (ones ? 1 : 0);
   cudaError_t e = cudaMemsetAsync(G, 0, sizeof(double) * ncols * ncols, st);
   if (e != cudaSuccess) return e;
   const int ntile = (ncols + kCT - 1) / kCT;
   const int pairs = ntile * (ntile + 1) / 2;
-  const int chunks = (int)((h->n + kChunk - 1) / kChunk);
-  core_gram_kernel<T><<<dim3(pairs, chunks), 256, 0, st>>>(F, rr, ncols, h->n, w, G, ntile);
+  // about 6 CTAs per SM (two waves of 3 resident ones), chunks of a multiple of kCgRows rows
+  const int64_t want = ((int64_t)6 * h->num_sms + pairs - 1) / pairs;
+  int64_t chunk = (h->n + want - 1) / want;
+  chunk = (chunk + kCgRows - 1) / kCgRows * kCgRows;
+  const int chunks = (int)((h->n + chunk - 1) / chunk);
+  core_gram_kernel<T><<<dim3(pairs, chunks), kCgThreads, 0, st>>>(F, rr, ncols, h->n, w, wmax, G, ntile, chunk);
   h->launches++;
   return cudaGetLastError();
 }
@@ -99,7 +208,17 @@ __global__ void add_diag_kernel(double* G, int N, double v, double last) {
   GRID_LOOP(i, N) G[i * N + i] += (i == N - 1) ? last : v;
 }
 
-__global__ void recip_kernel(double* out, const double* L, int64_t n) { GRID_LOOP(i, n) out[i] = 1.0 / L[i]; }
+// out = 1 / L and the bits of its maximum (non-negative doubles order like their bits).
+__global__ void recip_kernel(double* out, const double* L, int64_t n, unsigned long long* __restrict__ wmax) {
+  double m = 0.0;
+  GRID_LOOP(i, n) {
+    const double v = 1.0 / L[i];
+    out[i] = v;
+    m = fmax(m, v);
+  }
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(wmax, (unsigned long long)__double_as_longlong(m));
+}
 
 // t[a] += sum_i U_ai (Linv_i r_i) over a chunk of 2048 rows and 8 columns of U = [F 1].
 __global__ void __launch_bounds__(256) ut_kernel(const float* __restrict__ F, int r, int64_t n,
@@ -246,9 +365,11 @@ kqr_status precond_build(Handle* h, const double* Lpre, double gam, cudaStream_t
   double* W = h->core + (size_t)N * N;       // N x N, L^{-1}
   double* Ginv = W + (size_t)N * N;          // N x N
   cudaError_t e;
-  recip_kernel<<<grid_for(h->n), 256, 0, st>>>(h->Linv, Lpre, h->n);
+  unsigned long long* wmax = reinterpret_cast<unsigned long long*>(h->scal + S_COUNT - 2);
+  if ((e = cudaMemsetAsync(wmax, 0, sizeof(*wmax), st)) != cudaSuccess) return cuda_fail(h, e, "core");
+  recip_kernel<<<grid_for(h->n), 256, 0, st>>>(h->Linv, Lpre, h->n, wmax);
   h->launches++;
-  if ((e = core_gram<float>(h, h->F32, h->r, true, h->Linv, G, st)) != cudaSuccess) return cuda_fail(h, e, "core");
+  if ((e = core_gram<float>(h, h->F32, h->r, true, h->Linv, wmax, G, st)) != cudaSuccess) return cuda_fail(h, e, "core");
   add_diag_kernel<<<grid_for(N), 256, 0, st>>>(G, N, 1.0, 1.0 / gam);
   h->launches++;
   int* info = reinterpret_cast<int*>(h->scal + S_COUNT - 1);
@@ -624,7 +745,7 @@ kqr_status rpcholesky_setup(Handle* h, const double* uniforms) {
     double* xw = A + (size_t)rr0 * rr0;
     double* yw = xw + rr0;
     double* lam1 = yw + rr0;
-    core_gram<double>(h, F64, rr0, false, nullptr, A, st);
+    core_gram<double>(h, F64, rr0, false, nullptr, nullptr, A, st);
     power_iter_kernel<<<1, 512, 0, st>>>(A, rr0, xw, yw, 2000, lam1);
     h->launches++;
     double hl1 = 0.0;
@@ -634,7 +755,6 @@ kqr_status rpcholesky_setup(Handle* h, const double* uniforms) {
       cleanup();
       return cuda_fail(h, e, "power iteration");
     }
-    core_gram<double>(h, F64, rr0, false, nullptr, A, st);
     inertia_kernel<<<1, 1024, 0, st>>>(A, rr0, h->opt.xi * hl1, bad + 1);
     h->launches++;
     int neg = 0;

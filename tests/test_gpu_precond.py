@@ -46,3 +46,13 @@ def test_core_inverse_at_block_edges(K_, rank):
     L = np.random.default_rng(rank).uniform(0.5, 1.5, n)
     assert woodbury_error(K_, n, rank, L, 0.3, seed=rank) <= 4e-10
 
+
+# Weights from 1e-30 to 1e12 (their products leave the FP32 range without the power-of-two scaling), ranks
+# at the edges of the 64 x 64 tiles, rows at the edges of the 64-row sums.  Bound: the one of the Lemma 1
+# test (both sides solve with a core whose condition is at most that of L^-1 times that of U^T U).
+@pytest.mark.parametrize("n,rank", [(64, 5), (65, 63), (127, 64), (1000, 65), (1537, 128), (4099, 129)])
+@pytest.mark.parametrize("low", [1e-12, 1e-2, 1e30])
+def test_core_gram_at_tile_edges(K_, n, rank, low):
+    rng = np.random.default_rng(rank)
+    L = low * rng.uniform(1.0, 10.0, n)
+    assert woodbury_error(K_, n, rank, L, 0.3, seed=rank) <= 1e-8
