@@ -430,141 +430,199 @@ __global__ void chunk_sum_kernel(const double* __restrict__ d, int64_t n, int64_
 }
 
 // ---- fused RPCholesky steps ---------------------------------------------------------
-// One launch per pivot.  CTA b owns rows [b * kRpcChunk, (b + 1) * kRpcChunk); step t
-// forms column t of F for the pivot s = piv[t] chosen by the previous launch, updates the
-// residual diagonal and writes its chunk's sum of the new diagonal; the last CTA to finish
-// (a ticket counter, no waiting) draws the next pivot from the chunk sums.  state[0] is
-// the stop flag, state[1] the number of columns produced, state[2] the ticket counter.
-constexpr int kRpcChunk = 512;
-constexpr int kRpcThreads = 256;
+// One launch per pivot.  CTA b owns R = blockDim.x rows, one per thread; step t forms column t
+// of F for the pivot s = piv[t] chosen by the previous launch, updates the residual diagonal
+// and writes its chunk's sum of the new diagonal; the last CTA to finish (a ticket counter, no
+// waiting) draws the next pivot from the chunk sums.  state[0] is the stop flag, state[1] the
+// number of columns produced, state[2] the ticket counter.
+//
+// What bounds a step: at large n the FP64 pipe (t + 2 p FMAs per row at 2 per clock and SM;
+// the 8 t n bytes of F take two thirds of that), at small n the latency chain of one row and
+// of the draw.  So rows are spread one per thread over R = 64 rows per CTA while that fills at
+// most one wave (128 beyond), the pivot's residual is d[s] itself (the running diagonal is
+// updated by the very operations that would recompute it), and the draw is a scan by all
+// threads of the last CTA.  n = 10000, p = 50, t < 100: 141 us a step before (512 rows per
+// CTA, one thread scanning them from global memory).
+constexpr int kRpcMaxThreads = 128;
 
-// Residual column entry g_i = k(x_i, x_s) - sum_{c<t} F[c][i] F[c][s]; every CTA calls it
-// for row s too, so the pivot's g_s is bit-identical to the one its own row computes.
+static int rpc_rows(const Handle* h) { return h->n <= (int64_t)64 * h->num_sms ? 64 : kRpcMaxThreads; }
+
+// Residual column entry g_i = k(x_i, x_s) - sum_{c<t} F[c][i] F[c][s].
 __device__ __forceinline__ double rpc_entry(const double* __restrict__ xc, int64_t ldn, int p, double gamma, int lap,
                                             const double* __restrict__ F, int64_t n, int t, int64_t i,
                                             const double* xs, const double* fs) {
   double dist = 0.0;
+#pragma unroll 8
   for (int k = 0; k < p; ++k) {
     const double v = xc[(size_t)k * ldn + i] - xs[k];
     dist = lap ? dist + fabs(v) : fma(v, v, dist);
   }
   double acc = exp(-gamma * dist);
+#pragma unroll 16
   for (int c = 0; c < t; ++c) acc -= F[(size_t)c * n + i] * fs[c];
   return acc;
 }
 
-// Pivot draw by the last CTA: the smallest s with running sum of d > u * sum(d), the
-// sums taken chunk by chunk in a fixed order.  Thread 0 only.
+// Inclusive sum over the CTA's threads (blockDim.x a multiple of 32, at most kRpcMaxThreads);
+// *total receives the sum over all of them.  Contains barriers.
+__device__ __forceinline__ double rpc_scan(double v, double* ws, double* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += u;
+  }
+  __syncthreads();
+  if (lane == 31) ws[warp] = v;
+  __syncthreads();
+  double base = 0.0, all = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    if (w < warp) base += ws[w];
+    all += ws[w];
+  }
+  *total = all;
+  return base + v;
+}
+
+// Pivot draw by the last CTA: the smallest s with running sum of d > u * sum(d), among the
+// rows with d > 0 (the scan's rounding must not select an exhausted row).  Chunk sums first
+// (threads take contiguous runs of them), then the rows of the chosen chunk.
 __device__ void rpc_pick(const double* d, const double* csum, int64_t n, int nchunks, double u, long long* piv_out,
-                         int* state) {
-  double total = 0.0;
-  for (int c = 0; c < nchunks; ++c) total += __ldcg(csum + c);
+                         double* val_out, int* state) {
+  __shared__ double ws[kRpcMaxThreads / 32];
+  __shared__ int first;
+  __shared__ int chunk_sh;
+  __shared__ double run_sh;
+  const int T = blockDim.x, tid = threadIdx.x;
+  const int per = (nchunks + T - 1) / T;
+  const int c0 = min(nchunks, tid * per), c1 = min(nchunks, c0 + per);
+  double mine = 0.0;
+#pragma unroll 4
+  for (int c = c0; c < c1; ++c) mine += __ldcg(csum + c);
+  double total;
+  const double incl = rpc_scan(mine, ws, &total);
   if (!(total > 0.0)) {
-    *piv_out = -1;
-    state[0] = 1;
+    if (tid == 0) {
+      *piv_out = -1;
+      state[0] = 1;
+    }
     return;
   }
   const double target = u * total;
-  double run = 0.0;
-  int c = 0;
-  for (; c < nchunks - 1; ++c) {
-    const double cs = __ldcg(csum + c);
-    if (run + cs > target) break;
-    run += cs;
+  if (tid == 0) {
+    first = T;
+    chunk_sh = nchunks - 1;
+    run_sh = -INFINITY;   // stays if rounding left the target past the last chunk: no row qualifies
   }
-  int64_t s = (int64_t)c * kRpcChunk;
-  const int64_t end = min(n, s + kRpcChunk);
-  int64_t found = -1;
-  for (; s < end; ++s) {
-    run += __ldcg(d + s);
-    if (run > target) {
-      found = s;
-      break;
+  __syncthreads();
+  if (c1 > c0 && incl > target) atomicMin(&first, tid);
+  __syncthreads();
+  if (tid == first) {
+    double run = incl - mine;
+    int c = c0;
+    for (; c < c1 - 1; ++c) {
+      const double cs = __ldcg(csum + c);
+      if (run + cs > target) break;
+      run += cs;
     }
+    chunk_sh = c;
+    run_sh = run;
   }
-  if (found < 0) {  // rounding left the target past the last positive entry: take the last positive one
-    for (int64_t q = n - 1; q >= 0; --q)
-      if (__ldcg(d + q) > 0.0) {
-        found = q;
-        break;
-      }
+  __syncthreads();
+  const int64_t row = (int64_t)chunk_sh * T + tid;
+  const double dv = row < n ? __ldcg(d + row) : 0.0;
+  double dummy;
+  const double at = run_sh + rpc_scan(dv, ws, &dummy);
+  if (tid == 0) first = T;
+  __syncthreads();
+  if (dv > 0.0 && at > target) atomicMin(&first, tid);
+  __syncthreads();
+  if (first < T) {
+    if (tid == first) {
+      *piv_out = row;
+      *val_out = dv;
+    }
+  } else if (tid == 0) {   // rounding left the target past the last positive entry: take the last positive one
+    int64_t q = n - 1;
+    while (q > 0 && !(__ldcg(d + q) > 0.0)) --q;
+    *piv_out = q;
+    *val_out = __ldcg(d + q);
   }
-  *piv_out = found;
 }
 
 __device__ __forceinline__ void rpc_chunk_sum_and_ticket(double local, double* csum, const double* d, int64_t n,
                                                          int nchunks, const double* u, int t, int r0,
-                                                         long long* piv, int* state) {
-  __shared__ double ws[kRpcThreads / 32];
+                                                         long long* piv, double* pval, int* state) {
+  __shared__ double cs_ws[kRpcMaxThreads / 32];
   __shared__ int last;
   for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = local;
+  if ((threadIdx.x & 31) == 0) cs_ws[threadIdx.x >> 5] = local;
+  __threadfence();   // this thread's d and F entry before the ticket
   __syncthreads();
   if (threadIdx.x == 0) {
     double v = 0.0;
-    for (int w = 0; w < kRpcThreads / 32; ++w) v += ws[w];
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += cs_ws[w];
     csum[blockIdx.x] = v;
     __threadfence();
     last = atomicAdd(state + 2, 1) == nchunks - 1;
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
+  if (last) {
     __threadfence();
-    state[2] = 0;
-    state[1] = t + 1;
-    if (t + 1 < r0) rpc_pick(d, csum, n, nchunks, u[t + 1], piv + t + 1, state);
+    if (threadIdx.x == 0) {
+      state[2] = 0;
+      state[1] = t + 1;
+    }
+    if (t + 1 < r0) rpc_pick(d, csum, n, nchunks, u[t + 1], piv + t + 1, pval + t + 1, state);
   }
 }
 
 // d = diag(K) = 1 and the draw of the first pivot.
-__global__ void rpc_init_kernel(double* __restrict__ d, int64_t n, int nchunks, double* __restrict__ csum,
-                                const double* __restrict__ u, int r0, long long* __restrict__ piv,
-                                int* __restrict__ state) {
-  const int64_t i0 = (int64_t)blockIdx.x * kRpcChunk;
-  const int64_t i1 = min(n, i0 + kRpcChunk);
+__global__ void __launch_bounds__(kRpcMaxThreads) rpc_init_kernel(double* __restrict__ d, int64_t n, int nchunks,
+                                                                 double* __restrict__ csum,
+                                                                 const double* __restrict__ u, int r0,
+                                                                 long long* __restrict__ piv,
+                                                                 double* __restrict__ pval, int* __restrict__ state) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double local = 0.0;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += kRpcThreads) {
+  if (i < n) {
     d[i] = 1.0;   // k(x, x) = 1 for the RBF and Laplacian kernels
-    local += 1.0;
+    local = 1.0;
   }
-  rpc_chunk_sum_and_ticket(local, csum, d, n, nchunks, u, -1, r0, piv, state);
+  rpc_chunk_sum_and_ticket(local, csum, d, n, nchunks, u, -1, r0, piv, pval, state);
 }
 
-__global__ void __launch_bounds__(kRpcThreads) rpc_step_kernel(const double* __restrict__ xc, int64_t ldn, int p,
-                                                              double gamma, int lap, double* __restrict__ F,
+__global__ void __launch_bounds__(kRpcMaxThreads) rpc_step_kernel(const double* __restrict__ xc, int64_t ldn, int p,
+                                                              double gamma, int lap, double* F,
                                                               double* __restrict__ d, int64_t n, int t, int r0,
                                                               int nchunks, double* __restrict__ csum,
                                                               const double* __restrict__ u,
-                                                              long long* __restrict__ piv, int* __restrict__ state) {
+                                                              long long* __restrict__ piv,
+                                                              double* __restrict__ pval, int* __restrict__ state) {
   if (*(volatile int*)state) return;   // an earlier step stopped the factorization
   const long long s = piv[t];
-  extern __shared__ double sm[];
-  double* fs = sm;            // F[c][s], c < t
-  double* xs = sm + t;        // x_s
-  __shared__ double gs_sh;
-  for (int c = threadIdx.x; c < t; c += kRpcThreads) fs[c] = F[(size_t)c * n + s];
-  for (int k = threadIdx.x; k < p; k += kRpcThreads) xs[k] = xc[(size_t)k * ldn + s];
-  __syncthreads();
-  if (threadIdx.x == 0) gs_sh = rpc_entry(xc, ldn, p, gamma, lap, F, n, t, s, xs, fs);
-  __syncthreads();
-  const double gs = gs_sh;
-  if (!(gs > 0.0)) {     // the residual at the pivot vanished: stop with t columns
+  const double gs = pval[t];   // residual at the pivot
+  if (!(gs > 0.0)) {           // it vanished: stop with t columns
     if (blockIdx.x == 0 && threadIdx.x == 0) state[0] = 1;
     return;
   }
+  extern __shared__ double sm[];
+  double* fs = sm;            // F[c][s], c < t
+  double* xs = sm + t;        // x_s
+  for (int c = threadIdx.x; c < t; c += blockDim.x) fs[c] = F[(size_t)c * n + s];
+  for (int k = threadIdx.x; k < p; k += blockDim.x) xs[k] = xc[(size_t)k * ldn + s];
+  __syncthreads();
   const double inv = 1.0 / sqrt(gs);
-  const int64_t i0 = (int64_t)blockIdx.x * kRpcChunk;
-  const int64_t i1 = min(n, i0 + kRpcChunk);
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double local = 0.0;
-  double* Ft = F + (size_t)t * n;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += kRpcThreads) {
+  if (i < n) {
     const double f = rpc_entry(xc, ldn, p, gamma, lap, F, n, t, i, xs, fs) * inv;
-    Ft[i] = f;
+    F[(size_t)t * n + i] = f;
     const double di = fmax(d[i] - f * f, 0.0);
     d[i] = di;
-    local += di;
+    local = di;
   }
-  rpc_chunk_sum_and_ticket(local, csum, d, n, nchunks, u, t, r0, piv, state);
+  rpc_chunk_sum_and_ticket(local, csum, d, n, nchunks, u, t, r0, piv, pval, state);
 }
 
 __global__ void to_float_kernel(const double* __restrict__ src, float* __restrict__ dst, int64_t cnt) {
@@ -683,13 +741,15 @@ kqr_status rpcholesky_setup(Handle* h, const double* uniforms) {
   }
   const int64_t chunk = (n + kPivChunks - 1) / kPivChunks;
   const int nchunks = (int)((n + chunk - 1) / chunk);
-  const int rchunks = (int)((n + kRpcChunk - 1) / kRpcChunk);
+  const int rrows = rpc_rows(h);
+  const int rchunks = (int)((n + rrows - 1) / rrows);
   double* u_dev = (double*)dev_alloc(h, sizeof(double) * (r0 + 1));
   double* rsum = (double*)dev_alloc(h, sizeof(double) * (rchunks + 1));
+  double* piv_val = (double*)dev_alloc(h, sizeof(double) * (r0 + 1));
   long long* piv_all = (long long*)dev_alloc(h, sizeof(long long) * (r0 + 1));
   int* state = (int*)dev_alloc(h, sizeof(int) * 4);
-  auto cleanup2 = [&]() { dev_free(h, u_dev); dev_free(h, rsum); dev_free(h, piv_all); dev_free(h, state); };
-  if (!u_dev || !rsum || !piv_all || !state) {
+  auto cleanup2 = [&]() { dev_free(h, u_dev); dev_free(h, rsum); dev_free(h, piv_val); dev_free(h, piv_all); dev_free(h, state); };
+  if (!u_dev || !rsum || !piv_val || !piv_all || !state) {
     cleanup2();
     cleanup();
     return fail(h, KQR_OOM, "RPCholesky workspace");
@@ -709,12 +769,11 @@ kqr_status rpcholesky_setup(Handle* h, const double* uniforms) {
     cleanup();
     return cuda_fail(h, e, "RPCholesky start");
   }
-  rpc_init_kernel<<<rchunks, kRpcThreads, 0, st>>>(d, n, rchunks, rsum, u_dev, r0, piv_all, state);
+  rpc_init_kernel<<<rchunks, rrows, 0, st>>>(d, n, rchunks, rsum, u_dev, r0, piv_all, piv_val, state);
   h->launches++;
   for (int t = 0; t < r0; ++t) {
-    rpc_step_kernel<<<rchunks, kRpcThreads, smem, st>>>(h->xc64, h->ldn, (int)h->p, h->gamma,
-                                                        h->kind == KQR_LAPLACIAN, F64, d, n, t, r0, rchunks, rsum,
-                                                        u_dev, piv_all, state);
+    rpc_step_kernel<<<rchunks, rrows, smem, st>>>(h->xc64, h->ldn, (int)h->p, h->gamma, h->kind == KQR_LAPLACIAN,
+                                                  F64, d, n, t, r0, rchunks, rsum, u_dev, piv_all, piv_val, state);
     h->launches++;
   }
   int hstate[4] = {0, 0, 0, 0};

@@ -56,3 +56,16 @@ def test_core_gram_at_tile_edges(K_, n, rank, low):
     rng = np.random.default_rng(rank)
     L = low * rng.uniform(1.0, 10.0, n)
     assert woodbury_error(K_, n, rank, L, 0.3, seed=rank) <= 1e-8
+
+
+@pytest.mark.parametrize("kind,n,r0", [("laplacian", 2, 2), ("rbf", 63, 9), ("laplacian", 64, 20), ("rbf", 129, 30),
+                                       ("laplacian", 9728, 24), ("rbf", 9729, 24), ("laplacian", 13001, 16)])
+def test_rpcholesky_pivots_at_chunk_edges(K_, kind, n, r0):
+    """Pivot draws against the oracle (same uniforms) where the rows per CTA change and where chunks are ragged."""
+    wl = W.lap_large(n=n, p=7, seed=n) if kind == "laplacian" else W.rbf_mid(n=n, p=7, seed=n)
+    u = W.pivot_uniforms(r0, seed=5)
+    with K_.Problem(wl.X, wl.y, kind, wl.gamma, rank0=r0, adaptive_rank=0, pivot_uniforms=u, gram_store=0) as prob:
+        F, piv, r, _ = prob.factor()
+    F0, piv_o = O.rpcholesky(lambda s: O.gram(wl.X, wl.X[s:s + 1], kind, wl.gamma)[:, 0], np.ones(n), r0, u)
+    np.testing.assert_array_equal(piv, piv_o)
+    np.testing.assert_allclose(F, F0[:, :r], atol=2e-6 * np.max(np.abs(F0)))
