@@ -185,7 +185,7 @@ bool make_tmap_rowmajor_bf16_sw128(CUtensorMap* tm, void* base, int64_t ldn) {
 
 static void free_all(Handle* h) {
   void* bufs[] = {h->xs32, h->nrm32, h->hq, h->hl, h->exp_table, h->xc64, h->y, h->F32, h->dres, h->core, h->tvec,
-                  h->Linv, h->part, h->v32, h->vec_pool, h->scal, h->red_counter, h->red_part, h->err_flag,
+                  h->Linv, h->usplit, h->part, h->v32, h->vec_pool, h->scal, h->red_counter, h->red_part, h->err_flag,
                   h->st_alpha, h->st_v, h->st_z, h->sym_units, h->tc_hi, h->tc_lo, h->tc_bf, h->tc_sym_units, h->tc_a16, h->tc_b16};
   for (void* b : bufs) dev_free(h, b);
   kstore_free(h);
@@ -775,7 +775,8 @@ kqr_status kqr_get_factor(kqr_handle* kh, float* F, int64_t* pivots, int32_t* ra
   if (pivots)
     for (size_t i = 0; i < h->pivots.size(); ++i) pivots[i] = h->pivots[i];
   if (F && h->r > 0) {
-    if (cudaMemcpy(F, h->F32, sizeof(float) * (size_t)h->r * h->n, cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (cudaMemcpy2D(F, sizeof(float) * h->n, h->F32, sizeof(float) * h->ldn, sizeof(float) * h->n, h->r,
+                     cudaMemcpyDeviceToHost) != cudaSuccess)
       return fail(h, KQR_CUDA_ERROR, "copy factor");
   }
   return KQR_OK;

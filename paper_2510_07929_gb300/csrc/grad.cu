@@ -226,7 +226,7 @@ static kqr_status adjoint_cg(Handle* h, const double* L, const double* Lpre, dou
   AK(reduce(h, RED_NORM2, rn, n, dsc + 0, st));
   AK(get(0));
   if (std::sqrt(hs[0]) <= tol) return KQR_OK;
-  AK(precond_apply(h, Lpre, r, z, dsc + 1, st));
+  AK(precond_apply(h, Lpre, r, z, dsc + 1, st, dsc + 0));
   AK(get(1));
   double rz = hs[1];
   AK(vec_copy(h, p, z, n, st));
@@ -250,7 +250,7 @@ static kqr_status adjoint_cg(Handle* h, const double* L, const double* Lpre, dou
     AK(reduce(h, RED_NORM2, rn, n, dsc + 0, st));
     AK(get(0));
     if (std::sqrt(hs[0]) <= tol) break;
-    AK(precond_apply(h, Lpre, r, z, dsc + 1, st));
+    AK(precond_apply(h, Lpre, r, z, dsc + 1, st, dsc + 0));
     AK(get(1));
     adj_dir_kernel<<<grid_for(n), 256, 0, st>>>(p, z, hs[1] / rz, n);
     AK(cudaGetLastError());

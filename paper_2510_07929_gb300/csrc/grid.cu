@@ -300,6 +300,7 @@ static Handle* column_clone(Handle* base, GridRdv* g, kqr_status* st) {
   c->core = (double*)dev_alloc(base, sizeof(double) * 3 * (size_t)N * N);
   c->tvec = (double*)dev_alloc(base, sizeof(double) * 2 * N);
   c->Linv = (double*)dev_alloc(base, sizeof(double) * c->n);
+  c->usplit = (float2*)dev_alloc(base, sizeof(float2) * c->ldn);
   c->st_alpha = (double*)dev_alloc(base, sizeof(double) * c->ldn);
   c->st_v = (double*)dev_alloc(base, sizeof(double) * c->ldn);
   c->st_z = (double*)dev_alloc(base, sizeof(double) * c->ldn);
@@ -307,7 +308,7 @@ static Handle* column_clone(Handle* base, GridRdv* g, kqr_status* st) {
   c->has_state = false;
   *st = KQR_OK;
   if (!c->vec_pool || !c->scal || !c->red_counter || !c->red_part || !c->err_flag || !c->core || !c->tvec ||
-      !c->Linv || !c->st_alpha || !c->st_v || !c->st_z) {
+      !c->Linv || !c->usplit || !c->st_alpha || !c->st_v || !c->st_z) {
     *st = KQR_OOM;
     return c;
   }
@@ -330,7 +331,7 @@ static void column_free(Handle* base, Handle* c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream);
   void* bufs[] = {c->vec_pool, c->scal, c->red_counter, c->red_part, c->err_flag, c->core,
-                  c->tvec, c->Linv, c->st_alpha, c->st_v, c->st_z};
+                  c->tvec, c->Linv, c->usplit, c->st_alpha, c->st_v, c->st_z};
   for (void* b : bufs) dev_free(base, b);
   if (c->scal_host) cudaFreeHost(c->scal_host);
   if (c->rdv_ev) cudaEventDestroy(c->rdv_ev);

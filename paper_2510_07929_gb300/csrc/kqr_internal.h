@@ -101,7 +101,7 @@ struct Handle {
   double* xc64 = nullptr;
   double* y = nullptr;
 
-  // RPCholesky factor, column-major [r][n] (column c at F32 + c * n).
+  // RPCholesky factor, column-major [r][ldn] (column c at F32 + c * ldn, padding rows zero).
   int r0 = 0, r = 0;
   float* F32 = nullptr;
   double* dres = nullptr;             // residual diagonal diag(K - F F^T), FP32 factor
@@ -109,7 +109,8 @@ struct Handle {
 
   // Woodbury core (r + 1)^2, its Cholesky factor and work vectors.
   double* core = nullptr;
-  double* tvec = nullptr;             // r + 1
+  double* tvec = nullptr;             // U^T L^{-1} r (r + 1), then the core's result as hi + lo floats (r + 1)
+  float2* usplit = nullptr;           // L^{-1} r scaled, as hi + lo floats (ldn)
   double* Linv = nullptr;             // n
   bool core_valid = false;
   double core_gam = 0.0;              // gam the current core was built for
@@ -249,7 +250,7 @@ kqr_status precond_build(Handle* h, const double* Ldiag, double gam, cudaStream_
 // its distance to the exact P changes).  Lcore_i = 1 / Linv_i.
 kqr_status precond_update(Handle* h, const double* Lpre, double gam, double rtol, cudaStream_t st);
 cudaError_t precond_apply(Handle* h, const double* Ldiag, const double* r, double* out, double* rz_out,
-                          cudaStream_t st);
+                          cudaStream_t st, const double* rr = nullptr);
 kqr_status rpcholesky_setup(Handle* h, const double* uniforms);
 // Inverse of an SPD matrix over all SMs (spd_inverse.cu): G overwritten, W scratch, all N x N.
 cudaError_t spd_inverse(Handle* h, double* G, double* W, double* Ginv, int N, int* info, cudaStream_t st);
@@ -296,7 +297,9 @@ enum Scal {
   S_RED0 = 0, S_SUMP = 16, S_PAP = 17, S_A = 18, S_BETA = 19, S_RR = 20, S_RZ = 21,
   // device-resident CG control (solver.cu): new rz, status, iterations, tol^2, pending status, maxit
   S_RZN = 22, S_CGST = 23, S_CGITS = 24, S_TOL2 = 25, S_PEND = 26, S_MAXIT = 27, S_GAM = 28, S_PP = 29,
-  S_COUNT = 32
+  // preconditioner: bits of max L^{-1}, exponent that scales the current r, max |r| where the caller gives no norm
+  S_WMAX = 30, S_WEXP = 31, S_WMAXR = 32,
+  S_COUNT = 40
 };
 
 // Launch configuration for element-wise kernels.

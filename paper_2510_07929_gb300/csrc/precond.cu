@@ -13,7 +13,8 @@
 //   P^{-1} = L^{-1} - L^{-1} U (C + U^T L^{-1} U)^{-1} U^T L^{-1},
 //   U = [F 1], C = diag(I_r, 1/gam),
 // with the (r+1)^2 core built in FP64, Cholesky-factorised and inverted on the
-// device; each apply is two skinny FP64 products with the FP32 factor.
+// device; each apply is two skinny FP64-class products with the FP32 factor.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -56,7 +57,7 @@ __device__ __forceinline__ void df_split(double x, float& hi, float& lo) {
 // T: float (the FP32 factor, weights w; both triangles of G are written) or double (the set-up's FP64 factor, no weights).
 template <typename T>
 __global__ void __launch_bounds__(kCgThreads, 3)
-    core_gram_kernel(const T* __restrict__ F, int rr, int ncols, int64_t n, const double* __restrict__ w,
+    core_gram_kernel(const T* __restrict__ F, int64_t ldf, int rr, int ncols, int64_t n, const double* __restrict__ w,
                      const unsigned long long* __restrict__ wmax, double* __restrict__ G, int ntile,
                      int64_t chunk) {
   constexpr bool kPair = sizeof(T) == 8;   // the left operand needs its low part too
@@ -115,8 +116,8 @@ __global__ void __launch_bounds__(kCgThreads, 3)
         const int ca = ta * kCT + c, cb = tb * kCT + c;
         T ua = 0, ub = 0;
         if (i < i1) {
-          ua = ca < rr ? F[(size_t)ca * n + i] : (T)(ca < ncols ? 1 : 0);
-          ub = cb < rr ? F[(size_t)cb * n + i] : (T)(cb < ncols ? 1 : 0);
+          ua = ca < rr ? F[(size_t)ca * ldf + i] : (T)(ca < ncols ? 1 : 0);
+          ub = cb < rr ? F[(size_t)cb * ldf + i] : (T)(cb < ncols ? 1 : 0);
         }
         if (kPair) {
           df_split((double)ua, Ah[k][c], Al[kPair ? k : 0][c]);
@@ -187,7 +188,7 @@ __global__ void __launch_bounds__(kCgThreads, 3)
 
 // wmax (device, nullable): max_i w_i, for the scaling of the weights.
 template <typename T>
-static cudaError_t core_gram(Handle* h, const T* F, int rr, bool ones, const double* w,
+static cudaError_t core_gram(Handle* h, const T* F, int64_t ldf, int rr, bool ones, const double* w,
                              const unsigned long long* wmax, double* G, cudaStream_t st) {
   const int ncols = rr + (ones ? 1 : 0);
   cudaError_t e = cudaMemsetAsync(G, 0, sizeof(double) * ncols * ncols, st);
@@ -199,7 +200,7 @@ static cudaError_t core_gram(Handle* h, const T* F, int rr, bool ones, const dou
   int64_t chunk = (h->n + want - 1) / want;
   chunk = (chunk + kCgRows - 1) / kCgRows * kCgRows;
   const int chunks = (int)((h->n + chunk - 1) / chunk);
-  core_gram_kernel<T><<<dim3(pairs, chunks), kCgThreads, 0, st>>>(F, rr, ncols, h->n, w, wmax, G, ntile, chunk);
+  core_gram_kernel<T><<<dim3(pairs, chunks), kCgThreads, 0, st>>>(F, ldf, rr, ncols, h->n, w, wmax, G, ntile, chunk);
   h->launches++;
   return cudaGetLastError();
 }
@@ -220,43 +221,157 @@ __global__ void recip_kernel(double* out, const double* L, int64_t n, unsigned l
   if ((threadIdx.x & 31) == 0) atomicMax(wmax, (unsigned long long)__double_as_longlong(m));
 }
 
-// t[a] += sum_i U_ai (Linv_i r_i) over a chunk of 2048 rows and 8 columns of U = [F 1].
-__global__ void __launch_bounds__(256) ut_kernel(const float* __restrict__ F, int r, int64_t n,
-                                                 const double* __restrict__ Linv, const double* __restrict__ rv,
-                                                 double* __restrict__ t) {
-  const int c0 = blockIdx.y * 8;
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  const int64_t base = (int64_t)blockIdx.x * 2048;
-  for (int q = 0; q < 8; ++q) {
-    const int64_t i = base + q * 256 + threadIdx.x;
-    if (i >= n) break;
-    const double wi = Linv[i] * rv[i];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int col = c0 + c;
-      if (col < r) acc[c] = fma((double)F[(size_t)col * n + i], wi, acc[c]);
-      else if (col == r) acc[c] += wi;
-    }
+// ---- apply of Lemma 1 -----------------------------------------------------------------
+// out = L^{-1} (r - U G^{-1} U^T L^{-1} r): two passes over the FP32 factor F (r n entries each)
+// around a product with the (r + 1)^2 core inverse.
+//
+// What bounds it: reading F twice (80 MB each at n = 20011, r = 1024: from L2, beyond that from
+// HBM).  On the FP64 pipe the two passes cost 2 r n FMAs at 2 per clock and SM plus a conversion
+// of every F entry at the same rate, 160 and 334 us at that size with the latency of one thread
+// per row.  Here every product is FP32 x double-float (11 FP32-pipe operations, as in the core):
+// L^{-1} r and the core's result are split once into hi + lo, after scaling by powers of two
+// (the exponent of ||r|| and of max L^{-1}) that keep both parts inside the FP32 range for any r.
+// Sums run in double-float over at most 32 terms between renormalisations and are combined in
+// FP64.  Measured (n = 20011, r = 1024, cold caches): 37 and 68 us.
+__device__ __forceinline__ int norm_exponent(double rr, bool is_max) {   // e with 2^e about sqrt(rr), or rr
+  const int ex = (int)((__double_as_longlong(rr) >> 52) & 0x7ff) - 1023;
+  return is_max ? max(-1000, min(1000, ex)) : ex >> 1;
+}
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+__device__ __forceinline__ int max_exponent(unsigned long long wmax) {   // of max L^{-1}; 0 if it is not a normal number
+  const int ex = (int)((wmax >> 52) & 0x7ff);
+  return ex > 0 && ex < 2046 ? ex - 1023 : 0;
+}
+
+// (sh, sl) += x (yh + yl), x FP32.
+__device__ __forceinline__ void df_mac(float& sh, float& sl, float x, float yh, float yl) {
+  const float p = __fmul_rn(x, yh);
+  const float e = fmaf(x, yl, fmaf(x, yh, -p));
+  const float s = __fadd_rn(sh, p);
+  const float bb = __fsub_rn(s, sh);
+  const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+  sh = s;
+  sl = __fadd_rn(sl, __fadd_rn(er, e));
+}
+// (sh, sl) += (yh, yl), renormalised.
+__device__ __forceinline__ void df_add(float& sh, float& sl, float yh, float yl) {
+  const float s = __fadd_rn(sh, yh);
+  const float bb = __fsub_rn(s, sh);
+  const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(yh, bb));
+  const float l = __fadd_rn(__fadd_rn(sl, yl), er);
+  sh = __fadd_rn(s, l);
+  sl = __fsub_rn(l, __fsub_rn(sh, s));
+}
+__device__ __forceinline__ void df_renorm(float& sh, float& sl) {
+  const float v = __fadd_rn(sh, sl);
+  sl = __fsub_rn(sl, __fsub_rn(v, sh));
+  sh = v;
+}
+
+// bits of max |r|
+__global__ void absmax_kernel(const double* __restrict__ rv, int64_t n, unsigned long long* __restrict__ out) {
+  double m = 0.0;
+  GRID_LOOP(i, n) m = fmax(m, fabs(rv[i]));
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
+}
+
+// us = L^{-1} r scaled, as hi + lo (rows >= n: 0); t = 0; the exponent used for r into scal[S_WEXP].
+__global__ void __launch_bounds__(256) wb_split_kernel(const double* __restrict__ Linv, const double* __restrict__ rv,
+                                                       int64_t n, int64_t ldn, const double* __restrict__ rr,
+                                                       int is_max, double* __restrict__ scal, float2* __restrict__ us,
+                                                       double* __restrict__ t, int N) {
+  const int e = norm_exponent(*rr, is_max != 0);
+  const double sr = pow2(-e);
+  const double sw = pow2(-max_exponent(*reinterpret_cast<const unsigned long long*>(scal + S_WMAX)));
+  GRID_LOOP(i, ldn) {
+    float2 v = make_float2(0.f, 0.f);
+    if (i < n) df_split((Linv[i] * sw) * (rv[i] * sr), v.x, v.y);
+    us[i] = v;
   }
-  __shared__ double ws[8][8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    double v = acc[c];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) ws[warp][c] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < 8 && c0 + (int)threadIdx.x <= r) {
-    double v = 0.0;
-    for (int w = 0; w < 8; ++w) v += ws[w][threadIdx.x];
-    atomicAdd(&t[c0 + threadIdx.x], v);
+  if (blockIdx.x == 0) {
+    for (int c = threadIdx.x; c < N; c += blockDim.x) t[c] = 0.0;
+    if (threadIdx.x == 0) scal[S_WEXP] = (double)e;
   }
 }
 
-// t2 = Ginv t (N x N times N), one block per output row.
+// t[a] += sum_i U_ai (L^{-1} r)_i over `rows` rows (a multiple of 128) and 32 columns of U = [F 1]:
+// a warp takes four columns, a lane four consecutive rows per step.
+__global__ void __launch_bounds__(256) ut_kernel(const float* __restrict__ F, int64_t ldf, int r,
+                                                 const float2* __restrict__ us, const double* __restrict__ scal,
+                                                 double* __restrict__ t, int rows) {
+  extern __shared__ __align__(16) float su[];   // hi[rows], lo[rows]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i0 = (int64_t)blockIdx.x * rows;
+  const int cnt = (int)min((int64_t)rows, ldf - i0);   // a multiple of 128
+  for (int e = threadIdx.x; e < cnt; e += 256) {
+    const float2 v = us[i0 + e];
+    su[e] = v.x;
+    su[rows + e] = v.y;
+  }
+  __syncthreads();
+  const int c0 = blockIdx.y * 32 + warp * 4;
+  if (c0 > r) return;
+  float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
+  const float* Fc[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) Fc[c] = F + (size_t)min(c0 + c, r > 0 ? r - 1 : 0) * ldf + i0;
+  const float4 one = make_float4(1.f, 1.f, 1.f, 1.f), zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+  for (int k = lane * 4; k < cnt; k += 128) {
+    float4 f[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      f[c] = c0 + c < r ? __ldg(reinterpret_cast<const float4*>(Fc[c] + k)) : (c0 + c == r ? one : zero);
+    const float4 uh = *reinterpret_cast<const float4*>(su + k);
+    const float4 ul = *reinterpret_cast<const float4*>(su + rows + k);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      df_mac(sh[c], sl[c], f[c].x, uh.x, ul.x);
+      df_mac(sh[c], sl[c], f[c].y, uh.y, ul.y);
+      df_mac(sh[c], sl[c], f[c].z, uh.z, ul.z);
+      df_mac(sh[c], sl[c], f[c].w, uh.w, ul.w);
+    }
+  }
+  // reduce-scatter: lane bits 4 and 3 select the column, then the lanes of a column are added
+#pragma unroll
+  for (int c = 0; c < 4; ++c) df_renorm(sh[c], sl[c]);
+  const bool u4 = (lane & 16) != 0, u3 = (lane & 8) != 0;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const float gh = __shfl_xor_sync(0xffffffffu, u4 ? sh[c] : sh[c + 2], 16);
+    const float gl = __shfl_xor_sync(0xffffffffu, u4 ? sl[c] : sl[c + 2], 16);
+    if (u4) {
+      sh[c] = sh[c + 2];
+      sl[c] = sl[c + 2];
+    }
+    df_add(sh[c], sl[c], gh, gl);
+  }
+  {
+    const float gh = __shfl_xor_sync(0xffffffffu, u3 ? sh[0] : sh[1], 8);
+    const float gl = __shfl_xor_sync(0xffffffffu, u3 ? sl[0] : sl[1], 8);
+    if (u3) {
+      sh[0] = sh[1];
+      sl[0] = sl[1];
+    }
+    df_add(sh[0], sl[0], gh, gl);
+  }
+#pragma unroll
+  for (int o = 4; o >= 1; o >>= 1) {
+    const float gh = __shfl_xor_sync(0xffffffffu, sh[0], o);
+    const float gl = __shfl_xor_sync(0xffffffffu, sl[0], o);
+    df_add(sh[0], sl[0], gh, gl);
+  }
+  const int col = c0 + (u4 ? 2 : 0) + (u3 ? 1 : 0);
+  if ((lane & 7) == 0 && col <= r) {
+    const int ew = max_exponent(*reinterpret_cast<const unsigned long long*>(scal + S_WMAX));
+    atomicAdd(&t[col], (((double)sh[0] + (double)sl[0]) * pow2((int)scal[S_WEXP])) * pow2(ew));
+  }
+}
+
+// t2s = Ginv t (N x N times N) scaled by the exponent of r, as hi + lo; one block per output row.
 __global__ void gemv_core_kernel(const double* __restrict__ Ginv, const double* __restrict__ t, int N,
-                                 double* __restrict__ t2) {
+                                 const double* __restrict__ scal, float2* __restrict__ t2s) {
   const int a = blockIdx.x;
   double s = 0.0;
   for (int b = threadIdx.x; b < N; b += blockDim.x) s += Ginv[(size_t)a * N + b] * t[b];
@@ -267,37 +382,92 @@ __global__ void gemv_core_kernel(const double* __restrict__ Ginv, const double* 
   if (threadIdx.x == 0) {
     double v = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += ws[w];
-    t2[a] = v;
+    float2 q;
+    df_split(v * pow2(-(int)scal[S_WEXP]), q.x, q.y);
+    t2s[a] = q;
   }
 }
 
-// out_i = Linv_i (r_i - (F t2_F)_i - t2_r); rz += r_i out_i.
-__global__ void __launch_bounds__(256) woodbury_out_kernel(const float* __restrict__ F, int r, int64_t n,
+// out_i = Linv_i (r_i - (F t2_F)_i - t2_r); rz = r . out (the last block to finish adds the blocks'
+// sums).  A CTA takes 32 rows at a time (lane = row), its eight warps an eighth of the columns each.
+constexpr int kOutMaxBlocks = 1216;
+__global__ void __launch_bounds__(256) woodbury_out_kernel(const float* __restrict__ F, int64_t ldf, int r, int64_t n,
                                                            const double* __restrict__ Linv,
                                                            const double* __restrict__ rv,
-                                                           const double* __restrict__ t2, double* __restrict__ out,
+                                                           const float2* __restrict__ t2s,
+                                                           const double* __restrict__ scal, double* __restrict__ out,
+                                                           double* __restrict__ part,
+                                                           unsigned int* __restrict__ counter,
                                                            double* __restrict__ rz) {
-  extern __shared__ double ts[];
-  for (int c = threadIdx.x; c <= r; c += blockDim.x) ts[c] = t2[c];
+  extern __shared__ float2 ts[];   // r + 1
+  __shared__ float2 red[2][8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int c = threadIdx.x; c <= r; c += 256) ts[c] = t2s[c];
   __syncthreads();
+  const int per = (r + 7) / 8;
+  const int c0 = min(r, warp * per), c1 = min(r, c0 + per);
+  const double unscale = pow2((int)scal[S_WEXP]);
   double dot = 0.0;
-  GRID_LOOP(i, n) {
-    double s = ts[r];
-    for (int c = 0; c < r; ++c) s = fma((double)F[(size_t)c * n + i], ts[c], s);
-    const double o = Linv[i] * (rv[i] - s);
-    out[i] = o;
-    dot += rv[i] * o;
-  }
-  if (rz) {
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    __shared__ double ws[8];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = dot;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double v = 0.0;
-      for (int w = 0; w < 8; ++w) v += ws[w];
-      atomicAdd(rz, v);
+  int buf = 0;
+  for (int64_t base = (int64_t)blockIdx.x * 32; base < n; base += (int64_t)gridDim.x * 32, buf ^= 1) {
+    const int64_t i = base + lane;   // < ldf
+    const float* Fi = F + i;
+    double li = 0.0, ri = 0.0;
+    if (warp == 0 && i < n) {
+      li = Linv[i];
+      ri = rv[i];
     }
+    float sh = 0.f, sl = 0.f;
+    int c = c0;
+    for (; c + 16 <= c1; c += 16) {
+      float f[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) f[u] = __ldg(Fi + (size_t)(c + u) * ldf);
+#pragma unroll
+      for (int u = 0; u < 16; ++u) df_mac(sh, sl, f[u], ts[c + u].x, ts[c + u].y);
+      df_renorm(sh, sl);
+    }
+#pragma unroll 4
+    for (; c < c1; ++c) df_mac(sh, sl, __ldg(Fi + (size_t)c * ldf), ts[c].x, ts[c].y);
+    df_renorm(sh, sl);
+    red[buf][warp][lane] = make_float2(sh, sl);
+    __syncthreads();
+    if (warp == 0) {
+      sh = ts[r].x;
+      sl = ts[r].y;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) df_add(sh, sl, red[buf][w][lane].x, red[buf][w][lane].y);
+      if (i < n) {
+        const double o = li * (ri - ((double)sh + (double)sl) * unscale);
+        out[i] = o;
+        dot = fma(ri, o, dot);
+      }
+    }
+  }
+  if (!rz) return;
+  __shared__ bool last;
+  if (warp == 0) {
+    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    if (lane == 0) {
+      part[blockIdx.x] = dot;
+      __threadfence();
+      last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double v = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) v += __ldcg(part + b);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __shared__ double ws[8];
+  if (lane == 0) ws[warp] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double tot = 0.0;
+    for (int w = 0; w < 8; ++w) tot += ws[w];
+    *rz = tot;
+    *counter = 0u;
   }
 }
 
@@ -365,11 +535,11 @@ kqr_status precond_build(Handle* h, const double* Lpre, double gam, cudaStream_t
   double* W = h->core + (size_t)N * N;       // N x N, L^{-1}
   double* Ginv = W + (size_t)N * N;          // N x N
   cudaError_t e;
-  unsigned long long* wmax = reinterpret_cast<unsigned long long*>(h->scal + S_COUNT - 2);
+  unsigned long long* wmax = reinterpret_cast<unsigned long long*>(h->scal + S_WMAX);
   if ((e = cudaMemsetAsync(wmax, 0, sizeof(*wmax), st)) != cudaSuccess) return cuda_fail(h, e, "core");
   recip_kernel<<<grid_for(h->n), 256, 0, st>>>(h->Linv, Lpre, h->n, wmax);
   h->launches++;
-  if ((e = core_gram<float>(h, h->F32, h->r, true, h->Linv, wmax, G, st)) != cudaSuccess) return cuda_fail(h, e, "core");
+  if ((e = core_gram<float>(h, h->F32, h->ldn, h->r, true, h->Linv, wmax, G, st)) != cudaSuccess) return cuda_fail(h, e, "core");
   add_diag_kernel<<<grid_for(N), 256, 0, st>>>(G, N, 1.0, 1.0 / gam);
   h->launches++;
   int* info = reinterpret_cast<int*>(h->scal + S_COUNT - 1);
@@ -383,14 +553,15 @@ kqr_status precond_build(Handle* h, const double* Lpre, double gam, cudaStream_t
   return KQR_OK;
 }
 
-// out = P^{-1} r with the core built by precond_build for the same Lpre; rz_out
-// (device, nullable, zeroed here) receives r^T out.
+// out = P^{-1} r with the core built by precond_build for the same Lpre; rz_out (device,
+// nullable) receives r^T out.  rr (device, nullable): ||r||^2, for the scaling of the double-float
+// parts; without it max |r| is computed here.
 cudaError_t precond_apply(Handle* h, const double* Lpre, const double* rv, double* out, double* rz_out,
-                          cudaStream_t st) {
+                          cudaStream_t st, const double* rr) {
   (void)Lpre;
   cudaError_t e;
-  if (rz_out && (e = cudaMemsetAsync(rz_out, 0, sizeof(double), st)) != cudaSuccess) return e;
   if (h->opt.precond == KQR_PRECOND_NONE) {
+    if (rz_out && (e = cudaMemsetAsync(rz_out, 0, sizeof(double), st)) != cudaSuccess) return e;
     ident_dot_kernel<<<grid_for(h->n), 256, 0, st>>>(rv, out, h->n, rz_out);
     h->launches++;
     return cudaGetLastError();
@@ -398,15 +569,29 @@ cudaError_t precond_apply(Handle* h, const double* Lpre, const double* rv, doubl
   const int N = h->r + 1;
   const double* Ginv = h->core + 2 * (size_t)N * N;
   double* t = h->tvec;
-  double* t2 = h->tvec + N;
-  if ((e = cudaMemsetAsync(t, 0, sizeof(double) * N, st)) != cudaSuccess) return e;
-  ut_kernel<<<dim3((unsigned)((h->n + 2047) / 2048), (N + 7) / 8), 256, 0, st>>>(h->F32, h->r, h->n, h->Linv, rv, t);
-  h->launches++;
-  gemv_core_kernel<<<N, 256, 0, st>>>(Ginv, t, N, t2);
-  h->launches++;
-  woodbury_out_kernel<<<grid_for(h->n), 256, (size_t)N * sizeof(double), st>>>(h->F32, h->r, h->n, h->Linv, rv, t2,
-                                                                                out, rz_out);
-  h->launches++;
+  float2* t2s = reinterpret_cast<float2*>(h->tvec + N);
+  const int is_max = rr ? 0 : 1;
+  if (!rr) {
+    double* slot = h->scal + S_WMAXR;
+    if ((e = cudaMemsetAsync(slot, 0, sizeof(double), st)) != cudaSuccess) return e;
+    absmax_kernel<<<grid_for(h->n), 256, 0, st>>>(rv, h->n, reinterpret_cast<unsigned long long*>(slot));
+    h->launches++;
+    rr = slot;
+  }
+  wb_split_kernel<<<grid_for(h->ldn), 256, 0, st>>>(h->Linv, rv, h->n, h->ldn, rr, is_max, h->scal, h->usplit, t, N);
+  // rows per CTA of the first pass: about four CTAs per SM, 128 .. 1024 rows
+  const int groups = (N + 31) / 32;
+  const int64_t want = std::max<int64_t>(1, (int64_t)4 * h->num_sms / groups);
+  int64_t rows = (h->ldn / 128 + want - 1) / want * 128;
+  rows = std::min<int64_t>(std::max<int64_t>(rows, 128), 1024);
+  ut_kernel<<<dim3((unsigned)((h->ldn + rows - 1) / rows), groups), 256, (size_t)rows * 2 * sizeof(float), st>>>(
+      h->F32, h->ldn, h->r, h->usplit, h->scal, t, (int)rows);
+  gemv_core_kernel<<<N, 256, 0, st>>>(Ginv, t, N, h->scal, t2s);
+  const int blocks = (int)std::min<int64_t>((h->n + 31) / 32, kOutMaxBlocks);
+  woodbury_out_kernel<<<blocks, 256, (size_t)N * sizeof(float2), st>>>(h->F32, h->ldn, h->r, h->n, h->Linv, rv, t2s,
+                                                                       h->scal, out, h->red_part, h->red_counter,
+                                                                       rz_out);
+  h->launches += 4;
   return cudaGetLastError();
 }
 
@@ -625,15 +810,20 @@ __global__ void __launch_bounds__(kRpcMaxThreads) rpc_step_kernel(const double* 
   rpc_chunk_sum_and_ticket(local, csum, d, n, nchunks, u, t, r0, piv, pval, state);
 }
 
-__global__ void to_float_kernel(const double* __restrict__ src, float* __restrict__ dst, int64_t cnt) {
-  GRID_LOOP(i, cnt) dst[i] = (float)src[i];
+// FP64 factor [r][n] -> FP32 factor [r][ldn], zero in the padding rows.
+__global__ void to_float_kernel(const double* __restrict__ src, float* __restrict__ dst, int64_t n, int64_t ldn,
+                                int r) {
+  GRID_LOOP(e, (int64_t)r * ldn) {
+    const int64_t c = e / ldn, i = e % ldn;
+    dst[e] = i < n ? (float)src[c * n + i] : 0.f;
+  }
 }
 
-__global__ void dres_kernel(const float* __restrict__ F, int r, int64_t n, double* __restrict__ dres) {
+__global__ void dres_kernel(const float* __restrict__ F, int64_t ldf, int r, int64_t n, double* __restrict__ dres) {
   GRID_LOOP(i, n) {
     double s = 0.0;
     for (int c = 0; c < r; ++c) {
-      const double f = (double)F[(size_t)c * n + i];
+      const double f = (double)F[(size_t)c * ldf + i];
       s += f * f;
     }
     dres[i] = fmax(1.0 - s, 0.0);   // k(x, x) = 1 for the RBF and Laplacian kernels
@@ -804,7 +994,7 @@ kqr_status rpcholesky_setup(Handle* h, const double* uniforms) {
     double* xw = A + (size_t)rr0 * rr0;
     double* yw = xw + rr0;
     double* lam1 = yw + rr0;
-    core_gram<double>(h, F64, rr0, false, nullptr, nullptr, A, st);
+    core_gram<double>(h, F64, n, rr0, false, nullptr, nullptr, A, st);
     power_iter_kernel<<<1, 512, 0, st>>>(A, rr0, xw, yw, 2000, lam1);
     h->launches++;
     double hl1 = 0.0;
@@ -829,22 +1019,24 @@ kqr_status rpcholesky_setup(Handle* h, const double* uniforms) {
   }
   h->r = r;
   dev_free(h, h->F32); dev_free(h, h->dres); dev_free(h, h->core); dev_free(h, h->tvec); dev_free(h, h->Linv);
+  dev_free(h, h->usplit);
   h->core_valid = false;
-  h->F32 = (float*)dev_alloc(h, sizeof(float) * ((size_t)r * n + 1));
+  h->F32 = (float*)dev_alloc(h, sizeof(float) * ((size_t)r * h->ldn + 1));
   h->dres = (double*)dev_alloc(h, sizeof(double) * n);
   const int N = r + 1;
   h->core = (double*)dev_alloc(h, sizeof(double) * 3 * (size_t)N * N);
   h->tvec = (double*)dev_alloc(h, sizeof(double) * 2 * N);
   h->Linv = (double*)dev_alloc(h, sizeof(double) * n);
-  if (!h->F32 || !h->dres || !h->core || !h->tvec || !h->Linv) {
+  h->usplit = (float2*)dev_alloc(h, sizeof(float2) * h->ldn);
+  if (!h->F32 || !h->dres || !h->core || !h->tvec || !h->Linv || !h->usplit) {
     cleanup();
     return fail(h, KQR_OOM, "preconditioner buffers");
   }
   if (r > 0) {
-    to_float_kernel<<<grid_for((int64_t)r * n), 256, 0, st>>>(F64, h->F32, (int64_t)r * n);
+    to_float_kernel<<<grid_for((int64_t)r * h->ldn), 256, 0, st>>>(F64, h->F32, n, h->ldn, r);
     h->launches++;
   }
-  dres_kernel<<<grid_for(n), 256, 0, st>>>(h->F32, r, n, h->dres);
+  dres_kernel<<<grid_for(n), 256, 0, st>>>(h->F32, h->ldn, r, n, h->dres);
   h->launches++;
   // Floor the residual diagonal at 0.1 of its mean: it is 0 at the pivots, and
   // L + dres must stay away from 0 for a well-conditioned Woodbury core.

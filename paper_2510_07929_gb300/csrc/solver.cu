@@ -243,7 +243,7 @@ cudaError_t cg_after_product(Handle* h, const CgArgs& a, cudaStream_t st) {
   rd.b = Ap;
   if ((e = reduce(h, RED_DOT, rd, n, s + S_PAP, st)) != cudaSuccess) return e;
   if ((e = cg_step(h, a.noise_coef, a.x, a.Kx, r, p, Kp, Ap, st)) != cudaSuccess) return e;
-  if ((e = precond_apply(h, a.Lpre, r, zz, s + S_RZN, st)) != cudaSuccess) return e;
+  if ((e = precond_apply(h, a.Lpre, r, zz, s + S_RZN, st, s + S_RR)) != cudaSuccess) return e;
   return cg_dir(h, p, zz, st);
 }
 
@@ -271,7 +271,7 @@ kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const
   RedArgs rn;
   rn.a = r;
   CK(reduce(h, RED_NORM2, rn, n, s + S_RR, st));
-  CK(precond_apply(h, Lpre, r, zz, s + S_RZN, st));
+  CK(precond_apply(h, Lpre, r, zz, s + S_RZN, st, s + S_RR));
   CK(vec_copy(h, p, zz, n, st));
   RedArgs rp;
   rp.a = p;
@@ -311,7 +311,7 @@ kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const
       else e = gram_f32(h, p, Ap, 1, &ep, st);
       if (e != cudaSuccess) break;
       if ((e = cg_step(h, noise_coef, x, Kx, r, p, Kp, Ap, st)) != cudaSuccess) break;
-      if ((e = precond_apply(h, Lpre, r, zz, s + S_RZN, st)) != cudaSuccess) break;
+      if ((e = precond_apply(h, Lpre, r, zz, s + S_RZN, st, s + S_RR)) != cudaSuccess) break;
       e = cg_dir(h, p, zz, st);
     }
     return e;
@@ -326,7 +326,7 @@ kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const
   std::vector<const void*> key;
   if (graphs) {
     g = &h->cg_graph[x == vec(h, V_ALPHA) ? 0 : 1];
-    key = {x, Kx, b, L, Lpre, h->v32, h->part, h->F32, h->core, h->Linv, h->tvec, h->kstore, h->sym_units,
+    key = {x, Kx, b, L, Lpre, h->v32, h->part, h->F32, h->core, h->Linv, h->tvec, h->usplit, h->kstore, h->sym_units,
            h->tc_hi, reinterpret_cast<const void*>((intptr_t)(h->r * 8 + (lowprec ? 1 : 0) + 2 * h->opt.precond)),
            reinterpret_cast<const void*>((intptr_t)block), reinterpret_cast<const void*>(st)};
   }

@@ -69,3 +69,32 @@ def test_rpcholesky_pivots_at_chunk_edges(K_, kind, n, r0):
     F0, piv_o = O.rpcholesky(lambda s: O.gram(wl.X, wl.X[s:s + 1], kind, wl.gamma)[:, 0], np.ones(n), r0, u)
     np.testing.assert_array_equal(piv, piv_o)
     np.testing.assert_allclose(F, F0[:, :r], atol=2e-6 * np.max(np.abs(F0)))
+
+
+# The apply's passes over F at the edges of their tiles (32 columns, 128 rows) and with r and L far outside the
+# FP32 range (the double-float parts are scaled by powers of two): relative to the same apply at scale 1 the result
+# only picks up the power of two, exactly, where all scale factors are powers of two.
+@pytest.mark.parametrize("n,rank", [(127, 7), (129, 8), (1025, 31), (3000, 63)])
+def test_apply_scales_exactly(K_, n, rank):
+    import torch
+
+    wl = W.lap_large(n=n, p=6, seed=n)
+    rng = np.random.default_rng(n)
+    L = rng.uniform(0.5, 2.0, n)
+    rv = rng.standard_normal(n)
+    with K_.Problem(wl.X, wl.y, wl.kind, wl.gamma, rank0=rank, adaptive_rank=0) as prob:
+        F, _, _, _ = prob.factor()
+
+        def apply(r):
+            out = torch.empty(n, dtype=torch.float64, device="cuda")
+            prob.precond_apply_dev(torch.from_numpy(L).cuda(), 0.5, torch.from_numpy(r).cuda(), out)
+            return out.cpu().numpy()
+
+        base = apply(rv)
+        ref = O.woodbury_apply(F.astype(np.float64), L, 0.5, rv)
+        # condition of the core at most ~10 n: both sides' FP64 errors below 10 n N 2^-53
+        assert np.max(np.abs(base - ref)) <= 2e-9 * np.max(np.abs(ref))
+        for e in (-800, -150, 40, 400):
+            # the sums into U^T L^-1 r arrive in any order: FP64 rounding differs between calls
+            np.testing.assert_allclose(apply(np.ldexp(rv, e)), np.ldexp(base, e), rtol=0,
+                                       atol=2e-9 * np.ldexp(np.max(np.abs(base)), e))
