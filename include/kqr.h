@@ -67,8 +67,11 @@ typedef enum kqr_kernel {
 /* Arithmetic of a Gram product.
  * KQR_PREC_HIGH: entries and sums accurate to about 1e-13 relative (FP64 class;
  *   Laplacian: exact fixed-point L1 distances plus double-float exp and sums on
- *   the FP32/INT32 pipes; RBF with p <= 40: the same fixed-point scheme on the
- *   squared differences; RBF with p > 40: FP64 arithmetic).  Used for gradients
+ *   the FP32/INT32 pipes; RBF with p <= 32 and log2(e) gamma |x - mean|^2 < 28
+ *   for every point: the cross term as exact digit products on the tcgen05
+ *   tensor cores (options.rbf_tensor_cores and symmetric_gram on); other RBF
+ *   with p <= 40: the fixed-point scheme on the squared differences; RBF with
+ *   p > 40: FP64 arithmetic).  Used for gradients
  *   and KKT residuals, and for CG where FP32 cannot resolve K (options.cg_high).
  * KQR_PREC_FP32: FP32 entries and FP32 partial sums, about 1e-6 relative per
  *   entry.  Used inside CG.  RBF: the cross term x_i . x_j runs on the tcgen05
@@ -130,7 +133,7 @@ typedef struct kqr_options {
                                     diagonal moved by at most this relative amount (0: always rebuild) */
   double time_limit_s;           /* host wall-clock limit per solve; <= 0: none */
   int32_t phase1_only;           /* 1: stop after Phase I (for tests of Alg. 1) */
-  int32_t symmetric_gram;        /* 1: single-vector products (FP32, and FP64-class Laplacian) form each off-diagonal tile once and
+  int32_t symmetric_gram;        /* 1: single-vector products (FP32, FP64-class Laplacian, FP64-class RBF with p <= 32) form each off-diagonal tile once and
                                     use it for both K_IJ v_J and K_IJ^T v_I (n(n+1)/2 entries; summation
                                     order not fixed); 0: every entry formed (deterministic) */
   int32_t rbf_tensor_cores;      /* 1: RBF FP32 products on tcgen05 (three TF32 terms); 0: FP32 CUDA cores */

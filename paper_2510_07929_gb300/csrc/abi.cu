@@ -189,6 +189,7 @@ static void free_all(Handle* h) {
                   h->st_alpha, h->st_v, h->st_z, h->sym_units, h->tc_hi, h->tc_lo, h->tc_bf, h->tc_sym_units, h->tc_a16, h->tc_b16};
   for (void* b : bufs) dev_free(h, b);
   kstore_free(h);
+  high_tc_free(h);
   batch_free(h);
   for (auto& g : h->cg_graph)
     if (g.exec) {

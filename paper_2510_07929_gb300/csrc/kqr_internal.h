@@ -66,6 +66,10 @@ cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilog
 cudaError_t gram_high(Handle* h, const double* V, double* U, int m, cudaStream_t st);
 // Laplacian m = 1 FP64-class product with each off-diagonal tile formed once (gram_high_sym.cu).
 cudaError_t gram_high_sym(Handle* h, const double* V, double* U, cudaStream_t st);
+// RBF FP64-class products with the cross term on tcgen05 (gram_high_tc.cu).
+cudaError_t high_tc_ready(Handle* h, bool* ready);
+cudaError_t gram_high_tc(Handle* h, const double* V, double* U, int m, cudaStream_t st);
+void high_tc_free(Handle* h);
 // Stored-K product (gram_stored.cu): kstore_setup fills the packed upper-triangle tiles
 // when options.gram_store asks for it and they fit; gram_stored streams them (m = 1).
 size_t kstore_bytes(int64_t ldn);
@@ -132,6 +136,17 @@ struct Handle {
   float* tc_b16 = nullptr;
   int tc16_katoms = 0;
   CUtensorMap tm_tc_a16{}, tm_tc_b16{};
+
+  // FP64-class RBF products on tensor cores (gram_high_tc.cu): digits, point constants, table,
+  // work units (0: symmetric, 1: rows only) and the partial sums the latter need.
+  int ht_state = 0;
+  void* ht_dig = nullptr;
+  int4* ht_cst = nullptr;
+  float2* ht_table = nullptr;
+  int ht_parts = 0;
+  int4* ht_units[2] = {nullptr, nullptr};
+  int ht_nunits[2] = {0, 0};
+  CUtensorMap tm_ht_i{}, tm_ht_j{};
 
   // Symmetric Gram product: work-unit table (row tile, first and end column tile).
   int4* sym_units = nullptr;
