@@ -178,40 +178,20 @@ __global__ void dx_kernel(const double* __restrict__ alpha, const double* __rest
   }
 }
 
-// Ap = K p + gam (1^T p) 1 + L o p, with K p from the FP64-class product.
-__global__ void adj_op_kernel(double* __restrict__ Ap, const double* __restrict__ Kp, const double* __restrict__ p,
-                              const double* __restrict__ L, const double* __restrict__ sump, double gam, int64_t n) {
-  const double sg = gam * (*sump);
-  GRID_LOOP(i, n) Ap[i] = Kp[i] + sg + L[i] * p[i];
-}
-
-__global__ void adj_step_kernel(double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
-                                const double* __restrict__ Ap, double a, int64_t n) {
-  GRID_LOOP(i, n) {
-    x[i] += a * p[i];
-    r[i] -= a * Ap[i];
-  }
-}
-
-__global__ void adj_dir_kernel(double* __restrict__ p, const double* __restrict__ z, double b, int64_t n) {
-  GRID_LOOP(i, n) p[i] = z[i] + b * p[i];
-}
-
 // PCG on (K + gam 1 1^T + diag(L)) x = b with FP64-class Gram products and the problem's
 // Woodbury preconditioner (built for Lpre).  The adjoint system is as ill-conditioned as
-// K on the elbow set, where FP32 products would cap the gradient's accuracy.  dsc: 4
-// device doubles of scratch.
+// K on the elbow set, where FP32 products would cap the gradient's accuracy.  The iterations run
+// on the solver's device-resident CG (cg_after_product); the host reads the status once per
+// kAdjointBlock iterations (a stopped CG makes the rest of a block a no-op).  With a host read of
+// three scalars per iteration a product of 20 us at n = 3000 waited for the host most of the time.
+constexpr int kAdjointBlock = 4;
+
 static kqr_status adjoint_cg(Handle* h, const double* L, const double* Lpre, double gam, const double* b, double* x,
-                             double tol, int maxit, double* dsc, cudaStream_t st) {
+                             double tol, int maxit, cudaStream_t st) {
   const int64_t n = h->n;
-  double* r = vec(h, V_R);
-  double* z = vec(h, V_ZZ);
-  double* p = vec(h, V_P);
-  double* Kp = vec(h, V_KP);
-  double* Ap = vec(h, V_AP);
-  double hs[4];
-  auto get = [&](int k) -> cudaError_t {
-    cudaError_t e = cudaMemcpyAsync(hs + k, dsc + k, sizeof(double), cudaMemcpyDeviceToHost, st);
+  double* s = h->scal;
+  auto get = [&](int slot, int count) -> cudaError_t {
+    cudaError_t e = cudaMemcpyAsync(h->scal_host + slot, s + slot, sizeof(double) * count, cudaMemcpyDeviceToHost, st);
     return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
   };
 #define AK(call)                                              \
@@ -220,44 +200,29 @@ static kqr_status adjoint_cg(Handle* h, const double* L, const double* Lpre, dou
     if (_e != cudaSuccess) return cuda_fail(h, _e, #call);    \
   } while (0)
   AK(vec_fill(h, x, 0.0, n, st));
-  AK(vec_copy(h, r, b, n, st));
+  AK(vec_copy(h, vec(h, V_R), b, n, st));
   RedArgs rn;
-  rn.a = r;
-  AK(reduce(h, RED_NORM2, rn, n, dsc + 0, st));
-  AK(get(0));
-  if (std::sqrt(hs[0]) <= tol) return KQR_OK;
-  AK(precond_apply(h, Lpre, r, z, dsc + 1, st, dsc + 0));
-  AK(get(1));
-  double rz = hs[1];
-  AK(vec_copy(h, p, z, n, st));
-  for (int it = 0; it < maxit; ++it) {
-    RedArgs rs;
-    rs.a = p;
-    AK(reduce(h, RED_SUM, rs, n, dsc + 2, st));
-    AK(gram_high(h, p, Kp, 1, st));
-    adj_op_kernel<<<grid_for(n), 256, 0, st>>>(Ap, Kp, p, L, dsc + 2, gam, n);
-    AK(cudaGetLastError());
-    RedArgs rd;
-    rd.a = p;
-    rd.b = Ap;
-    AK(reduce(h, RED_DOT, rd, n, dsc + 3, st));
-    AK(get(3));
-    const double pAp = hs[3];
-    if (!std::isfinite(pAp)) return fail(h, KQR_BREAKDOWN, "adjoint CG: non-finite curvature");
-    if (!(pAp > 0.0)) break;
-    adj_step_kernel<<<grid_for(n), 256, 0, st>>>(x, r, p, Ap, rz / pAp, n);
-    AK(cudaGetLastError());
-    AK(reduce(h, RED_NORM2, rn, n, dsc + 0, st));
-    AK(get(0));
-    if (std::sqrt(hs[0]) <= tol) break;
-    AK(precond_apply(h, Lpre, r, z, dsc + 1, st, dsc + 0));
-    AK(get(1));
-    adj_dir_kernel<<<grid_for(n), 256, 0, st>>>(p, z, hs[1] / rz, n);
-    AK(cudaGetLastError());
-    rz = hs[1];
+  rn.a = b;
+  AK(reduce(h, RED_NORM2, rn, n, s + S_RR, st));
+  AK(get(S_RR, 1));
+  if (std::sqrt(h->scal_host[S_RR]) <= tol) return KQR_OK;
+  AK(cg_begin(h, Lpre, gam, tol, maxit, st));
+  CgArgs a;
+  a.L = L;
+  a.Lpre = Lpre;
+  a.gam = gam;
+  a.x = x;
+  for (;;) {
+    for (int j = 0; j < kAdjointBlock; ++j) {
+      AK(gram_high(h, vec(h, V_P), vec(h, V_KP), 1, st));
+      AK(cg_after_product(h, a, st));
+    }
+    AK(get(S_CGST, 1));
+    const int state = (int)h->scal_host[S_CGST];
+    if (state == CG_NONFINITE) return fail(h, KQR_BREAKDOWN, "adjoint CG: non-finite curvature");
+    if (state != CG_RUN) return KQR_OK;
   }
 #undef AK
-  return KQR_OK;
 }
 
 }  // namespace kqr
@@ -363,9 +328,9 @@ extern "C" kqr_status kqr_heldout_grad(kqr_handle* kh, const double* X, const do
     GK(cudaMemcpyAsync(h->scal_host + S_RED0 + 15, h->scal + S_RED0 + 15, sizeof(double), cudaMemcpyDeviceToHost, st));
     GK(cudaStreamSynchronize(st));
     const double nb1 = std::sqrt(h->scal_host[S_RED0 + 15]);
-    s = adjoint_cg(h, Ld, Lp, gam, rhs1, s1, std::fmax(1e-300, 1e-11 * nb1), 3000, sums + 12, st);
+    s = adjoint_cg(h, Ld, Lp, gam, rhs1, s1, std::fmax(1e-300, 1e-11 * nb1), 3000, st);
     if (s != KQR_OK) return done(s);
-    s = adjoint_cg(h, Ld, Lp, gam, rhs2, s2, 1e-11 * std::sqrt(nE), 3000, sums + 12, st);
+    s = adjoint_cg(h, Ld, Lp, gam, rhs2, s2, 1e-11 * std::sqrt(nE), 3000, st);
     if (s != KQR_OK) return done(s);
     masked_sums_kernel<<<grid_for(n), 256, 0, st>>>(s1, s2, mask, n, sums + 4);
     GK(cudaGetLastError());

@@ -16,6 +16,7 @@
 
 #include "kqr_internal.h"
 #include "ptx.cuh"
+#include "reduce.cuh"
 
 namespace kqr {
 
@@ -158,50 +159,39 @@ __global__ void __launch_bounds__(kThreads, 2)
 }
 
 // v (FP64, n) -> v32 [ldn] zero padded; acc [ldn] zeroed; optional sum of v.
-__global__ void sym_prep_kernel(const double* __restrict__ V, float* __restrict__ v32, float* __restrict__ acc,
-                                int64_t n, int64_t ldn, double* __restrict__ sum_out) {
-  double s = 0.0;
+__global__ void __launch_bounds__(256) sym_prep_kernel(const double* __restrict__ V, float* __restrict__ v32,
+                                                       float* __restrict__ acc, int64_t n, int64_t ldn,
+                                                       double* __restrict__ part, unsigned int* __restrict__ counter,
+                                                       double* __restrict__ sum_out) {
+  double s[1] = {0.0};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ldn; i += (int64_t)gridDim.x * blockDim.x) {
     const double x = i < n ? V[i] : 0.0;
     v32[i] = (float)x;
     acc[i] = 0.f;
-    s += x;
+    s[0] += x;
   }
-  if (sum_out) {
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    __shared__ double ws[32];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += ws[w];
-      atomicAdd(sum_out, t);
-    }
-  }
+  if (!sum_out) return;
+  double tot;
+  if (grid_sums(s, part, counter, &tot) && threadIdx.x == 0) *sum_out = tot;
 }
 
-// out = acc (+ gam sum_p + L p), dot_out += p . out, raw_out = acc.
-__global__ void sym_finish_kernel(const float* __restrict__ acc, int64_t n, double* __restrict__ out, GramEpilogue ep) {
-  double dot = 0.0;
-  const double sump = ep.sum_p ? *ep.sum_p : 0.0;
+// out = acc (+ gam sum_p + L p), *dot_out = p . out, raw_out = acc.
+__global__ void __launch_bounds__(256) sym_finish_kernel(const float* __restrict__ acc, int64_t n,
+                                                         double* __restrict__ out, GramEpilogue ep,
+                                                         double* __restrict__ part,
+                                                         unsigned int* __restrict__ counter) {
+  double dot[1] = {0.0};
+  const double add = ep.L ? (ep.gam_dev ? *ep.gam_dev : ep.gam) * (ep.sum_p ? *ep.sum_p : 0.0) : 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double s = (double)acc[i];
     if (ep.raw_out) ep.raw_out[i] = s;
-    if (ep.L) s += (ep.gam_dev ? *ep.gam_dev : ep.gam) * sump + ep.L[i] * ep.pvec[i];
+    if (ep.L) s += add + ep.L[i] * ep.pvec[i];
     out[i] = s;
-    if (ep.dot_out) dot += ep.pvec[i] * s;
+    if (ep.dot_out) dot[0] += ep.pvec[i] * s;
   }
-  if (ep.dot_out) {
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    __shared__ double ws[32];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = dot;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += ws[w];
-      atomicAdd(ep.dot_out, t);
-    }
-  }
+  if (!ep.dot_out) return;
+  double tot;
+  if (grid_sums(dot, part, counter, &tot) && threadIdx.x == 0) *ep.dot_out = tot;
 }
 
 static size_t sym_smem_bytes(int p) {
@@ -231,22 +221,11 @@ cudaError_t sym_units_ensure(Handle* h) {
 cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilogue* ep, cudaStream_t st) {
   cudaError_t e = sym_units_ensure(h);
   if (e != cudaSuccess) return e;
-  const size_t need = (size_t)h->ldn * sizeof(float) * 2;   // v32 + acc
-  if (h->v32_cap < need) {
-    dev_free(h, h->v32);
-    h->v32 = (float*)dev_alloc(h, need);
-    h->v32_cap = h->v32 ? need : 0;
-    if (!h->v32) return cudaErrorMemoryAllocation;
-  }
-  float* v32 = h->v32;
-  float* acc = h->v32 + h->ldn;
+  float *v32, *acc;
+  if ((e = sym_buffers(h, &v32, &acc)) != cudaSuccess) return e;
   GramEpilogue none;
   const GramEpilogue& g = ep ? *ep : none;
-  double* sum_out = g.sum_p ? const_cast<double*>(g.sum_p) : nullptr;
-  if (sum_out && (e = cudaMemsetAsync(sum_out, 0, sizeof(double), st)) != cudaSuccess) return e;
-  sym_prep_kernel<<<grid_for(h->ldn), 256, 0, st>>>(V, v32, acc, h->n, h->ldn, sum_out);
-  h->launches++;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (!g.prepped && (e = sym_prep(h, V, v32, acc, const_cast<double*>(g.sum_p), st)) != cudaSuccess) return e;
   const size_t smem = sym_smem_bytes((int)h->p);
   prof_mark(h, 0, true, st);
   if (h->kind == KQR_LAPLACIAN) {
@@ -263,31 +242,37 @@ cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilog
   prof_mark(h, 0, false, st);
   h->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (g.dot_out && (e = cudaMemsetAsync(g.dot_out, 0, sizeof(double), st)) != cudaSuccess) return e;
-  sym_finish_kernel<<<grid_for(h->n), 256, 0, st>>>(acc, h->n, U, g);
-  h->launches++;
-  return cudaGetLastError();
+  return sym_finish(h, acc, U, g, st);
 }
 
 }  // namespace kqr
 
 namespace kqr {
 
+cudaError_t sym_buffers(Handle* h, float** v32, float** acc) {
+  const size_t need = (size_t)h->ldn * sizeof(float) * 2;
+  if (h->v32_cap < need) {
+    dev_free(h, h->v32);
+    h->v32 = (float*)dev_alloc(h, need);
+    h->v32_cap = h->v32 ? need : 0;
+    if (!h->v32) return cudaErrorMemoryAllocation;
+  }
+  *v32 = h->v32;
+  *acc = h->v32 + h->ldn;
+  return cudaSuccess;
+}
+
 // v -> FP32 copy and zeroed FP32 accumulator (and 1^T v into *sum_out if given),
 // for products that accumulate with atomics (symmetric tiles, stored K).
 cudaError_t sym_prep(Handle* h, const double* V, float* v32, float* acc, double* sum_out, cudaStream_t st) {
-  cudaError_t e;
-  if (sum_out && (e = cudaMemsetAsync(sum_out, 0, sizeof(double), st)) != cudaSuccess) return e;
-  sym_prep_kernel<<<grid_for(h->ldn), 256, 0, st>>>(V, v32, acc, h->n, h->ldn, sum_out);
+  sym_prep_kernel<<<grid_for(h->ldn), 256, 0, st>>>(V, v32, acc, h->n, h->ldn, h->red_part, h->red_counter, sum_out);
   h->launches++;
   return cudaGetLastError();
 }
 
-// out = acc (+ the CG operator's terms of g), as at the end of gram_f32_sym.
+// out = acc (+ the CG operator's terms of g).
 cudaError_t sym_finish(Handle* h, const float* acc, double* U, const GramEpilogue& g, cudaStream_t st) {
-  cudaError_t e;
-  if (g.dot_out && (e = cudaMemsetAsync(g.dot_out, 0, sizeof(double), st)) != cudaSuccess) return e;
-  sym_finish_kernel<<<grid_for(h->n), 256, 0, st>>>(acc, h->n, U, g);
+  sym_finish_kernel<<<grid_for(h->n), 256, 0, st>>>(acc, h->n, U, g, h->red_part, h->red_counter);
   h->launches++;
   return cudaGetLastError();
 }

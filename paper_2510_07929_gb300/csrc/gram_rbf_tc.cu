@@ -775,7 +775,6 @@ static size_t tc_sym_smem(int katoms) {
          (1 + 4 + 2 * kSymBufs) * sizeof(uint64_t) + 32;
 }
 
-cudaError_t sym_prep(Handle* h, const double* V, float* v32, float* acc, double* sum_out, cudaStream_t st);
 
 // Work units of the symmetric tensor-core tiles: (row tile I, column tiles [J0, J1)) with
 // I <= J0, about 8 per SM (one CTA resident), so that each CTA's TMA/MMA pipeline runs over
@@ -798,7 +797,6 @@ static cudaError_t tc_sym_units_ensure(Handle* h) {
   h->tc_sym_T = T;
   return cudaMemcpy(h->tc_sym_units, u.data(), u.size() * sizeof(int4), cudaMemcpyHostToDevice);
 }
-cudaError_t sym_finish(Handle* h, const float* acc, double* U, const GramEpilogue& g, cudaStream_t st);
 
 // m = 1 RBF product on symmetric tensor-core tiles; nt = 3: FP32 class (fp16 parts when
 // the row factors fold and 3p <= 128, else TF32 parts), 1: TF32.
@@ -807,18 +805,11 @@ static cudaError_t rbf_tc_sym_product(Handle* h, const double* V, double* U, int
   cudaError_t e = rbf_tc_prepare(h);
   if (e != cudaSuccess) return e;
   if ((e = tc_sym_units_ensure(h)) != cudaSuccess) return e;
-  const size_t need = (size_t)h->ldn * sizeof(float) * 2;   // v32 + acc
-  if (h->v32_cap < need) {
-    dev_free(h, h->v32);
-    h->v32 = (float*)dev_alloc(h, need);
-    h->v32_cap = h->v32 ? need : 0;
-    if (!h->v32) return cudaErrorMemoryAllocation;
-  }
-  float* v32 = h->v32;
-  float* acc = h->v32 + h->ldn;
+  float *v32, *acc;
+  if ((e = sym_buffers(h, &v32, &acc)) != cudaSuccess) return e;
   GramEpilogue none;
   const GramEpilogue& g = ep ? *ep : none;
-  if ((e = sym_prep(h, V, v32, acc, g.sum_p ? const_cast<double*>(g.sum_p) : nullptr, st)) != cudaSuccess) return e;
+  if (!g.prepped && (e = sym_prep(h, V, v32, acc, const_cast<double*>(g.sum_p), st)) != cudaSuccess) return e;
   const bool f16 = nt == 3 && h->tc_fold_rows && 3 * h->p <= 128;
   if (f16 && (e = rbf_f16_prepare(h)) != cudaSuccess) return e;
   const int katoms = f16 ? h->tc16_katoms : h->tc_Kp / 32;

@@ -37,8 +37,6 @@
 
 namespace kqr {
 
-cudaError_t sym_prep(Handle* h, const double* V, float* v32, float* acc, double* sum_out, cudaStream_t st);
-cudaError_t sym_finish(Handle* h, const float* acc, double* U, const GramEpilogue& g, cudaStream_t st);
 
 constexpr int kKsTileFloats = kTile * kTile;                     // 16384 floats = 64 KB
 constexpr int kKsChunkRows = 32;
@@ -386,19 +384,12 @@ void kstore_free(Handle* h) {
 }
 
 cudaError_t gram_stored(Handle* h, const double* V, double* U, const GramEpilogue* ep, cudaStream_t st) {
-  const size_t need = (size_t)h->ldn * sizeof(float) * 2;   // v32 + acc
-  if (h->v32_cap < need) {
-    dev_free(h, h->v32);
-    h->v32 = (float*)dev_alloc(h, need);
-    h->v32_cap = h->v32 ? need : 0;
-    if (!h->v32) return cudaErrorMemoryAllocation;
-  }
-  float* v32 = h->v32;
-  float* acc = h->v32 + h->ldn;
+  cudaError_t e;
+  float *v32, *acc;
+  if ((e = sym_buffers(h, &v32, &acc)) != cudaSuccess) return e;
   GramEpilogue none;
   const GramEpilogue& g = ep ? *ep : none;
-  cudaError_t e = sym_prep(h, V, v32, acc, g.sum_p ? const_cast<double*>(g.sum_p) : nullptr, st);
-  if (e != cudaSuccess) return e;
+  if (!g.prepped && (e = sym_prep(h, V, v32, acc, const_cast<double*>(g.sum_p), st)) != cudaSuccess) return e;
   prof_mark(h, 2, true, st);
   kstore_gemv_kernel<<<h->kstore_grid, kKsThreads, kstore_smem(), st>>>(h->kstore, v32, acc, h->kstore_sched,
                                                                        (int)(h->ldn / kTile), h->err_flag);

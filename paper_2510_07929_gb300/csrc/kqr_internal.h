@@ -52,6 +52,7 @@ struct GramEpilogue {
   const double* pvec = nullptr;    // device vector p (FP64)
   double* dot_out = nullptr;       // device scalar, accumulates p^T out
   double* raw_out = nullptr;       // device, receives K p alone (nullable)
+  bool prepped = false;            // the FP32 copy of p, the zeroed sums (sym_buffers) and *sum_p are there already
 };
 
 cudaError_t gram_f32(Handle* h, const double* V, double* U, int m, const GramEpilogue* ep, cudaStream_t st);
@@ -63,6 +64,11 @@ cudaError_t gram_rbf_tc(Handle* h, const double* V, double* U, int m, bool three
 cudaError_t gram_rbf_tc_bf16(Handle* h, const double* V, double* U, int m, cudaStream_t st);
 // m = 1 product with each off-diagonal tile formed once (gram_f32_sym.cu).
 cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilogue* ep, cudaStream_t st);
+// FP32 copy of the vector and FP32 sums of the products that accumulate with atomics
+// (symmetric tiles, stored K): ldn floats each, and the kernel that fills them.
+cudaError_t sym_buffers(Handle* h, float** v32, float** acc);
+cudaError_t sym_prep(Handle* h, const double* V, float* v32, float* acc, double* sum_out, cudaStream_t st);
+cudaError_t sym_finish(Handle* h, const float* acc, double* U, const GramEpilogue& g, cudaStream_t st);
 cudaError_t gram_high(Handle* h, const double* V, double* U, int m, cudaStream_t st);
 // Laplacian m = 1 FP64-class product with each off-diagonal tile formed once (gram_high_sym.cu).
 cudaError_t gram_high_sym(Handle* h, const double* V, double* U, cudaStream_t st);
@@ -234,13 +240,6 @@ cudaError_t reduce(Handle* h, RedKind kind, const RedArgs& a, int64_t n, double*
 
 cudaError_t vec_fill(Handle* h, double* x, double val, int64_t n, cudaStream_t st);
 cudaError_t vec_copy(Handle* h, double* dst, const double* src, int64_t n, cudaStream_t st);
-// y = a * x + y (device scalar a read from *a_dev, scaled by sgn)
-cudaError_t cg_update(Handle* h, double* x, double* Kx, double* r, const double* p, const double* Kp,
-                      const double* Ap, const double* a_dev, int64_t n, double* rr_out, cudaStream_t st);
-// p = z + beta p (beta read from beta_dev); a non-zero *stop_dev (nullable) skips it;
-// ||p||^2 into *pp_out (device).
-cudaError_t cg_direction(Handle* h, double* p, const double* z, const double* beta_dev, const double* stop_dev,
-                         int64_t n, double* pp_out, cudaStream_t st);
 cudaError_t op_residual(Handle* h, double* r, const double* b, const double* x, const double* Kx, double gam,
                         const double* sum_x, const double* L, int64_t n, cudaStream_t st);
 cudaError_t admm_rhs(Handle* h, double* b, const double* y, double beta, const double* z, const double* v,
@@ -265,7 +264,16 @@ kqr_status precond_build(Handle* h, const double* Ldiag, double gam, cudaStream_
 // its distance to the exact P changes).  Lcore_i = 1 / Linv_i.
 kqr_status precond_update(Handle* h, const double* Lpre, double gam, double rtol, cudaStream_t st);
 cudaError_t precond_apply(Handle* h, const double* Ldiag, const double* r, double* out, double* rz_out,
-                          cudaStream_t st, const double* rr = nullptr);
+                          cudaStream_t st, const double* rr = nullptr, bool split = false);
+// What the CG step kernel needs to leave its residual split for precond_apply(split = true); all null
+// when the preconditioner is off.
+struct WbSplit {
+  const double* Linv = nullptr;
+  float2* us = nullptr;
+  double* t = nullptr;
+  int N = 0;
+};
+WbSplit precond_split(Handle* h);
 kqr_status rpcholesky_setup(Handle* h, const double* uniforms);
 // Inverse of an SPD matrix over all SMs (spd_inverse.cu): G overwritten, W scratch, all N x N.
 cudaError_t spd_inverse(Handle* h, double* G, double* W, double* Ginv, int N, int* info, cudaStream_t st);
@@ -287,6 +295,8 @@ kqr_status kkt(Handle* h, const double* alpha, const double* v, double beta, con
 // other terms, the device-resident step lengths and stopping test, the preconditioner and
 // the direction update (solver.cu).  Used by the grid's shared CG engine (grid.cu), which
 // runs the products of several columns together and this chain on each column's stream.
+// CG status (S_CGST): running, met tol, stopped at a non-positive curvature, non-finite, maxit.
+enum CgState { CG_RUN = 0, CG_MET = 1, CG_TRUNC = 2, CG_NONFINITE = 3, CG_MAXIT = 4 };
 struct CgArgs {
   const double* L = nullptr;
   const double* Lpre = nullptr;
@@ -296,6 +306,9 @@ struct CgArgs {
   double noise_coef = 0.0;
 };
 cudaError_t cg_after_product(Handle* h, const CgArgs& a, cudaStream_t st);
+// Start of a CG on the residual in vec(h, V_R) with ||r||^2 in S_RR: preconditioned direction, its sum and
+// square, the device control words.  maxit as a count, tol on ||r||.
+cudaError_t cg_begin(Handle* h, const double* Lpre, double gam, double tol, int maxit, cudaStream_t st);
 // Runs a grid column's CG (set up by pcg on the column's stream) in the grid's shared
 // engine until its device status leaves "running" (grid.cu).
 cudaError_t grid_cg(Handle* h, const CgArgs& a);

@@ -20,6 +20,8 @@
 #include <vector>
 
 #include "kqr_internal.h"
+#include "reduce.cuh"
+#include "wb_split.cuh"
 
 namespace kqr {
 
@@ -48,11 +50,6 @@ constexpr int kCT = 64;      // core tile
 constexpr int kCR = 16;      // rows per shared-memory step
 constexpr int kCgRows = 32;  // rows per double-float sum
 constexpr int kCgThreads = 128;
-
-__device__ __forceinline__ void df_split(double x, float& hi, float& lo) {
-  hi = (float)x;
-  lo = (float)(x - (double)hi);
-}
 
 // T: float (the FP32 factor, weights w; both triangles of G are written) or double (the set-up's FP64 factor, no weights).
 template <typename T>
@@ -233,16 +230,6 @@ __global__ void recip_kernel(double* out, const double* L, int64_t n, unsigned l
 // (the exponent of ||r|| and of max L^{-1}) that keep both parts inside the FP32 range for any r.
 // Sums run in double-float over at most 32 terms between renormalisations and are combined in
 // FP64.  Measured (n = 20011, r = 1024, cold caches): 37 and 68 us.
-__device__ __forceinline__ int norm_exponent(double rr, bool is_max) {   // e with 2^e about sqrt(rr), or rr
-  const int ex = (int)((__double_as_longlong(rr) >> 52) & 0x7ff) - 1023;
-  return is_max ? max(-1000, min(1000, ex)) : ex >> 1;
-}
-__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
-__device__ __forceinline__ int max_exponent(unsigned long long wmax) {   // of max L^{-1}; 0 if it is not a normal number
-  const int ex = (int)((wmax >> 52) & 0x7ff);
-  return ex > 0 && ex < 2046 ? ex - 1023 : 0;
-}
-
 // (sh, sl) += x (yh + yl), x FP32.
 __device__ __forceinline__ void df_mac(float& sh, float& sl, float x, float yh, float yl) {
   const float p = __fmul_rn(x, yh);
@@ -445,50 +432,21 @@ __global__ void __launch_bounds__(256) woodbury_out_kernel(const float* __restri
     }
   }
   if (!rz) return;
-  __shared__ bool last;
-  if (warp == 0) {
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    if (lane == 0) {
-      part[blockIdx.x] = dot;
-      __threadfence();
-      last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double v = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) v += __ldcg(part + b);
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __shared__ double ws[8];
-  if (lane == 0) ws[warp] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double tot = 0.0;
-    for (int w = 0; w < 8; ++w) tot += ws[w];
-    *rz = tot;
-    *counter = 0u;
-  }
+  double dots[1] = {dot}, tot;
+  if (grid_sums(dots, part, counter, &tot) && threadIdx.x == 0) *rz = tot;
 }
 
-__global__ void ident_dot_kernel(const double* __restrict__ rv, double* __restrict__ out, int64_t n,
-                                 double* __restrict__ rz) {
+__global__ void __launch_bounds__(256) ident_dot_kernel(const double* __restrict__ rv, double* __restrict__ out,
+                                                        int64_t n, double* __restrict__ part,
+                                                        unsigned int* __restrict__ counter, double* __restrict__ rz) {
   double dot = 0.0;
   GRID_LOOP(i, n) {
     out[i] = rv[i];
     dot += rv[i] * rv[i];
   }
-  if (rz) {
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    __shared__ double ws[8];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = dot;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double v = 0.0;
-      for (int w = 0; w < 8; ++w) v += ws[w];
-      atomicAdd(rz, v);
-    }
-  }
+  if (!rz) return;
+  double dots[1] = {dot}, tot;
+  if (grid_sums(dots, part, counter, &tot) && threadIdx.x == 0) *rz = tot;
 }
 
 // max_i |Lpre_i Linv_i - 1| (relative change of the diagonal since the last build)
@@ -555,14 +513,14 @@ kqr_status precond_build(Handle* h, const double* Lpre, double gam, cudaStream_t
 
 // out = P^{-1} r with the core built by precond_build for the same Lpre; rz_out (device,
 // nullable) receives r^T out.  rr (device, nullable): ||r||^2, for the scaling of the double-float
-// parts; without it max |r| is computed here.
+// parts; without it max |r| is computed here.  split: usplit, t and S_WEXP are there already (the CG
+// step kernel left them).
 cudaError_t precond_apply(Handle* h, const double* Lpre, const double* rv, double* out, double* rz_out,
-                          cudaStream_t st, const double* rr) {
+                          cudaStream_t st, const double* rr, bool split) {
   (void)Lpre;
   cudaError_t e;
   if (h->opt.precond == KQR_PRECOND_NONE) {
-    if (rz_out && (e = cudaMemsetAsync(rz_out, 0, sizeof(double), st)) != cudaSuccess) return e;
-    ident_dot_kernel<<<grid_for(h->n), 256, 0, st>>>(rv, out, h->n, rz_out);
+    ident_dot_kernel<<<grid_for(h->n), 256, 0, st>>>(rv, out, h->n, h->red_part, h->red_counter, rz_out);
     h->launches++;
     return cudaGetLastError();
   }
@@ -570,15 +528,18 @@ cudaError_t precond_apply(Handle* h, const double* Lpre, const double* rv, doubl
   const double* Ginv = h->core + 2 * (size_t)N * N;
   double* t = h->tvec;
   float2* t2s = reinterpret_cast<float2*>(h->tvec + N);
-  const int is_max = rr ? 0 : 1;
-  if (!rr) {
-    double* slot = h->scal + S_WMAXR;
-    if ((e = cudaMemsetAsync(slot, 0, sizeof(double), st)) != cudaSuccess) return e;
-    absmax_kernel<<<grid_for(h->n), 256, 0, st>>>(rv, h->n, reinterpret_cast<unsigned long long*>(slot));
+  if (!split) {
+    const int is_max = rr ? 0 : 1;
+    if (!rr) {
+      double* slot = h->scal + S_WMAXR;
+      if ((e = cudaMemsetAsync(slot, 0, sizeof(double), st)) != cudaSuccess) return e;
+      absmax_kernel<<<grid_for(h->n), 256, 0, st>>>(rv, h->n, reinterpret_cast<unsigned long long*>(slot));
+      h->launches++;
+      rr = slot;
+    }
+    wb_split_kernel<<<grid_for(h->ldn), 256, 0, st>>>(h->Linv, rv, h->n, h->ldn, rr, is_max, h->scal, h->usplit, t, N);
     h->launches++;
-    rr = slot;
   }
-  wb_split_kernel<<<grid_for(h->ldn), 256, 0, st>>>(h->Linv, rv, h->n, h->ldn, rr, is_max, h->scal, h->usplit, t, N);
   // rows per CTA of the first pass: about four CTAs per SM, 128 .. 1024 rows
   const int groups = (N + 31) / 32;
   const int64_t want = std::max<int64_t>(1, (int64_t)4 * h->num_sms / groups);
@@ -591,8 +552,18 @@ cudaError_t precond_apply(Handle* h, const double* Lpre, const double* rv, doubl
   woodbury_out_kernel<<<blocks, 256, (size_t)N * sizeof(float2), st>>>(h->F32, h->ldn, h->r, h->n, h->Linv, rv, t2s,
                                                                        h->scal, out, h->red_part, h->red_counter,
                                                                        rz_out);
-  h->launches += 4;
+  h->launches += 3;
   return cudaGetLastError();
+}
+
+WbSplit precond_split(Handle* h) {
+  WbSplit w;
+  if (h->opt.precond == KQR_PRECOND_NONE) return w;
+  w.Linv = h->Linv;
+  w.us = h->usplit;
+  w.t = h->tvec;
+  w.N = h->r + 1;
+  return w;
 }
 
 // ---- RPCholesky set-up --------------------------------------------------------------

@@ -13,6 +13,8 @@
 #include <cstdio>
 
 #include "kqr_internal.h"
+#include "reduce.cuh"
+#include "wb_split.cuh"
 
 namespace kqr {
 
@@ -37,11 +39,6 @@ static cudaError_t fetch(Handle* h, int slot, int count, cudaStream_t st) {
   return cudaStreamSynchronize(st);
 }
 
-static cudaError_t put(Handle* h, int slot, double v, cudaStream_t st) {
-  h->scal_host[slot] = v;
-  return cudaMemcpyAsync(h->scal + slot, h->scal_host + slot, sizeof(double), cudaMemcpyHostToDevice, st);
-}
-
 static kqr_status check_device_flag(Handle* h, cudaStream_t st) {
   int flag = 0;
   cudaError_t e = cudaMemcpyAsync(&flag, h->err_flag, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -59,28 +56,28 @@ static cudaError_t raw_product(Handle* h, const double* p, double* out, bool hig
   return high ? gram_high(h, p, out, 1, st) : gram_f32(h, p, out, 1, nullptr, st);
 }
 
-// Ap = K p + gam (1^T p) 1 + L o p; Kp = K p; pAp into *dot.
-__global__ void high_op_kernel(double* __restrict__ Ap, const double* __restrict__ Kp, const double* __restrict__ p,
-                               const double* __restrict__ L, const double* __restrict__ sump, double gam, int64_t n) {
-  const double sg = gam * (*sump);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    Ap[i] = Kp[i] + sg + L[i] * p[i];
+// Ap = K p + gam (1^T p) 1 + L o p and p^T Ap, for products that return K p alone (FP64-class
+// products, a grid's shared products); 1^T p and gam in S_SUMP and S_GAM.
+__global__ void __launch_bounds__(256) cg_operator_kernel(double* __restrict__ Ap, const double* __restrict__ Kp,
+                                                          const double* __restrict__ p, const double* __restrict__ L,
+                                                          double* __restrict__ s, int64_t n, double* __restrict__ part,
+                                                          unsigned int* __restrict__ counter) {
+  const double sg = s[S_GAM] * s[S_SUMP];
+  double dot[1] = {0.0}, tot;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const double pi = p[i], a = Kp[i] + sg + L[i] * pi;
+    Ap[i] = a;
+    dot[0] = fma(pi, a, dot[0]);
+  }
+  if (grid_sums(dot, part, counter, &tot) && threadIdx.x == 0) s[S_PAP] = tot;
 }
 
-static cudaError_t op_product(Handle* h, const double* p, double* Ap, double* Kp, const double* L, double gam,
-                              double* sump, double* dot, bool high, cudaStream_t st) {
-  RedArgs rs;
-  rs.a = p;
-  cudaError_t e = reduce(h, RED_SUM, rs, h->n, sump, st);
-  if (e != cudaSuccess) return e;
-  if ((e = raw_product(h, p, Kp, high, st)) != cudaSuccess) return e;
-  high_op_kernel<<<grid_for(h->n), 256, 0, st>>>(Ap, Kp, p, L, sump, gam, h->n);
+static cudaError_t cg_operator(Handle* h, double* Ap, const double* Kp, const double* p, const double* L,
+                               cudaStream_t st) {
+  cg_operator_kernel<<<grid_for(h->n, 256, 304), 256, 0, st>>>(Ap, Kp, p, L, h->scal, h->n, h->red_part,
+                                                               h->red_counter);
   h->launches++;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  RedArgs rd;
-  rd.a = p;
-  rd.b = Ap;
-  return reduce(h, RED_DOT, rd, h->n, dot, st);
+  return cudaGetLastError();
 }
 
 // ---- device-resident CG control ---------------------------------------------------
@@ -89,37 +86,6 @@ static cudaError_t op_product(Handle* h, const double* p, double* Ap, double* Kp
 // last), so the host reads one status word per block of iterations instead of three
 // blocking copies per iteration.  Status (S_CGST):
 // 0 running, 1 met tol, 2 stopped at a non-positive curvature, 3 non-finite, 4 maxit.
-enum CgState { CG_RUN = 0, CG_MET = 1, CG_TRUNC = 2, CG_NONFINITE = 3, CG_MAXIT = 4 };
-
-// Block sum of v over the CTA's 256 threads into part[blockIdx.x]; returns true in the
-// CTA that finishes last, whose thread 0 then holds the sum over all CTAs (added in
-// CTA order) in *total.  Resets the counter for the next reduction.
-__device__ __forceinline__ bool cg_block_sum(double v, double* __restrict__ part, unsigned int* __restrict__ counter,
-                                             double* total) {
-  __shared__ double ws[8];
-  __shared__ bool last;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double b = 0.0;
-    for (int w = 0; w < 8; ++w) b += ws[w];
-    part[blockIdx.x] = b;
-    __threadfence();
-    last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!last) return false;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    double t = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) t += __ldcg(part + b);
-    *total = t;
-    *counter = 0u;
-  }
-  return true;
-}
-
 // One CG step after p^T A p is known: the step length a = rz / pAp (rz in S_RZN), or the
 // truncation step when the curvature is at or below the product's rounding level
 // (noise_coef: that level per unit ||p||^2, 2^-22 sqrt(n) for FP32 entries and sums);
@@ -127,10 +93,13 @@ __device__ __forceinline__ bool cg_block_sum(double v, double* __restrict__ part
 // iteration count, rz copied to S_RZ for the next direction, and the status
 // (0 running, 1 met tol, 2 rounding-level curvature, 3 non-finite, 4 maxit).  A stopped CG
 // (status != 0, set by an earlier launch, so the same in every CTA) makes this a no-op.
+// The new residual is also left split for the Woodbury apply (w; scaled by the exponent of the
+// previous ||r||, which every CTA reads before the last one overwrites it), so that the apply
+// needs no pass of its own.
 __global__ void __launch_bounds__(256) cg_step_kernel(double* __restrict__ s, double noise_coef, double* __restrict__ x,
                                                       double* __restrict__ Kx, double* __restrict__ r,
                                                       const double* __restrict__ p, const double* __restrict__ Kp,
-                                                      const double* __restrict__ Ap, int64_t n,
+                                                      const double* __restrict__ Ap, int64_t n, WbSplit w,
                                                       double* __restrict__ part, unsigned int* __restrict__ counter) {
   if ((int)s[S_CGST] != CG_RUN) return;
   const double pAp = s[S_PAP];
@@ -151,17 +120,28 @@ __global__ void __launch_bounds__(256) cg_step_kernel(double* __restrict__ s, do
     a = s[S_RZN] / pAp;
     pend = CG_RUN;
   }
-  double acc = 0.0;
+  const int e = norm_exponent(s[S_RR], false);
+  const double sr = pow2(-e);
+  const double sw = w.us ? pow2(-max_exponent(*reinterpret_cast<const unsigned long long*>(s + S_WMAX))) : 0.0;
+  double acc[1] = {0.0};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     x[i] += a * p[i];
     if (Kx) Kx[i] += a * Kp[i];
     const double ri = r[i] - a * Ap[i];
     r[i] = ri;
-    acc += ri * ri;
+    if (w.us) {
+      float2 v;
+      df_split((w.Linv[i] * sw) * (ri * sr), v.x, v.y);
+      w.us[i] = v;
+    }
+    acc[0] += ri * ri;
   }
+  if (w.us && blockIdx.x == 0)
+    for (int c = threadIdx.x; c < w.N; c += 256) w.t[c] = 0.0;
   double rr;
-  if (!cg_block_sum(acc, part, counter, &rr) || threadIdx.x != 0) return;
+  if (!grid_sums(acc, part, counter, &rr) || threadIdx.x != 0) return;
   s[S_RR] = rr;
+  s[S_WEXP] = (double)e;
   s[S_A] = a;
   s[S_RZ] = s[S_RZN];
   if (a != 0.0) s[S_CGITS] += 1.0;
@@ -174,34 +154,47 @@ __global__ void __launch_bounds__(256) cg_step_kernel(double* __restrict__ s, do
   s[S_CGST] = st;
 }
 
-// p = z + beta p with beta = rz_new / rz (S_RZN, S_RZ), and ||p||^2 into S_PP, while CG runs.
+// p = z + beta p with beta = rz_new / rz (S_RZN, S_RZ), and ||p||^2 and 1^T p into S_PP and S_SUMP,
+// while CG runs.  v32 (nullable): the FP32 copy of p and the zeroed sums acc that the next FP32
+// product wants (rows n .. ldn stay as sym_prep left them for v32).
 __global__ void __launch_bounds__(256) cg_dir_kernel(double* __restrict__ s, double* __restrict__ p,
-                                                     const double* __restrict__ z, int64_t n,
+                                                     const double* __restrict__ z, int64_t n, int64_t ldn,
+                                                     float* __restrict__ v32, float* __restrict__ acc,
                                                      double* __restrict__ part, unsigned int* __restrict__ counter) {
   if ((int)s[S_CGST] != CG_RUN) return;
   const double b = s[S_RZN] / s[S_RZ];
-  double acc = 0.0;
+  double sums[2] = {0.0, 0.0}, tot;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double pi = z[i] + b * p[i];
     p[i] = pi;
-    acc += pi * pi;
+    if (v32) {
+      v32[i] = (float)pi;
+      acc[i] = 0.f;
+    }
+    sums[0] += pi * pi;
+    sums[1] += pi;
   }
-  double pp;
-  if (!cg_block_sum(acc, part, counter, &pp) || threadIdx.x != 0) return;
-  s[S_PP] = pp;
-  s[S_BETA] = b;
+  if (v32 && blockIdx.x == 0 && n + threadIdx.x < ldn) acc[n + threadIdx.x] = 0.f;   // ldn - n < 128
+  if (!grid_sums(sums, part, counter, &tot)) return;
+  if (threadIdx.x == 0) {
+    s[S_PP] = tot;
+    s[S_BETA] = b;
+  } else if (threadIdx.x == 1) {
+    s[S_SUMP] = tot;
+  }
 }
 
 static cudaError_t cg_step(Handle* h, double noise_coef, double* x, double* Kx, double* r, const double* p,
                            const double* Kp, const double* Ap, cudaStream_t st) {
-  cg_step_kernel<<<grid_for(h->n, 256, 304), 256, 0, st>>>(h->scal, noise_coef, x, Kx, r, p, Kp, Ap, h->n, h->red_part,
-                                                           h->red_counter);
+  cg_step_kernel<<<grid_for(h->n, 256, 304), 256, 0, st>>>(h->scal, noise_coef, x, Kx, r, p, Kp, Ap, h->n,
+                                                           precond_split(h), h->red_part, h->red_counter);
   h->launches++;
   return cudaGetLastError();
 }
 
-static cudaError_t cg_dir(Handle* h, double* p, const double* z, cudaStream_t st) {
-  cg_dir_kernel<<<grid_for(h->n, 256, 304), 256, 0, st>>>(h->scal, p, z, h->n, h->red_part, h->red_counter);
+static cudaError_t cg_dir(Handle* h, double* p, const double* z, float* v32, float* acc, cudaStream_t st) {
+  cg_dir_kernel<<<grid_for(h->n, 256, 304), 256, 0, st>>>(h->scal, p, z, h->n, h->ldn, v32, acc, h->red_part,
+                                                          h->red_counter);
   h->launches++;
   return cudaGetLastError();
 }
@@ -217,34 +210,39 @@ __global__ void cg_init_kernel(double* __restrict__ s, double tol2, double maxit
 // CG iterations per host status read: one per product when a product costs far more
 // than a host round trip, more when the products are cheap (small n).
 static int cg_block(Handle* h) {
-  if (h->rdv) return 1;                 // grid columns meet at every product on the host
+  if (h->rdv) return 1;                 // grid columns run in the grid's CG engine
   if (h->n <= 8192) return 16;
   if (h->n <= 32768) return 4;
   return 1;
 }
 
 cudaError_t cg_after_product(Handle* h, const CgArgs& a, cudaStream_t st) {
-  const int64_t n = h->n;
   double* s = h->scal;
   double* r = vec(h, V_R);
   double* zz = vec(h, V_ZZ);
   double* p = vec(h, V_P);
   double* Ap = vec(h, V_AP);
   double* Kp = vec(h, V_KP);
-  RedArgs rs;
-  rs.a = p;
-  cudaError_t e = reduce(h, RED_SUM, rs, n, s + S_SUMP, st);
+  cudaError_t e = cg_operator(h, Ap, Kp, p, a.L, st);
   if (e != cudaSuccess) return e;
-  high_op_kernel<<<grid_for(n), 256, 0, st>>>(Ap, Kp, p, a.L, s + S_SUMP, a.gam, n);
-  h->launches++;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  RedArgs rd;
-  rd.a = p;
-  rd.b = Ap;
-  if ((e = reduce(h, RED_DOT, rd, n, s + S_PAP, st)) != cudaSuccess) return e;
   if ((e = cg_step(h, a.noise_coef, a.x, a.Kx, r, p, Kp, Ap, st)) != cudaSuccess) return e;
-  if ((e = precond_apply(h, a.Lpre, r, zz, s + S_RZN, st, s + S_RR)) != cudaSuccess) return e;
-  return cg_dir(h, p, zz, st);
+  if ((e = precond_apply(h, a.Lpre, r, zz, s + S_RZN, st, s + S_RR, true)) != cudaSuccess) return e;
+  return cg_dir(h, p, zz, nullptr, nullptr, st);
+}
+
+cudaError_t cg_begin(Handle* h, const double* Lpre, double gam, double tol, int maxit, cudaStream_t st) {
+  double* s = h->scal;
+  double* zz = vec(h, V_ZZ);
+  double* p = vec(h, V_P);
+  cudaError_t e = precond_apply(h, Lpre, vec(h, V_R), zz, s + S_RZN, st, s + S_RR);
+  if (e != cudaSuccess || (e = vec_copy(h, p, zz, h->n, st)) != cudaSuccess) return e;
+  RedArgs rp;
+  rp.a = p;
+  if ((e = reduce(h, RED_NORM2, rp, h->n, s + S_PP, st)) != cudaSuccess) return e;
+  if ((e = reduce(h, RED_SUM, rp, h->n, s + S_SUMP, st)) != cudaSuccess) return e;
+  cg_init_kernel<<<1, 1, 0, st>>>(s, tol * tol, (double)maxit, gam);
+  h->launches++;
+  return cudaGetLastError();
 }
 
 kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const double* b, double* x, double* Kx,
@@ -271,14 +269,7 @@ kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const
   RedArgs rn;
   rn.a = r;
   CK(reduce(h, RED_NORM2, rn, n, s + S_RR, st));
-  CK(precond_apply(h, Lpre, r, zz, s + S_RZN, st, s + S_RR));
-  CK(vec_copy(h, p, zz, n, st));
-  RedArgs rp;
-  rp.a = p;
-  CK(reduce(h, RED_NORM2, rp, n, s + S_PP, st));
-  cg_init_kernel<<<1, 1, 0, st>>>(s, tol * tol, (double)maxit, gam);
-  h->launches++;
-  CK(cudaGetLastError());
+  CK(cg_begin(h, Lpre, gam, tol, maxit, st));
   CK(fetch(h, S_RR, 1, st));
   const double rr0 = h->scal_host[S_RR];
   if (!std::isfinite(rr0)) return fail(h, KQR_BREAKDOWN, "CG: non-finite residual");
@@ -293,6 +284,13 @@ kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const
   // there the guard only keeps the step from overflowing on a near-zero curvature.
   const double noise_coef = std::sqrt((double)n) * (high_products ? std::ldexp(1.0, -44)
                                                                    : (lowprec ? std::ldexp(1.0, -40) : std::ldexp(1.0, -22)));
+  // FP32 products that accumulate with atomics find their vector prepared: by sym_prep here, by the
+  // direction kernel afterwards.
+  float *v32 = nullptr, *acc = nullptr;
+  if (!h->rdv && !(h->cg_high_on && !lowprec) && (h->opt.symmetric_gram || (h->kstore && !lowprec))) {
+    CK(sym_buffers(h, &v32, &acc));
+    CK(sym_prep(h, p, v32, acc, nullptr, st));
+  }
   // One block of CG iterations, every scalar on the device.
   auto enqueue_block = [&]() -> cudaError_t {
     cudaError_t e = cudaSuccess;
@@ -305,14 +303,16 @@ kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const
       ep.pvec = p;
       ep.dot_out = s + S_PAP;
       ep.raw_out = Kp;
-      if (h->rdv) e = op_product(h, p, Ap, Kp, L, gam, s + S_SUMP, s + S_PAP, h->cg_high_on, st);
-      else if (h->cg_high_on && !lowprec) e = op_product(h, p, Ap, Kp, L, gam, s + S_SUMP, s + S_PAP, true, st);
-      else if (lowprec) e = gram_rbf_tc(h, p, Ap, 1, false, &ep, st);
+      ep.prepped = v32 != nullptr;
+      if (h->cg_high_on && !lowprec) {
+        e = gram_high(h, p, Kp, 1, st);
+        if (e == cudaSuccess) e = cg_operator(h, Ap, Kp, p, L, st);
+      } else if (lowprec) e = gram_rbf_tc(h, p, Ap, 1, false, &ep, st);
       else e = gram_f32(h, p, Ap, 1, &ep, st);
       if (e != cudaSuccess) break;
       if ((e = cg_step(h, noise_coef, x, Kx, r, p, Kp, Ap, st)) != cudaSuccess) break;
-      if ((e = precond_apply(h, Lpre, r, zz, s + S_RZN, st, s + S_RR)) != cudaSuccess) break;
-      e = cg_dir(h, p, zz, st);
+      if ((e = precond_apply(h, Lpre, r, zz, s + S_RZN, st, s + S_RR, true)) != cudaSuccess) break;
+      e = cg_dir(h, p, zz, v32, acc, st);
     }
     return e;
   };

@@ -5,9 +5,10 @@
 // residuals and of the line search of Alg. 3.  All FP64.
 //
 // Reductions are deterministic: each block writes its partial sums, and the
-// last block to finish adds the partials in block order.
+// last block to finish adds the partials in a fixed order.
 #include "kqr_internal.h"
 #include "ptx.cuh"
+#include "reduce.cuh"
 
 namespace kqr {
 
@@ -23,33 +24,8 @@ __global__ void __launch_bounds__(256) reduce_kernel(F f, int64_t n, double* __r
   for (int s = 0; s < NS; ++s) acc[s] = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     f(i, acc);
-  __shared__ double ws[8][NS];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    double v = acc[s];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) ws[warp][s] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < NS) {
-    double v = 0.0;
-    for (int w = 0; w < 8; ++w) v += ws[w][threadIdx.x];
-    part[blockIdx.x * NS + threadIdx.x] = v;
-  }
-  __threadfence();
-  __shared__ bool last;
-  if (threadIdx.x == 0) last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (last) {
-    __threadfence();
-    if (threadIdx.x < NS) {
-      double v = 0.0;
-      for (int b = 0; b < (int)gridDim.x; ++b) v += part[b * NS + threadIdx.x];
-      out[threadIdx.x] = v;
-    }
-    if (threadIdx.x == 0) *counter = 0u;
-  }
+  double tot;
+  if (grid_sums(acc, part, counter, &tot) && threadIdx.x < NS) out[threadIdx.x] = tot;
 }
 
 template <int NS, typename F>
@@ -140,35 +116,6 @@ __global__ void fill_L_kernel(double* L, double base, const double* dres, int64_
   GRID_LOOP(i, n) L[i] = base + (dres ? dres[i] : 0.0);
 }
 
-// CG step: x += a p, Kx += a Kp, r -= a Ap, and ||r||^2.
-struct FCgUpdate {
-  double *x, *Kx, *r;
-  const double *p, *Kp, *Ap, *a_dev;
-  __device__ void operator()(int64_t i, double* acc) const {
-    const double a = *a_dev;
-    x[i] += a * p[i];
-    if (Kx) Kx[i] += a * Kp[i];
-    const double ri = r[i] - a * Ap[i];
-    r[i] = ri;
-    acc[0] += ri * ri;
-  }
-};
-
-// p = z + beta p, unless the device-resident CG status (stop_dev, nullable) says it
-// stopped; and ||p||^2 of the resulting p.
-struct FCgDir {
-  double* p;
-  const double *z, *beta_dev, *stop_dev;
-  __device__ void operator()(int64_t i, double* acc) const {
-    double pi = p[i];
-    if (!(stop_dev && *stop_dev != 0.0)) {
-      pi = z[i] + (*beta_dev) * pi;
-      p[i] = pi;
-    }
-    acc[0] += pi * pi;
-  }
-};
-
 __global__ void op_residual_kernel(double* r, const double* b, const double* x, const double* Kx, double gam,
                                    const double* sum_x, const double* L, int64_t n) {
   const double sx = *sum_x;
@@ -195,13 +142,14 @@ __global__ void mult_update_kernel(const double* alpha, double* v, double* z, do
 // Eq. (2.3) and eq. (3.1): w, v = Pi_B(w), S, grad, L (and L + residual diagonal), ||grad||^2.
 struct FBoxGrad {
   const double *alpha, *z, *Ka, *y, *dres;
-  double beta, sigma, tau, lam, eps, sum_alpha;
+  double beta, sigma, tau, lam, eps;
+  const double* sum_alpha;   // device
   double *v, *S, *grad, *L, *Lpre;
   __device__ void operator()(int64_t i, double* acc) const {
     const double w = alpha[i] + z[i] / sigma;
     const double vi = clampd(w, tau - 1.0, tau);
     const double si = (w > tau - 1.0 && w < tau) ? 1.0 : 0.0;
-    const double g = Ka[i] / lam - y[i] + beta + sigma * sum_alpha + sigma * (w - vi);
+    const double g = Ka[i] / lam - y[i] + beta + sigma * (*sum_alpha) + sigma * (w - vi);
     if (v) v[i] = vi;
     if (S) S[i] = si;
     if (grad) grad[i] = g;
@@ -237,14 +185,6 @@ cudaError_t fill_L(Handle* h, double* L, double base, const double* dres, int64_
   fill_L_kernel<<<grid_for(n), 256, 0, st>>>(L, base, dres, n);
   return post(h);
 }
-cudaError_t cg_update(Handle* h, double* x, double* Kx, double* r, const double* p, const double* Kp,
-                      const double* Ap, const double* a_dev, int64_t n, double* rr_out, cudaStream_t st) {
-  return run_reduce<1>(h, FCgUpdate{x, Kx, r, p, Kp, Ap, a_dev}, n, rr_out, st);
-}
-cudaError_t cg_direction(Handle* h, double* p, const double* z, const double* beta_dev, const double* stop_dev,
-                         int64_t n, double* pp_out, cudaStream_t st) {
-  return run_reduce<1>(h, FCgDir{p, z, beta_dev, stop_dev}, n, pp_out, st);
-}
 cudaError_t op_residual(Handle* h, double* r, const double* b, const double* x, const double* Kx, double gam,
                         const double* sum_x, const double* L, int64_t n, cudaStream_t st) {
   op_residual_kernel<<<grid_for(n), 256, 0, st>>>(r, b, x, Kx, gam, sum_x, L, n);
@@ -271,11 +211,7 @@ cudaError_t box_grad(Handle* h, const double* alpha, const double* z, const doub
   // sum_i alpha_i first (deterministic), then the fused element-wise pass.
   cudaError_t e = run_reduce<1>(h, FSum{alpha}, n, h->scal + S_RED0 + 12, st);
   if (e != cudaSuccess) return e;
-  e = cudaMemcpyAsync(h->scal_host + S_RED0 + 12, h->scal + S_RED0 + 12, sizeof(double), cudaMemcpyDeviceToHost, st);
-  if (e != cudaSuccess) return e;
-  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-  const double sa = h->scal_host[S_RED0 + 12];
-  return run_reduce<1>(h, FBoxGrad{alpha, z, Kalpha, y, dres, beta, sigma, tau, lam, eps, sa, v, S, grad, Ldiag, Lpre},
+  return run_reduce<1>(h, FBoxGrad{alpha, z, Kalpha, y, dres, beta, sigma, tau, lam, eps, h->scal + S_RED0 + 12, v, S, grad, Ldiag, Lpre},
                        n, h->scal + S_RED0 + 13, st);
 }
 
