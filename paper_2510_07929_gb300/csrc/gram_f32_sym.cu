@@ -160,14 +160,14 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 // v (FP64, n) -> v32 [ldn] zero padded; acc [ldn] zeroed; optional sum of v.
 __global__ void __launch_bounds__(256) sym_prep_kernel(const double* __restrict__ V, float* __restrict__ v32,
-                                                       float* __restrict__ acc, int64_t n, int64_t ldn,
+                                                       double* __restrict__ acc, int64_t n, int64_t ldn,
                                                        double* __restrict__ part, unsigned int* __restrict__ counter,
                                                        double* __restrict__ sum_out) {
   double s[1] = {0.0};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ldn; i += (int64_t)gridDim.x * blockDim.x) {
     const double x = i < n ? V[i] : 0.0;
     v32[i] = (float)x;
-    acc[i] = 0.f;
+    acc[i] = 0.0;
     s[0] += x;
   }
   if (!sum_out) return;
@@ -176,7 +176,8 @@ __global__ void __launch_bounds__(256) sym_prep_kernel(const double* __restrict_
 }
 
 // out = acc (+ gam sum_p + L p), *dot_out = p . out, raw_out = acc.
-__global__ void __launch_bounds__(256) sym_finish_kernel(const float* __restrict__ acc, int64_t n,
+template <typename T>
+__global__ void __launch_bounds__(256) sym_finish_kernel(const T* __restrict__ acc, int64_t n,
                                                          double* __restrict__ out, GramEpilogue ep,
                                                          double* __restrict__ part,
                                                          unsigned int* __restrict__ counter) {
@@ -221,11 +222,13 @@ cudaError_t sym_units_ensure(Handle* h) {
 cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilogue* ep, cudaStream_t st) {
   cudaError_t e = sym_units_ensure(h);
   if (e != cudaSuccess) return e;
-  float *v32, *acc;
-  if ((e = sym_buffers(h, &v32, &acc)) != cudaSuccess) return e;
+  float* v32;
+  double* sums;
+  if ((e = sym_buffers(h, &v32, &sums)) != cudaSuccess) return e;
   GramEpilogue none;
   const GramEpilogue& g = ep ? *ep : none;
-  if (!g.prepped && (e = sym_prep(h, V, v32, acc, const_cast<double*>(g.sum_p), st)) != cudaSuccess) return e;
+  if (!g.prepped && (e = sym_prep(h, V, v32, sums, const_cast<double*>(g.sum_p), st)) != cudaSuccess) return e;
+  float* acc = reinterpret_cast<float*>(sums);
   const size_t smem = sym_smem_bytes((int)h->p);
   prof_mark(h, 0, true, st);
   if (h->kind == KQR_LAPLACIAN) {
@@ -242,15 +245,15 @@ cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilog
   prof_mark(h, 0, false, st);
   h->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return sym_finish(h, acc, U, g, st);
+  return sym_finish(h, acc, false, U, g, st);
 }
 
 }  // namespace kqr
 
 namespace kqr {
 
-cudaError_t sym_buffers(Handle* h, float** v32, float** acc) {
-  const size_t need = (size_t)h->ldn * sizeof(float) * 2;
+cudaError_t sym_buffers(Handle* h, float** v32, double** acc) {
+  const size_t need = (size_t)h->ldn * (sizeof(float) + sizeof(double));
   if (h->v32_cap < need) {
     dev_free(h, h->v32);
     h->v32 = (float*)dev_alloc(h, need);
@@ -258,21 +261,24 @@ cudaError_t sym_buffers(Handle* h, float** v32, float** acc) {
     if (!h->v32) return cudaErrorMemoryAllocation;
   }
   *v32 = h->v32;
-  *acc = h->v32 + h->ldn;
+  *acc = reinterpret_cast<double*>(h->v32 + h->ldn);   // ldn is a multiple of 128
   return cudaSuccess;
 }
 
-// v -> FP32 copy and zeroed FP32 accumulator (and 1^T v into *sum_out if given),
-// for products that accumulate with atomics (symmetric tiles, stored K).
-cudaError_t sym_prep(Handle* h, const double* V, float* v32, float* acc, double* sum_out, cudaStream_t st) {
+// v -> FP32 copy and zeroed sums (and 1^T v into *sum_out if given), for products that accumulate
+// with atomics (symmetric tiles, stored K).
+cudaError_t sym_prep(Handle* h, const double* V, float* v32, double* acc, double* sum_out, cudaStream_t st) {
   sym_prep_kernel<<<grid_for(h->ldn), 256, 0, st>>>(V, v32, acc, h->n, h->ldn, h->red_part, h->red_counter, sum_out);
   h->launches++;
   return cudaGetLastError();
 }
 
 // out = acc (+ the CG operator's terms of g).
-cudaError_t sym_finish(Handle* h, const float* acc, double* U, const GramEpilogue& g, cudaStream_t st) {
-  sym_finish_kernel<<<grid_for(h->n), 256, 0, st>>>(acc, h->n, U, g, h->red_part, h->red_counter);
+cudaError_t sym_finish(Handle* h, const void* acc, bool f64, double* U, const GramEpilogue& g, cudaStream_t st) {
+  if (f64)
+    sym_finish_kernel<double><<<grid_for(h->n), 256, 0, st>>>((const double*)acc, h->n, U, g, h->red_part, h->red_counter);
+  else
+    sym_finish_kernel<float><<<grid_for(h->n), 256, 0, st>>>((const float*)acc, h->n, U, g, h->red_part, h->red_counter);
   h->launches++;
   return cudaGetLastError();
 }

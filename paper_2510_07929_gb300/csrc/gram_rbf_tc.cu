@@ -88,6 +88,38 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// A load of 16 columns, and the wait that makes its registers valid (it waits for all of the thread's loads).
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                 "+r"(r[15])::"memory");
+}
+
+// Waits for all tensor-memory loads of this thread; a load of 8 columns without the wait.
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// Untiled bulk copy global -> shared (16-byte aligned addresses, size a multiple of 16).
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major operand in the canonical 128-byte
 // swizzled layout (8-row groups 1024 bytes apart), tcgen05 version bits 0b001.
 __device__ __forceinline__ uint64_t umma_desc_sw128(const void* p) {
@@ -522,280 +554,380 @@ static cudaError_t rbf_tc_product(Handle* h, const double* V, double* U, int m, 
 
 // ---- symmetric tiles for one right-hand side ------------------------------------------
 // K is symmetric, so each off-diagonal 128 x 128 tile K_JI (J > I) is formed once on the
-// tensor cores and used twice: u_J += K_JI v_I and u_I += K_JI^T v_J.  A work unit is a
-// row tile I and a run of column tiles J in [J0, J1) with J0 >= I.  The MMA computes
+// tensor cores and used twice: u_J += K_JI v_I and u_I += K_JI^T v_J.  The MMA computes
 // D = X_J X_I^T, so TMEM lane l is row j = J*128 + l and TMEM column c is i = I*128 + c.
 //
 // Operands (NTERMS): 3 = TF32 parts hi.hi + hi.lo + lo.hi, three MMAs per K = 8 step;
 // 16 = the same three products from fp16 parts concatenated along K (A' = [hi | hi | lo]
-// for J, B' = [hi | lo | hi] for I), one chain of ceil(3p / 16) MMAs of K = 16.  The MMAs
-// of a tile accumulate into one TMEM buffer and so run one after another; the short
-// chain of the fp16 form is what makes it faster; 1 = TF32 hi.hi alone (the TF32 product).
+// for J, B' = [hi | lo | hi] for I), one chain of ceil(3p / 16) MMAs of K = 16; 1 = TF32
+// hi.hi alone (the TF32 product).
 //
-// One CTA = 8 warps, two CTAs per SM; warp w reads TMEM lanes 32 (w mod 4) .. + 31 (the
-// lanes its warp may access) over the 64 columns 64 (w / 4) .. + 63.  Per element a thread
-// forms e = exp2(2 xs_j.xs_i - n_j [- n_i]) and adds e w_i to its row j's sum (a register
-// sum: u_J needs no exchange between threads) and e v_j to column i's sum, which stays in
-// a register across all tiles of the unit (I is fixed), so the exchange across the warp's
-// 32 rows happens once per unit.  With FOLD (every n < 60) exp2(-n_i) is folded into
-// w_i = v_i exp2(-n_i) and into the column results.
-//
-// No CTA-wide barrier inside the tile loop: thread 0 issues the TMA copies and MMAs; a
-// copy refills a stage once the MMAs that read it have completed (mma_done), an MMA
-// reuses a TMEM buffer once all 8 warps have read it out (tmem_free, one arrival per
-// warp).  Row sums go to the output with FP32 atomics per tile, column sums per unit.
+// What bounds it: one ex2 per entry, 32 lanes per clock and SM, 512 cycles a tile; the issue
+// slots come next (2.5 per entry: the exponent's FFMA and the two sums' FFMAs are packed
+// f32x2, one slot for two entries).  The rest of a tile has to hide behind that, so:
+//   - one persistent CTA per SM walks an equal share of the tiles, with no set-up or drain
+//     between tiles (units of 60 tiles spent a seventh of their time on it).  Tiles are
+//     ordered by rows 0, T-1, 1, T-2, ... of the upper triangle, so that short rows, where
+//     the row tile changes often, are spread over the CTAs;
+//   - 16 epilogue warps take their tiles at their own pace (warp w: TMEM lanes
+//     32 (w mod 4) .. + 31, 32 columns of I), four accumulators of 128 columns in tensor
+//     memory.  A warp's 32 columns are read in halves of 16, each while the half before it is
+//     worked on, the first half of the next tile included (0.36 ms without);
+//   - one warp issues the copies and another the MMAs, each with running stage indexes and
+//     descriptors and converged, an elected lane issuing: the thread that did both computed
+//     for longer than the tile's epilogue takes (0.80 ms), two threads in branches of their
+//     own took 0.45 ms.
+// n = 50000, p = 20 (fp16 operands): 0.31 ms a product, 0.50 ms with 16 warps on tiles of 60-tile
+// units and a CTA-wide barrier per tile; 0.127 ms is the ex2 unit's share.
+// Per element a thread forms e = exp2(2 xs_j.xs_i - n_j [- n_i]) and adds e w_i to its row
+// j's sum and e v_j to column i's sum, which stays in a register while the row tile I is the
+// same, so the exchange across the warp's 32 rows happens once per I.  With FOLD (every
+// n < 60) exp2(-n_i) is folded into w_i = v_i exp2(-n_i) and into the column results.  Row
+// sums per tile and column sums per I go to FP64 sums with atomics (FP32 ones, added to
+// a thousand times per row, were the largest error of the product).
 // Every wait is bounded; on a timeout the CTA records the error, drains its own copies
 // and MMAs (bounded) and frees its tensor memory.
-constexpr int kSymWarps = 8;
-constexpr int kSymCols = 64;  // columns of tile I per warp: two 32-column TMEM loads
-constexpr int kSymBufs = 2;   // TMEM accumulator buffers of 128 columns (two CTAs per SM)
+constexpr int kSymEpi = 16;                         // epilogue warps
+constexpr int kSymCols = 32;                       // columns of tile I per warp
+static_assert(kSymEpi * 32 * kSymCols == kTile * kTile, "the warps cover a tile");
+constexpr int kSymThreads = (kSymEpi + 2) * 32;    // + copy warp + MMA warp
+constexpr int kSymBufs = 4;                        // TMEM accumulators of 128 columns
+constexpr int kSymMaxStages = 4;
 
-// nstage X_J stages; the MMAs of tile q are issued nstage / 2 iterations before its
-// epilogue, and the copy of tile q + nstage is issued as soon as the MMAs of tile q have
-// completed.
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t r, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// Walk over the order of tiles: row pair k = rows k and T - 1 - k, T + 1 tiles together (the middle
+// row of an odd T alone).  I, J: the current tile; left: tiles of this row from here on.
+struct SymWalk {
+  int T, k, I, J, left;
+  bool second;
+  __device__ __forceinline__ SymWalk(int64_t t, int T_) : T(T_) {
+    k = (int)(t / (T + 1));
+    const int off = (int)(t - (int64_t)k * (T + 1));
+    second = off >= T - k;
+    I = second ? T - 1 - k : k;
+    J = I + (second ? off - (T - k) : off);
+    left = T - J;
+  }
+  // to the next tile; true if it begins another row
+  __device__ __forceinline__ bool next() {
+    ++J;
+    if (--left) return false;
+    if (second) ++k;
+    second = !second;
+    I = second ? T - 1 - k : k;
+    J = I;
+    left = T - I;
+    return true;
+  }
+};
+
 template <int NTERMS, bool FOLD>
-__global__ void __launch_bounds__(kSymWarps * 32, 2)
+__global__ void __launch_bounds__(kSymThreads, 1)
     gram_rbf_tc_sym_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
-                           const float* __restrict__ nrm, const float* __restrict__ v32, const int4* __restrict__ units,
-                           float* __restrict__ acc, int ksteps, int katoms, int nstage, int* __restrict__ err) {
+                           const float* __restrict__ nrm, const float* __restrict__ v32, double* __restrict__ acc, int T,
+                           int ksteps, int katoms, int nibuf, int nstage, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                          ~static_cast<uintptr_t>(1023));
   const uint32_t tb = (uint32_t)katoms * kAtomBytes;
-  unsigned char* XIh = base;
-  unsigned char* XIl = XIh + tb;
-  // stage s: hi part at base + (2 + 2 s) tb, lo part right after it
-  float* s_w = reinterpret_cast<float*>(base + (size_t)(2 + 2 * nstage) * tb);   // [128] column factors of tile I
-  float* s_ni = s_w + 128;                                                       // [128] n_i of tile I (without FOLD)
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_ni + 128);
-  uint64_t* full_i = &bars[0];
-  uint64_t* full_j = &bars[1];                   // [nstage] X_J stage landed
-  uint64_t* mma_done = &bars[1 + 4];             // [kSymBufs] MMAs of TMEM buffer b completed
-  uint64_t* tmem_free = &bars[1 + 4 + kSymBufs]; // [kSymBufs] all warps have read TMEM buffer b
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 1 + 4 + 2 * kSymBufs);
+  const uint32_t sb = (NTERMS == 3 ? 2u : 1u) * tb;   // one tile: hi part, then (NTERMS = 3) lo part
+  unsigned char* xj = base + nibuf * sb;              // nibuf (1 or 2) row tiles I, then nstage tiles J
+  float* s_w = reinterpret_cast<float*>(xj + (size_t)nstage * sb);   // [kSymEpi][kSymCols] column factors of each warp
+  float* s_ni = s_w + 512;                                           // [kSymEpi][kSymCols] n_i (without FOLD)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_ni + 512);
+  uint64_t* full_i = &bars[0];                        // [2] row tile landed
+  uint64_t* full_j = &bars[2];                        // [nstage] X_J stage landed
+  uint64_t* mma_done = &bars[2 + kSymMaxStages];      // [kSymBufs] MMAs of TMEM buffer b completed
+  uint64_t* tmem_free = mma_done + kSymBufs;          // [kSymBufs] all warps have read TMEM buffer b
+  uint64_t* stage_free = tmem_free + kSymBufs;        // [nstage] the MMAs that read the stage completed
+  uint64_t* i_free = stage_free + kSymMaxStages;      // [2] the MMAs that read the row tile completed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(i_free + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  // thread 0's bookkeeping, in shared memory to spare registers: the latest tile whose copy,
-  // and the latest whose MMAs, may still be in flight
-  int* load_pending = reinterpret_cast<int*>(tmem_slot + 2);
-  int* mma_pending = load_pending + 1;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int lq = warp & 3, cq = warp >> 2;
-  const int4 unit = units[blockIdx.x];
-  const int ti = unit.x;
-  const int jt0 = unit.y, jt1 = unit.z;
-  const int nt = jt1 - jt0;
-  const int look = nstage / 2;
-  const uint32_t load_bytes = (NTERMS == 3 ? 2u : 1u) * tb;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const int64_t total = (int64_t)T * (T + 1) / 2;
+  const int64_t t0 = total * blockIdx.x / gridDim.x;
+  const int nt = (int)(total * (blockIdx.x + 1) / gridDim.x - t0);
 
-  if (warp == 0) {
+  if (warp == kSymEpi) {
     tmem_alloc(tmem_slot, 128 * kSymBufs);
     tmem_relinquish();
   }
   if (tid == 0) {
-    mbar_init(full_i, 1);
-    for (int s = 0; s < nstage; ++s) mbar_init(&full_j[s], 1);
+    for (int k = 0; k < 2; ++k) {
+      mbar_init(&full_i[k], 1);
+      mbar_init(&i_free[k], 1);
+    }
+    for (int s = 0; s < nstage; ++s) {
+      mbar_init(&full_j[s], 1);
+      mbar_init(&stage_free[s], 1);
+    }
     for (int b = 0; b < kSymBufs; ++b) {
       mbar_init(&mma_done[b], 1);
-      mbar_init(&tmem_free[b], kSymWarps);
+      mbar_init(&tmem_free[b], kSymEpi);
     }
     *abort_flag = 0;
     fence_mbar_init();
-  }
-  if (tid < 128) {
-    const float n_i = nrm[ti * 128 + tid];
-    s_w[tid] = v32[ti * 128 + tid] * (FOLD ? ex2_approx(-n_i) : 1.f);
-    s_ni[tid] = n_i;
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  auto stage_hi = [&](int s) { return base + (size_t)(2 + 2 * s) * tb; };
-  auto load_tile = [&](int t) {   // tile t of the unit into stage t mod nstage
-    const int s = t % nstage;
-    unsigned char* dh = stage_hi(s);
-    mbar_arrive_expect_tx(&full_j[s], load_bytes);
-    for (int a = 0; a < katoms; ++a) {
-      tma_load_2d(dh + a * kAtomBytes, &tm_hi, a * 32, (jt0 + t) * 128, &full_j[s]);
-      if (NTERMS == 3) tma_load_2d(dh + tb + a * kAtomBytes, &tm_lo, a * 32, (jt0 + t) * 128, &full_j[s]);
-    }
-  };
-  if (tid == 0) {
-    *load_pending = -1;
-    *mma_pending = -1;
-    mbar_arrive_expect_tx(full_i, load_bytes);
-    for (int a = 0; a < katoms; ++a) {
+  if (warp == kSymEpi) {
+    // ---- copies, in the order of the MMAs (converged warp, one elected lane)
+    if (nt > 0) {
+      const bool elected = elect_one();
       // with fp16 operands tm_hi maps A' (the J rows) and tm_lo maps B' (the I rows)
-      tma_load_2d(XIh + a * kAtomBytes, NTERMS == 16 ? &tm_lo : &tm_hi, a * 32, ti * 128, full_i);
-      if (NTERMS == 3) tma_load_2d(XIl + a * kAtomBytes, &tm_lo, a * 32, ti * 128, full_i);
-    }
-    for (int t = 0; t < nstage && t < nt; ++t) {
-      load_tile(t);
-      *load_pending = t;
-    }
-  }
-  // FP32 accumulate, A and B K-major, N = 128, M = 128; operands TF32 (format 2) or fp16 (0)
-  const uint32_t idesc = (1u << 4) | (NTERMS == 16 ? 0u : (2u << 7) | (2u << 10)) | ((128u >> 3) << 17) |
-                         ((128u >> 4) << 24);
-  float cacc[kSymCols];   // column sums of tile I over this warp's 32 rows, across the unit's tiles
-#pragma unroll
-  for (int c = 0; c < kSymCols; ++c) cacc[c] = 0.f;
-  bool ok = true;   // warp-uniform: every wait of this warp succeeded
-  // this thread's row of the next epilogue tile, loaded one tile ahead
-  const int jrow = jt0 * 128 + lq * 32 + lane;
-  float n_nx = __ldg(nrm + jrow);
-  float v_nx = jt0 == ti ? 0.f : __ldg(v32 + jrow);   // the diagonal tile gives row sums only
-
-  for (int q = 0; q < nt + look; ++q) {
-    if (tid == 0 && q < nt) {
-      const int s = q % nstage, b = q % kSymBufs;
-      bool w_ok = true;
-      if (q == 0) w_ok = mbar_wait_bounded(full_i, 0, err);
-      if (w_ok) w_ok = mbar_wait_bounded(&full_j[s], (uint32_t)((q / nstage) & 1), err);
-      // TMEM buffer b last held tile q - kSymBufs: every warp must have read it out
-      if (w_ok && q >= kSymBufs)
-        w_ok = mbar_wait_bounded(&tmem_free[b], (uint32_t)((q / kSymBufs - 1) & 1), err);
-      if (w_ok) {
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(b * 128);
-        const unsigned char* ah = stage_hi(s);
-        const unsigned char* al = ah + tb;
-        for (int k = 0; k < ksteps; ++k) {
-          const uint32_t off = (uint32_t)(k >> 2) * kAtomBytes + (uint32_t)(k & 3) * 32u;
-          if (NTERMS == 16) umma_f16(d, umma_desc_sw128(ah + off), umma_desc_sw128(XIh + off), idesc, k > 0 ? 1u : 0u);
-          else umma_tf32(d, umma_desc_sw128(ah + off), umma_desc_sw128(XIh + off), idesc, k > 0 ? 1u : 0u);
-          if (NTERMS == 3) {
-            umma_tf32(d, umma_desc_sw128(ah + off), umma_desc_sw128(XIl + off), idesc, 1u);
-            umma_tf32(d, umma_desc_sw128(al + off), umma_desc_sw128(XIh + off), idesc, 1u);
+      auto load_tile = [&](unsigned char* dst, int row_tile, const CUtensorMap* hi, uint64_t* bar) {
+        if (!elected) return;
+        mbar_arrive_expect_tx(bar, sb);
+        for (int a = 0; a < katoms; ++a) {
+          tma_load_2d(dst + a * kAtomBytes, hi, a * 32, row_tile * 128, bar);
+          if (NTERMS == 3) tma_load_2d(dst + tb + a * kAtomBytes, &tm_lo, a * 32, row_tile * 128, bar);
+        }
+      };
+      SymWalk w(t0, T);
+      int s = 0, ib = 0, q = 0, ki = 0;
+      uint32_t ph = 1, iph = 1;    // parity of the free barriers: the first use of a buffer does not wait
+      bool fresh = true, ok = true;
+      for (; q < nt; ++q) {
+        if (fresh) {
+          ok = __all_sync(0xffffffffu, mbar_wait_bounded(&i_free[ib], iph, err));
+          if (!ok) break;
+          load_tile(base + (size_t)ib * sb, w.I, NTERMS == 16 ? &tm_lo : &tm_hi, &full_i[ib]);
+          __syncwarp();
+          ++ki;
+          if (++ib == nibuf) {
+            ib = 0;
+            iph ^= 1;
           }
         }
-        umma_commit(&mma_done[b]);
-        *mma_pending = q;
-      } else {
-        *abort_flag = 1;
+        ok = __all_sync(0xffffffffu, *abort_flag == 0 && mbar_wait_bounded(&stage_free[s], ph, err));
+        if (!ok) break;
+        load_tile(xj + (size_t)s * sb, w.J, &tm_hi, &full_j[s]);
+        __syncwarp();
+        if (++s == nstage) {
+          s = 0;
+          ph ^= 1;
+        }
+        fresh = w.next();
+      }
+      if (!ok) *abort_flag = 1;
+      // the CTA must not exit with a copy in flight: wait (bounded) for the last one of every buffer
+      for (int k = ki > nibuf ? ki - nibuf : 0; k < ki; ++k)
+        mbar_wait_bounded(&full_i[k % nibuf], (uint32_t)((k / nibuf) & 1), err);
+      for (int t = q > nstage ? q - nstage : 0; t < q; ++t)
+        mbar_wait_bounded(&full_j[t % nstage], (uint32_t)((t / nstage) & 1), err);
+    }
+  } else if (warp == kSymEpi + 1) {
+    // ---- MMAs: the warp stays converged, so that indexes and descriptors are uniform values; one
+    // elected lane issues (issued from a branch of one lane an MMA took hundreds of cycles)
+    if (nt > 0) {
+      const bool elected = elect_one();
+      // FP32 accumulate, A and B K-major, N = 128, M = 128; operands TF32 (format 2) or fp16 (0)
+      const uint32_t idesc = (1u << 4) | (NTERMS == 16 ? 0u : (2u << 7) | (2u << 10)) | ((128u >> 3) << 17) |
+                             ((128u >> 4) << 24);
+      const uint64_t desc_i = umma_desc_sw128(base), desc_j = umma_desc_sw128(xj);
+      const uint32_t dhi = (uint32_t)(desc_i >> 32), t16 = tb / 16u, s16 = sb / 16u;
+      auto dsc = [&](uint32_t lo) { return ((uint64_t)dhi << 32) | lo; };
+      SymWalk w(t0, T);
+      int s = 0, ib = 0, b = 0, q = 0;
+      uint32_t ph = 0, iph = 0, fph = 1;
+      uint32_t aj = (uint32_t)desc_j, bi = (uint32_t)desc_i;
+      bool fresh = true, ok = true;
+      for (; q < nt; ++q) {
+        if (fresh) ok = mbar_wait_bounded(&full_i[ib], iph, err);
+        // TMEM buffer b last held tile q - kSymBufs: every warp must have read it out
+        ok = ok && mbar_wait_bounded(&tmem_free[b], fph, err) && mbar_wait_bounded(&full_j[s], ph, err);
+        if (!__all_sync(0xffffffffu, ok && *abort_flag == 0)) break;
+        tc_fence_after();
+        const uint32_t d = tmem + (uint32_t)(b * 128);
+        if (elected) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            if (k < ksteps) {
+              const uint32_t off = ((uint32_t)(k >> 2) * kAtomBytes + (uint32_t)(k & 3) * 32u) / 16u;
+              if (NTERMS == 16) umma_f16(d, dsc(aj + off), dsc(bi + off), idesc, k > 0 ? 1u : 0u);
+              else umma_tf32(d, dsc(aj + off), dsc(bi + off), idesc, k > 0 ? 1u : 0u);
+              if (NTERMS == 3) {
+                umma_tf32(d, dsc(aj + off), dsc(bi + t16 + off), idesc, 1u);
+                umma_tf32(d, dsc(aj + t16 + off), dsc(bi + off), idesc, 1u);
+              }
+            }
+          }
+          umma_commit(&mma_done[b]);
+          umma_commit(&stage_free[s]);
+        }
+        __syncwarp();
+        if (++b == kSymBufs) {
+          b = 0;
+          fph ^= 1;
+        }
+        aj += s16;
+        if (++s == nstage) {
+          s = 0;
+          ph ^= 1;
+          aj = (uint32_t)desc_j;
+        }
+        fresh = w.next();
+        if (fresh && q + 1 < nt) {
+          if (elected) umma_commit(&i_free[ib]);
+          __syncwarp();
+          bi += s16;
+          if (++ib == nibuf) {
+            ib = 0;
+            iph ^= 1;
+            bi = (uint32_t)desc_i;
+          }
+        }
+      }
+      if (q < nt) *abort_flag = 1;
+      // let the MMAs and commits in flight finish (bounded) before the tensor memory is freed
+      if (q > 0) {
+        mbar_wait_bounded(&mma_done[(q - 1) % kSymBufs], (uint32_t)(((q - 1) / kSymBufs) & 1), err);
+        mbar_wait_bounded(&stage_free[(q - 1) % nstage], (uint32_t)(((q - 1) / nstage) & 1), err);
       }
     }
-    if (q >= look) {
-      const int pq = q - look, b = pq % kSymBufs;
-      const float n_j = n_nx, v_j = v_nx;
-      if (pq + 1 < nt) {
-        n_nx = __ldg(nrm + jrow + (pq + 1) * 128);
-        v_nx = jt0 + pq + 1 == ti ? 0.f : __ldg(v32 + jrow + (pq + 1) * 128);
+  } else if (nt > 0) {
+    const int lq = warp & 3, cq = warp >> 2;
+    float* wq = s_w + warp * kSymCols;
+    float* nq = s_ni + warp * kSymCols;
+    uint64_t cacc[kSymCols / 2];   // column sums of tile I over this warp's 32 rows, across the tiles of this I
+    const uint64_t two = pack2(2.f, 2.f);
+    SymWalk w(t0, T);
+    int I = -1;
+    bool fresh = true, ok = true;
+    const int lrow = lq * 32 + lane;
+    float n_nx = __ldg(nrm + w.J * 128 + lrow);
+    float v_nx = w.J == w.I ? 0.f : __ldg(v32 + w.J * 128 + lrow);   // the diagonal tile gives row sums only
+    // column sums: reduce-scatter each 32 over the warp's 32 rows, so that lane l ends with column l
+    auto flush = [&]() {
+      float ch[32];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) unpack2(cacc[c], ch[2 * c], ch[2 * c + 1]);
+#pragma unroll
+      for (int wd = 16; wd >= 1; wd >>= 1) {
+        const bool up = (lane & wd) != 0;
+#pragma unroll
+        for (int i = 0; i < wd; ++i) {
+          const float keep = up ? ch[i + wd] : ch[i], send = up ? ch[i] : ch[i + wd];
+          ch[i] = keep + __shfl_xor_sync(0xffffffffu, send, wd);
+        }
       }
-      const bool landed = __all_sync(
-          0xffffffffu, *abort_flag == 0 && mbar_wait_bounded(&mma_done[b], (uint32_t)((pq / kSymBufs) & 1), err));
-      if (!landed) {
-        ok = false;
+      const float f = FOLD ? ex2_approx(-nq[lane]) : 1.f;
+      atomicAdd(acc + I * 128 + cq * kSymCols + lane, (double)(ch[0] * f));
+    };
+    const uint32_t tcol = tmem + (uint32_t)(cq * kSymCols) + ((uint32_t)(lq * 32) << 16);
+    uint32_t ph = 0;
+    int b = 0;
+    // the accumulators come in halves of 16 columns, each loaded while the half before it is worked on
+    uint32_t g0[16], g1[16];
+    auto wait_tile = [&]() {
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(&mma_done[b], ph, err));
+      if (!ok) {
         *abort_flag = 1;
-        break;
+        return;
       }
       tc_fence_after();
-      // the MMAs of tile pq have completed, so its stage is free: refill it with tile pq + nstage
-      if (tid == 0 && pq + nstage < nt) {
-        load_tile(pq + nstage);
-        *load_pending = pq + nstage;
-      }
-      float racc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int h = 0; h < kSymCols / 32; ++h) {
-      float g[32];
-      tmem_ld32(tmem + (uint32_t)(b * 128 + cq * kSymCols + h * 32) + ((uint32_t)(lq * 32) << 16), g);
-      if (h == kSymCols / 32 - 1) {
-        tc_fence_before();
+      tmem_ld16_nowait(tcol + (uint32_t)(b * 128), g0);
+    };
+    wait_tile();
+    for (int q = 0; q < nt && ok; ++q) {
+      if (fresh) {
+        if (I >= 0) flush();
+        I = w.I;
         __syncwarp();
-        if (lane == 0) mbar_arrive(&tmem_free[b]);
-      }
-      const float* wq = s_w + cq * kSymCols + h * 32;
-      const float* nq = s_ni + cq * kSymCols + h * 32;
+        const float n_i = __ldg(nrm + I * 128 + cq * kSymCols + lane);
+        wq[lane] = __ldg(v32 + I * 128 + cq * kSymCols + lane) * (FOLD ? ex2_approx(-n_i) : 1.f);
+        nq[lane] = n_i;
+        __syncwarp();
 #pragma unroll
-      for (int c4 = 0; c4 < 8; ++c4) {
-        const float4 w4 = *reinterpret_cast<const float4*>(wq + c4 * 4);
-        const float ww[4] = {w4.x, w4.y, w4.z, w4.w};
-        float nn[4] = {n_j, n_j, n_j, n_j};
-        if (!FOLD) {
-          const float4 n4 = *reinterpret_cast<const float4*>(nq + c4 * 4);
-          nn[0] += n4.x;
-          nn[1] += n4.y;
-          nn[2] += n4.z;
-          nn[3] += n4.w;
-        }
+        for (int c = 0; c < kSymCols / 2; ++c) cacc[c] = 0ull;
+      }
+      const int jrow = w.J * 128 + lrow;
+      const float n_j = n_nx, v_j = v_nx;
+      fresh = w.next();
+      if (q + 1 < nt) {
+        n_nx = __ldg(nrm + w.J * 128 + lrow);
+        v_nx = fresh ? 0.f : __ldg(v32 + w.J * 128 + lrow);   // a row begins with its diagonal tile
+      }
+      const uint64_t nj2 = pack2(-n_j, -n_j), vj2 = pack2(v_j, v_j);
+      uint64_t racc[2] = {0ull, 0ull};
+      auto half = [&](const uint32_t (&g)[16], auto half_tag) {
+        constexpr int hh = decltype(half_tag)::value;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int c = c4 * 4 + u;
-          const float e = ex2_approx(fmaf(2.f, g[c], -nn[u]));
-          racc[u] = fmaf(e, ww[u], racc[u]);
-          cacc[h * 32 + c] = fmaf(e, v_j, cacc[h * 32 + c]);
+        for (int c4 = 0; c4 < 4; ++c4) {
+          const float4 w4 = *reinterpret_cast<const float4*>(wq + hh * 16 + c4 * 4);
+          float4 n4;
+          if (!FOLD) n4 = *reinterpret_cast<const float4*>(nq + hh * 16 + c4 * 4);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int c = c4 * 2 + u;
+            uint64_t off = nj2;
+            if (!FOLD) off = add2(nj2, u ? pack2(-n4.z, -n4.w) : pack2(-n4.x, -n4.y));
+            float e0, e1;
+            unpack2(fma2(pack2(__uint_as_float(g[2 * c]), __uint_as_float(g[2 * c + 1])), two, off), e0, e1);
+            const uint64_t e = pack2(ex2_approx(e0), ex2_approx(e1));
+            racc[u] = fma2(e, u ? pack2(w4.z, w4.w) : pack2(w4.x, w4.y), racc[u]);
+            cacc[hh * 8 + c] = fma2(e, vj2, cacc[hh * 8 + c]);
+          }
         }
+      };
+      tmem_wait16(g0);
+      tmem_ld16_nowait(tcol + (uint32_t)(b * 128 + 16), g1);
+      half(g0, std::integral_constant<int, 0>{});
+      tmem_wait16(g1);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tmem_free[b]);
+      if (++b == kSymBufs) {
+        b = 0;
+        ph ^= 1;
       }
-      }
-      atomicAdd(acc + jrow + pq * 128, (racc[0] + racc[1]) + (racc[2] + racc[3]));
+      if (q + 1 < nt) wait_tile();
+      half(g1, std::integral_constant<int, 1>{});
+      float r0, r1;
+      unpack2(add2(racc[0], racc[1]), r0, r1);
+      atomicAdd(acc + jrow, (double)(r0 + r1));
     }
-  }
-  // column sums: reduce-scatter each 32 column partials over the warp's 32 rows, so that
-  // lane l ends with column cq kSymCols + 32 h + l of tile I
-  if (__all_sync(0xffffffffu, ok && *abort_flag == 0)) {
-#pragma unroll
-    for (int h = 0; h < kSymCols / 32; ++h) {
-      float* ch = cacc + h * 32;
-#pragma unroll
-      for (int w = 16; w >= 1; w >>= 1) {
-        const bool up = (lane & w) != 0;
-#pragma unroll
-        for (int i = 0; i < w; ++i) {
-          const float keep = up ? ch[i + w] : ch[i], send = up ? ch[i] : ch[i + w];
-          ch[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
-        }
-      }
-      const int col = cq * kSymCols + h * 32 + lane;
-      const float f = FOLD ? ex2_approx(-s_ni[col]) : 1.f;
-      atomicAdd(acc + ti * 128 + col, ch[0] * f);
-    }
-  }
-  if (tid == 0 && *abort_flag) {
-    // a wait gave up: let this CTA's own copies and MMAs finish (bounded) before it frees
-    // its tensor memory and exits; copies go out in tile order, so each stage's latest is
-    // one of the last nstage tiles issued, and the last commit covers every earlier MMA
-    mbar_wait_bounded(full_i, 0, err);
-    const int lp = *load_pending, mp = *mma_pending;
-    for (int t = lp; t >= 0 && t > lp - nstage; --t)
-      mbar_wait_bounded(&full_j[t % nstage], (uint32_t)((t / nstage) & 1), err);
-    if (mp >= 0) mbar_wait_bounded(&mma_done[mp % kSymBufs], (uint32_t)((mp / kSymBufs) & 1), err);
+    if (__all_sync(0xffffffffu, ok && *abort_flag == 0)) flush();
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 128 * kSymBufs);
+  tc_fence_after();
+  if (warp == kSymEpi) tmem_dealloc(tmem, 128 * kSymBufs);
 }
 
-static int tc_sym_stages(int) { return 2; }
-
-static size_t tc_sym_smem(int katoms) {
-  return 1024 + (size_t)(2 + 2 * tc_sym_stages(katoms)) * katoms * kAtomBytes + 256 * sizeof(float) +
-         (1 + 4 + 2 * kSymBufs) * sizeof(uint64_t) + 32;
+// Row-tile buffers and J stages: 2 + 4 (tiles of 16 KB), 2 + 3 (32 KB), 1 + 2 (64 KB).
+static void tc_sym_stages(size_t tile_bytes, int* nibuf, int* nstage) {
+  *nibuf = tile_bytes <= 32 * 1024 ? 2 : 1;
+  *nstage = tile_bytes <= 16 * 1024 ? kSymMaxStages : (tile_bytes <= 32 * 1024 ? 3 : 2);
 }
 
-
-// Work units of the symmetric tensor-core tiles: (row tile I, column tiles [J0, J1)) with
-// I <= J0, about 8 per SM (one CTA resident), so that each CTA's TMA/MMA pipeline runs over
-// tens of tiles; the longest units come first, for the block scheduler's tail.
-static cudaError_t tc_sym_units_ensure(Handle* h) {
-  const int T = (int)(h->ldn / kTile);
-  if (h->tc_sym_units && h->tc_sym_T == T) return cudaSuccess;
-  const int64_t pairs = (int64_t)T * (T + 1) / 2;
-  const int64_t target = (int64_t)8 * h->num_sms;
-  int C = (int)((pairs + target - 1) / target);
-  if (C < 1) C = 1;
-  std::vector<int4> u;
-  for (int I = 0; I < T; ++I)
-    for (int J0 = I; J0 < T; J0 += C) u.push_back(make_int4(I, J0, J0 + C < T ? J0 + C : T, 0));
-  std::stable_sort(u.begin(), u.end(), [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
-  dev_free(h, h->tc_sym_units);
-  h->tc_sym_units = (int4*)dev_alloc(h, u.size() * sizeof(int4));
-  if (!h->tc_sym_units) return cudaErrorMemoryAllocation;
-  h->tc_sym_nunits = (int)u.size();
-  h->tc_sym_T = T;
-  return cudaMemcpy(h->tc_sym_units, u.data(), u.size() * sizeof(int4), cudaMemcpyHostToDevice);
+static size_t tc_sym_smem(size_t tile_bytes) {
+  int ni, ns;
+  tc_sym_stages(tile_bytes, &ni, &ns);
+  return 1024 + (size_t)(ni + ns) * tile_bytes + 2 * 512 * sizeof(float) +
+         (4 + 2 * kSymMaxStages + 2 * kSymBufs) * sizeof(uint64_t) + 16;
 }
 
 // m = 1 RBF product on symmetric tensor-core tiles; nt = 3: FP32 class (fp16 parts when
@@ -804,8 +936,8 @@ static cudaError_t rbf_tc_sym_product(Handle* h, const double* V, double* U, int
                                       cudaStream_t st) {
   cudaError_t e = rbf_tc_prepare(h);
   if (e != cudaSuccess) return e;
-  if ((e = tc_sym_units_ensure(h)) != cudaSuccess) return e;
-  float *v32, *acc;
+  float* v32;
+  double* acc;
   if ((e = sym_buffers(h, &v32, &acc)) != cudaSuccess) return e;
   GramEpilogue none;
   const GramEpilogue& g = ep ? *ep : none;
@@ -814,20 +946,24 @@ static cudaError_t rbf_tc_sym_product(Handle* h, const double* V, double* U, int
   if (f16 && (e = rbf_f16_prepare(h)) != cudaSuccess) return e;
   const int katoms = f16 ? h->tc16_katoms : h->tc_Kp / 32;
   const int ksteps = f16 ? (int)((3 * h->p + 15) / 16) : (int)((h->p + 7) / 8);
-  const size_t smem = tc_sym_smem(katoms);
+  const size_t tile = (size_t)(!f16 && nt == 3 ? 2 : 1) * katoms * kAtomBytes;
+  const size_t smem = tc_sym_smem(tile);
+  int nibuf, nstage;
+  tc_sym_stages(tile, &nibuf, &nstage);
   auto kern = f16 ? gram_rbf_tc_sym_kernel<16, true>
                   : nt == 3 ? (h->tc_fold_rows ? gram_rbf_tc_sym_kernel<3, true> : gram_rbf_tc_sym_kernel<3, false>)
                             : (h->tc_fold_rows ? gram_rbf_tc_sym_kernel<1, true> : gram_rbf_tc_sym_kernel<1, false>);
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return e;
+  const int T = (int)(h->ldn / kTile);
+  const int grid = (int)std::min<int64_t>(h->num_sms, (int64_t)T * (T + 1) / 2);
   prof_mark(h, 0, true, st);
-  kern<<<h->tc_sym_nunits, kSymWarps * 32, smem, st>>>(f16 ? h->tm_tc_a16 : h->tm_tc_hi, f16 ? h->tm_tc_b16 : h->tm_tc_lo,
-                                                       h->nrm32, v32, h->tc_sym_units, acc, ksteps, katoms,
-                                                       tc_sym_stages(katoms), h->err_flag);
+  kern<<<grid, kSymThreads, smem, st>>>(f16 ? h->tm_tc_a16 : h->tm_tc_hi, f16 ? h->tm_tc_b16 : h->tm_tc_lo, h->nrm32,
+                                        v32, acc, T, ksteps, katoms, nibuf, nstage, h->err_flag);
   prof_mark(h, 0, false, st);
   h->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return sym_finish(h, acc, U, g, st);
+  return sym_finish(h, acc, true, U, g, st);
 }
 
 cudaError_t gram_rbf_tc(Handle* h, const double* V, double* U, int m, bool three_terms, const GramEpilogue* ep,

@@ -312,7 +312,7 @@ kqr_status kstore_setup(Handle* h) {
   if (mode == 2 && bytes > free_b / 2) return KQR_OK;   // automatic: only when it fits comfortably
   // automatic: once the stored tiles no longer fit in L2, the symmetric tcgen05 RBF tiles
   // (p <= 32, one 128-byte atom per row) form K faster than a stored K streams from HBM
-  // (0.48 against 0.74 ms at n = 50000)
+  // (0.31 against 0.74 ms at n = 50000)
   if (mode == 2 && h->kind == KQR_RBF && h->opt.rbf_tensor_cores && h->opt.symmetric_gram && h->p <= 32 &&
       bytes > kStoreL2Bytes)
     return KQR_OK;
@@ -385,18 +385,20 @@ void kstore_free(Handle* h) {
 
 cudaError_t gram_stored(Handle* h, const double* V, double* U, const GramEpilogue* ep, cudaStream_t st) {
   cudaError_t e;
-  float *v32, *acc;
-  if ((e = sym_buffers(h, &v32, &acc)) != cudaSuccess) return e;
+  float* v32;
+  double* sums;
+  if ((e = sym_buffers(h, &v32, &sums)) != cudaSuccess) return e;
+  float* acc = reinterpret_cast<float*>(sums);
   GramEpilogue none;
   const GramEpilogue& g = ep ? *ep : none;
-  if (!g.prepped && (e = sym_prep(h, V, v32, acc, const_cast<double*>(g.sum_p), st)) != cudaSuccess) return e;
+  if (!g.prepped && (e = sym_prep(h, V, v32, sums, const_cast<double*>(g.sum_p), st)) != cudaSuccess) return e;
   prof_mark(h, 2, true, st);
   kstore_gemv_kernel<<<h->kstore_grid, kKsThreads, kstore_smem(), st>>>(h->kstore, v32, acc, h->kstore_sched,
                                                                        (int)(h->ldn / kTile), h->err_flag);
   prof_mark(h, 2, false, st);
   h->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return sym_finish(h, acc, U, g, st);
+  return sym_finish(h, acc, false, U, g, st);
 }
 
 }  // namespace kqr

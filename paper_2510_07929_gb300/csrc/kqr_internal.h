@@ -64,11 +64,12 @@ cudaError_t gram_rbf_tc(Handle* h, const double* V, double* U, int m, bool three
 cudaError_t gram_rbf_tc_bf16(Handle* h, const double* V, double* U, int m, cudaStream_t st);
 // m = 1 product with each off-diagonal tile formed once (gram_f32_sym.cu).
 cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilogue* ep, cudaStream_t st);
-// FP32 copy of the vector and FP32 sums of the products that accumulate with atomics
-// (symmetric tiles, stored K): ldn floats each, and the kernel that fills them.
-cudaError_t sym_buffers(Handle* h, float** v32, float** acc);
-cudaError_t sym_prep(Handle* h, const double* V, float* v32, float* acc, double* sum_out, cudaStream_t st);
-cudaError_t sym_finish(Handle* h, const float* acc, double* U, const GramEpilogue& g, cudaStream_t st);
+// FP32 copy of the vector (ldn floats) and sums (ldn doubles, or floats in their first half) of the
+// products that accumulate with atomics (symmetric tiles, stored K), the kernel that fills and zeroes
+// them, and the one that reads the sums (f64: as doubles).
+cudaError_t sym_buffers(Handle* h, float** v32, double** acc);
+cudaError_t sym_prep(Handle* h, const double* V, float* v32, double* acc, double* sum_out, cudaStream_t st);
+cudaError_t sym_finish(Handle* h, const void* acc, bool f64, double* U, const GramEpilogue& g, cudaStream_t st);
 cudaError_t gram_high(Handle* h, const double* V, double* U, int m, cudaStream_t st);
 // Laplacian m = 1 FP64-class product with each off-diagonal tile formed once (gram_high_sym.cu).
 cudaError_t gram_high_sym(Handle* h, const double* V, double* U, cudaStream_t st);
@@ -157,8 +158,6 @@ struct Handle {
   // Symmetric Gram product: work-unit table (row tile, first and end column tile).
   int4* sym_units = nullptr;
   int sym_nunits = 0, sym_T = 0;
-  int4* tc_sym_units = nullptr;       // the same for the symmetric tensor-core tiles (fewer, longer units)
-  int tc_sym_nunits = 0, tc_sym_T = 0;
 
   // Gram-product scratch.
   float* part = nullptr;  size_t part_cap = 0;      // per-split partial sums (bytes)

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) cg_step_kernel(double* __restrict__ s, do
 // product wants (rows n .. ldn stay as sym_prep left them for v32).
 __global__ void __launch_bounds__(256) cg_dir_kernel(double* __restrict__ s, double* __restrict__ p,
                                                      const double* __restrict__ z, int64_t n, int64_t ldn,
-                                                     float* __restrict__ v32, float* __restrict__ acc,
+                                                     float* __restrict__ v32, double* __restrict__ acc,
                                                      double* __restrict__ part, unsigned int* __restrict__ counter) {
   if ((int)s[S_CGST] != CG_RUN) return;
   const double b = s[S_RZN] / s[S_RZ];
@@ -169,12 +169,12 @@ __global__ void __launch_bounds__(256) cg_dir_kernel(double* __restrict__ s, dou
     p[i] = pi;
     if (v32) {
       v32[i] = (float)pi;
-      acc[i] = 0.f;
+      acc[i] = 0.0;
     }
     sums[0] += pi * pi;
     sums[1] += pi;
   }
-  if (v32 && blockIdx.x == 0 && n + threadIdx.x < ldn) acc[n + threadIdx.x] = 0.f;   // ldn - n < 128
+  if (v32 && blockIdx.x == 0 && n + threadIdx.x < ldn) acc[n + threadIdx.x] = 0.0;   // ldn - n < 128
   if (!grid_sums(sums, part, counter, &tot)) return;
   if (threadIdx.x == 0) {
     s[S_PP] = tot;
@@ -192,7 +192,7 @@ static cudaError_t cg_step(Handle* h, double noise_coef, double* x, double* Kx, 
   return cudaGetLastError();
 }
 
-static cudaError_t cg_dir(Handle* h, double* p, const double* z, float* v32, float* acc, cudaStream_t st) {
+static cudaError_t cg_dir(Handle* h, double* p, const double* z, float* v32, double* acc, cudaStream_t st) {
   cg_dir_kernel<<<grid_for(h->n, 256, 304), 256, 0, st>>>(h->scal, p, z, h->n, h->ldn, v32, acc, h->red_part,
                                                           h->red_counter);
   h->launches++;
@@ -286,7 +286,8 @@ kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const
                                                                    : (lowprec ? std::ldexp(1.0, -40) : std::ldexp(1.0, -22)));
   // FP32 products that accumulate with atomics find their vector prepared: by sym_prep here, by the
   // direction kernel afterwards.
-  float *v32 = nullptr, *acc = nullptr;
+  float* v32 = nullptr;
+  double* acc = nullptr;
   if (!h->rdv && !(h->cg_high_on && !lowprec) && (h->opt.symmetric_gram || (h->kstore && !lowprec))) {
     CK(sym_buffers(h, &v32, &acc));
     CK(sym_prep(h, p, v32, acc, nullptr, st));
