@@ -966,9 +966,408 @@ static cudaError_t rbf_tc_sym_product(Handle* h, const double* V, double* U, int
   return sym_finish(h, acc, true, U, g, st);
 }
 
+// ---- several right-hand sides, FP32 class (p <= 32) -------------------------------------
+// u_I += K_IJ V_J for M = 2, 4 or 8 vectors, all n^2 entries, row sums only (deterministic).  A
+// step is 256 rows (two row tiles, one after the other in tensor memory) x 128 columns.
+//
+// What bounds it: the FFMAs with the vectors, 4 issue slots per entry at M = 8 as packed f32x2
+// over column pairs (the even and odd columns' sums are separate chains), beside 1.5 for the
+// exponent and the ex2, and the broadcast loads of V, which serve two rows of a thread each.
+// n = 19999, p = 8, M = 8: 257 us; the plain kernel (one row per thread, unpacked, a CTA-wide
+// barrier per tile and one thread of the epilogue computing descriptors for 3 ksteps MMAs) 602 us.
+// Loading 4-column chunks ahead of their use gave nothing (260 us).
+// One persistent CTA per SM walks an equal share of the steps (row pairs in order, all columns of
+// a pair); copies and MMAs are issued by a warp each; 16 epilogue warps: warp w has TMEM lanes
+// 32 (w mod 4) .. + 31 and columns 32 (w / 4) .. + 31.  Sums of a step's 32 columns start at zero
+// and are added to per-thread totals in shared memory, which keeps FP32 chains short.  A CTA's
+// sums for a row pair go to its own partial (slot = CTA minus the pair's first CTA); a second
+// kernel adds the partials in FP64.
+constexpr int kMtEpi = 16;
+constexpr int kMtThreads = (kMtEpi + 2) * 32;
+constexpr int kMtStages = 3;
+
+__host__ __device__ __forceinline__ int mt_cta_of(int64_t step, int64_t total, int grid) {
+  return (int)(((step + 1) * grid - 1) / total);   // the CTA whose share [total b / grid, ...) holds the step
+}
+
+template <int M>
+__global__ void __launch_bounds__(kMtThreads, 1)
+    gram_rbf_tc_multi_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
+                             const float* __restrict__ nrm, const float* __restrict__ vp, float* __restrict__ part,
+                             int ksteps, int64_t ldn, int T, int fold_rows, int* __restrict__ err) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                         ~static_cast<uintptr_t>(1023));
+  constexpr uint32_t kTile16 = kAtomBytes / 16u;
+  constexpr uint32_t kStage = 2 * kAtomBytes;              // hi, lo
+  constexpr uint32_t kVBytesM = 128u * M * 4u;
+  unsigned char* xj = base + 4 * kAtomBytes;               // row tiles: hi 0, lo 0, hi 1, lo 1
+  unsigned char* cst = xj + kMtStages * kStage;            // [stage]: 128 norms, 128 x M of V in column pairs
+  constexpr uint32_t kCst = 512u + kVBytesM;
+  float4* tot = reinterpret_cast<float4*>(cst + kMtStages * kCst);   // [2 M / 4][512]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tot + (2 * M / 4) * 512);
+  uint64_t* full_i = bars;
+  uint64_t* i_free = bars + 1;
+  uint64_t* full_j = bars + 2;                  // [kMtStages]
+  uint64_t* stage_free = full_j + kMtStages;    // [kMtStages] MMAs done and constants read
+  uint64_t* mma_done = stage_free + kMtStages;  // [2]
+  uint64_t* tmem_free = mma_done + 2;           // [2]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_free + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const int pairs = (T + 1) / 2;
+  const int64_t total = (int64_t)pairs * T;
+  const int64_t t0 = total * blockIdx.x / gridDim.x;
+  const int nt = (int)(total * (blockIdx.x + 1) / gridDim.x - t0);
+
+  if (warp == kMtEpi) {
+    tmem_alloc(tmem_slot, 512);
+    tmem_relinquish();
+  }
+  if (tid == 0) {
+    mbar_init(full_i, 1);
+    mbar_init(i_free, 1);
+    for (int s = 0; s < kMtStages; ++s) {
+      mbar_init(&full_j[s], 1);
+      mbar_init(&stage_free[s], 1 + kMtEpi);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&mma_done[b], 1);
+      mbar_init(&tmem_free[b], kMtEpi);
+    }
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  int P = (int)(t0 / T), J = (int)(t0 % T);   // row pair and column tile of the first step
+
+  if (warp == kMtEpi) {
+    // ---- copies (converged warp, one elected lane)
+    if (nt > 0) {
+      const bool elected = elect_one();
+      int s = 0, q = 0, ki = 0;
+      uint32_t ph = 1;
+      bool ok = true;
+      for (; q < nt; ++q) {
+        if (q == 0 || J == 0) {
+          if (ki > 0) ok = __all_sync(0xffffffffu, mbar_wait_bounded(i_free, (uint32_t)((ki - 1) & 1), err));
+          if (!ok) break;
+          if (elected) {
+            mbar_arrive_expect_tx(full_i, 4 * kAtomBytes);
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {   // rows beyond ldn read as zero
+              tma_load_2d(base + hh * kStage, &tm_hi, 0, (2 * P + hh) * 128, full_i);
+              tma_load_2d(base + hh * kStage + kAtomBytes, &tm_lo, 0, (2 * P + hh) * 128, full_i);
+            }
+          }
+          __syncwarp();
+          ++ki;
+        }
+        ok = __all_sync(0xffffffffu, *abort_flag == 0 && mbar_wait_bounded(&stage_free[s], ph, err));
+        if (!ok) break;
+        if (elected) {
+          mbar_arrive_expect_tx(&full_j[s], kStage + kCst);
+          tma_load_2d(xj + s * kStage, &tm_hi, 0, J * 128, &full_j[s]);
+          tma_load_2d(xj + s * kStage + kAtomBytes, &tm_lo, 0, J * 128, &full_j[s]);
+          bulk_copy(cst + s * kCst, nrm + J * 128, 512u, &full_j[s]);
+          bulk_copy(cst + s * kCst + 512, vp + (size_t)J * 128 * M, kVBytesM, &full_j[s]);
+        }
+        __syncwarp();
+        if (++s == kMtStages) {
+          s = 0;
+          ph ^= 1;
+        }
+        if (++J == T) {
+          J = 0;
+          ++P;
+        }
+      }
+      if (!ok) *abort_flag = 1;
+      if (ki > 0) mbar_wait_bounded(full_i, (uint32_t)((ki - 1) & 1), err);
+      for (int t = q > kMtStages ? q - kMtStages : 0; t < q; ++t)
+        mbar_wait_bounded(&full_j[t % kMtStages], (uint32_t)((t / kMtStages) & 1), err);
+    }
+  } else if (warp == kMtEpi + 1) {
+    // ---- MMAs (converged warp, one elected lane, as in the symmetric kernel)
+    if (nt > 0) {
+      const bool elected = elect_one();
+      // FP32 accumulate, TF32 A and B, K-major, N = 128, M = 128
+      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+      const uint64_t desc_i = umma_desc_sw128(base), desc_j = umma_desc_sw128(xj);
+      const uint32_t dhi = (uint32_t)(desc_i >> 32);
+      auto dsc = [&](uint32_t lo) { return ((uint64_t)dhi << 32) | lo; };
+      int s = 0, b = 0, q = 0, ki = 0;
+      uint32_t ph = 0, fph = 1;
+      bool ok = true;
+      for (; q < nt; ++q) {
+        if (q == 0 || J == 0) {
+          ok = mbar_wait_bounded(full_i, (uint32_t)(ki & 1), err);
+          ++ki;
+        }
+        ok = ok && mbar_wait_bounded(&tmem_free[b], fph, err) && mbar_wait_bounded(&full_j[s], ph, err);
+        if (!__all_sync(0xffffffffu, ok && *abort_flag == 0)) break;
+        tc_fence_after();
+        const uint32_t bj = (uint32_t)desc_j + (uint32_t)s * (2 * kTile16);
+        if (elected) {
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh) {
+            const uint32_t d = tmem + (uint32_t)(b * 256 + hh * 128);
+            const uint32_t ai = (uint32_t)desc_i + (uint32_t)hh * (2 * kTile16);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (k < ksteps) {
+                umma_tf32(d, dsc(ai + k * 2u), dsc(bj + k * 2u), idesc, k > 0 ? 1u : 0u);
+                umma_tf32(d, dsc(ai + k * 2u), dsc(bj + kTile16 + k * 2u), idesc, 1u);
+                umma_tf32(d, dsc(ai + kTile16 + k * 2u), dsc(bj + k * 2u), idesc, 1u);
+              }
+          }
+          umma_commit(&stage_free[s]);
+          if (J + 1 == T && q + 1 < nt) umma_commit(i_free);
+          umma_commit(&mma_done[b]);
+        }
+        __syncwarp();
+        if (++J == T) {
+          J = 0;
+          ++P;
+        }
+        b ^= 1;
+        if (b == 0) fph ^= 1;
+        if (++s == kMtStages) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      if (q < nt) *abort_flag = 1;
+      if (q > 0) mbar_wait_bounded(&mma_done[(q - 1) & 1], (uint32_t)(((q - 1) >> 1) & 1), err);
+    }
+  } else if (nt > 0) {
+    // ---- epilogue
+    const int lq = warp & 3, cg = warp >> 2;
+    const uint32_t lane_off = (uint32_t)(lq * 32) << 16;
+    const uint64_t two = pack2(2.f, 2.f);
+    const int lrow = lq * 32 + lane;
+    float ni[2] = {0.f, 0.f};       // row norms, inside the exponent unless the row factors fold
+    auto row_norms = [&](int pair) {
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        const int64_t row = (int64_t)pair * 256 + hh * 128 + lrow;
+        ni[hh] = !fold_rows && row < ldn ? __ldg(nrm + row) : 0.f;
+      }
+    };
+    auto zero_totals = [&]() {
+#pragma unroll
+      for (int e = 0; e < 2 * M / 4; ++e) tot[e * 512 + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    // the totals of the four column groups, added in a fixed order, to this CTA's partial of the pair
+    auto flush = [&](int pair) {
+      const int slot = blockIdx.x - mt_cta_of((int64_t)pair * T, total, gridDim.x);
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+      for (int e = tid; e < 256 * M; e += kMtEpi * 32) {
+        const int row = e / M, c = e % M;
+        const int idx = (row >> 7) * M + c, t = ((row >> 5) & 3) * 32 + (row & 31);
+        float v = 0.f;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) v += reinterpret_cast<const float*>(tot + (idx >> 2) * 512 + g * 128 + t)[idx & 3];
+        const int64_t gr = (int64_t)pair * 256 + row;
+        if (gr < ldn) {
+          if (fold_rows) v *= ex2_approx(-__ldg(nrm + gr));
+          part[((size_t)slot * ldn + gr) * M + c] = v;
+        }
+      }
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+    };
+    row_norms(P);
+    zero_totals();
+    bool ok = true;
+    int s = 0, b = 0;
+    uint32_t ph = 0, mph = 0;
+    for (int q = 0; q < nt; ++q) {
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full_j[s], ph, err) && mbar_wait_bounded(&mma_done[b], mph, err))) {
+        ok = false;
+        *abort_flag = 1;
+      }
+      if (ok) {
+        tc_fence_after();
+        const float* nj = reinterpret_cast<const float*>(cst + s * kCst) + cg * 32;
+        const float* vj = reinterpret_cast<const float*>(cst + s * kCst + 512) + cg * 32 * M;
+        uint64_t acc[2][M];   // even and odd columns' sums of this step
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh)
+#pragma unroll
+          for (int c = 0; c < M; ++c) acc[hh][c] = 0ull;
+#pragma unroll 1
+        for (int ch = 0; ch < 4; ++ch) {
+          uint32_t g[2][8];
+          tmem_ld8_nowait(tmem + (uint32_t)(b * 256 + cg * 32 + ch * 8) + lane_off, g[0]);
+          tmem_ld8_nowait(tmem + (uint32_t)(b * 256 + 128 + cg * 32 + ch * 8) + lane_off, g[1]);
+          tmem_wait_ld();
+          if (ch == 3) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tmem_free[b]);
+          }
+#pragma unroll
+          for (int c2 = 0; c2 < 4; ++c2) {
+            const int col = ch * 8 + 2 * c2;
+            const float2 n2 = *reinterpret_cast<const float2*>(nj + col);
+            uint64_t e[2];
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+              float e0, e1;
+              unpack2(fma2(pack2(__uint_as_float(g[hh][2 * c2]), __uint_as_float(g[hh][2 * c2 + 1])), two,
+                           pack2(-(n2.x + ni[hh]), -(n2.y + ni[hh]))),
+                      e0, e1);
+              e[hh] = pack2(ex2_approx(e0), ex2_approx(e1));
+            }
+#pragma unroll
+            for (int c = 0; c < M; c += 2) {
+              const float4 v = *reinterpret_cast<const float4*>(vj + col * M + 2 * c);
+#pragma unroll
+              for (int hh = 0; hh < 2; ++hh) {
+                acc[hh][c] = fma2(e[hh], pack2(v.x, v.y), acc[hh][c]);
+                acc[hh][c + 1] = fma2(e[hh], pack2(v.z, v.w), acc[hh][c + 1]);
+              }
+            }
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&stage_free[s]);
+        float sums[2 * M];
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh)
+#pragma unroll
+          for (int c = 0; c < M; ++c) {
+            float a0, a1;
+            unpack2(acc[hh][c], a0, a1);
+            sums[hh * M + c] = a0 + a1;
+          }
+#pragma unroll
+        for (int e = 0; e < 2 * M / 4; ++e) {
+          float4 t = tot[e * 512 + tid];
+          t.x += sums[4 * e];
+          t.y += sums[4 * e + 1];
+          t.z += sums[4 * e + 2];
+          t.w += sums[4 * e + 3];
+          tot[e * 512 + tid] = t;
+        }
+        b ^= 1;
+        if (b == 0) mph ^= 1;
+        if (++s == kMtStages) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      // every warp comes here for every step, also after a timeout: the flush has barriers
+      if (++J == T || q + 1 == nt) {
+        flush(P);
+        if (J == T) {
+          J = 0;
+          ++P;
+        }
+        if (q + 1 < nt) {
+          row_norms(P);
+          zero_totals();
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == kMtEpi) tmem_dealloc(tmem, 512);
+}
+
+// V (n x m) -> FP32 in column-pair order of the rows: vp[(i / 2) 2 M + 2 c + (i mod 2)], zero padded.
+__global__ void mt_prep_kernel(const double* __restrict__ V, float* __restrict__ vp, int64_t n, int64_t ldn, int m,
+                               int M) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ldn * M; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = e / (2 * M) * 2 + (e & 1);
+    const int c = (int)(e % (2 * M)) >> 1;
+    vp[e] = (i < n && c < m) ? (float)V[i * m + c] : 0.f;
+  }
+}
+
+// out = sum of the pair's partials, in FP64.
+__global__ void mt_reduce_kernel(const float* __restrict__ part, int64_t ldn, int T, int grid, int M, int m, int64_t n,
+                                 double* __restrict__ out) {
+  const int64_t total = (int64_t)((T + 1) / 2) * T;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * m; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = e / m, pair = row >> 8;
+    const int c = (int)(e % m);
+    const int slots = mt_cta_of(pair * T + T - 1, total, grid) - mt_cta_of(pair * T, total, grid) + 1;
+    double s = 0.0;
+    for (int q = 0; q < slots; ++q) s += (double)part[((size_t)q * ldn + row) * M + c];
+    out[e] = s;
+  }
+}
+
+template <int M>
+static cudaError_t launch_multi(Handle* h, int grid, int ksteps, cudaStream_t st) {
+  const size_t smem = 1024 + 4 * kAtomBytes + kMtStages * (2 * kAtomBytes + 512 + 128 * M * 4) +
+                      (size_t)(2 * M / 4) * 512 * 16 + (2 + 2 * kMtStages + 4) * 8 + 16;
+  auto kern = gram_rbf_tc_multi_kernel<M>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  prof_mark(h, 0, true, st);
+  kern<<<grid, kMtThreads, smem, st>>>(h->tm_tc_hi, h->tm_tc_lo, h->nrm32, h->v32, h->part, ksteps, h->ldn,
+                                       (int)(h->ldn / kTile), h->tc_fold_rows, h->err_flag);
+  prof_mark(h, 0, false, st);
+  h->launches++;
+  return cudaGetLastError();
+}
+
+// From this many row tiles on: 256 x 128 steps leave most SMs without work below (n = 1000, M = 8:
+// 24.9 us a call, 23.2 with the plain kernel; n = 2000: 25.6 against 31.4).
+constexpr int kMtMinTiles = 12;
+
+// FP32-class product with 2 to 8 right-hand sides, p <= 32 (one 128-byte atom per row and part).
+static cudaError_t rbf_tc_multi_product(Handle* h, const double* V, double* U, int m, cudaStream_t st) {
+  cudaError_t e = rbf_tc_prepare(h);
+  if (e != cudaSuccess) return e;
+  const int M = m <= 2 ? 2 : (m <= 4 ? 4 : 8);
+  const int T = (int)(h->ldn / kTile);
+  const int64_t total = (int64_t)((T + 1) / 2) * T;
+  const int grid = (int)std::min<int64_t>(h->num_sms, total);
+  // CTAs that share a row pair: at most its T steps over the shortest share, plus the two cut ones
+  const int64_t slots = std::min<int64_t>(grid, T / (total / grid) + 2);
+  const size_t vb = (size_t)h->ldn * M * sizeof(float);
+  if (h->v32_cap < vb) {
+    dev_free(h, h->v32);
+    h->v32 = (float*)dev_alloc(h, vb);
+    h->v32_cap = h->v32 ? vb : 0;
+    if (!h->v32) return cudaErrorMemoryAllocation;
+  }
+  const size_t pb = (size_t)slots * h->ldn * M * sizeof(float);
+  if (h->part_cap < pb) {
+    dev_free(h, h->part);
+    h->part = (float*)dev_alloc(h, pb);
+    h->part_cap = h->part ? pb : 0;
+    if (!h->part) return cudaErrorMemoryAllocation;
+  }
+  mt_prep_kernel<<<grid_for(h->ldn * M), 256, 0, st>>>(V, h->v32, h->n, h->ldn, m, M);
+  h->launches++;
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const int ksteps = (int)((h->p + 7) / 8);
+  switch (M) {
+    case 2: e = launch_multi<2>(h, grid, ksteps, st); break;
+    case 4: e = launch_multi<4>(h, grid, ksteps, st); break;
+    default: e = launch_multi<8>(h, grid, ksteps, st); break;
+  }
+  if (e != cudaSuccess) return e;
+  mt_reduce_kernel<<<grid_for(h->n * m), 256, 0, st>>>(h->part, h->ldn, T, grid, M, m, h->n, U);
+  h->launches++;
+  return cudaGetLastError();
+}
+
 cudaError_t gram_rbf_tc(Handle* h, const double* V, double* U, int m, bool three_terms, const GramEpilogue* ep,
                         cudaStream_t st) {
   if (m == 1 && h->opt.symmetric_gram) return rbf_tc_sym_product(h, V, U, three_terms ? 3 : 1, ep, st);
+  if (m >= 2 && three_terms && !ep && h->p <= 32 && h->ldn >= kMtMinTiles * kTile)
+    return rbf_tc_multi_product(h, V, U, m, st);
   return rbf_tc_product(h, V, U, m, three_terms ? 3 : 1, ep, st);
 }
 

@@ -1,7 +1,8 @@
-"""The persistent symmetric RBF tiles of gram_rbf_tc.cu: shares of the tile order that start, end or change
-row tile anywhere, for one to a few hundred row tiles, in each operand form (fp16 parts, TF32 parts with
-one and two atoms per row, one TF32 term), against the FP64 oracle.  Bounds: those of the existing tests
-of the same products (FP32 class 1e-5 of max |K v|; TF32: 2^-9 of the cross terms, entrywise below)."""
+"""The persistent RBF tiles of gram_rbf_tc.cu (symmetric for one vector, row sums for several): shares of
+the tile order that start, end or change row tile anywhere, for one to a few hundred row tiles, in each
+operand form (fp16 parts, TF32 parts with one and two atoms per row, one TF32 term), against the FP64
+oracle.  Bounds: those of the existing tests of the same products (FP32 class 1e-5 of max |K v|; TF32:
+2^-9 of the cross terms, entrywise below)."""
 import numpy as np
 import pytest
 
@@ -48,3 +49,25 @@ def test_symmetric_tiles_cover_every_pair(K_, n, p, spread):
     # one TF32 term: the exponent 2 xs_i . xs_j errs by at most 2 * 2^-11 * 2 |xs_i||xs_j|
     bound = (K * np.expm1(np.log(2.0) * 2.0 ** -9 * np.outer(nr, nr) * 1.1 + 1e-6)) @ np.abs(v) + 1e-5 * np.max(np.abs(ref)) + far
     assert np.all(np.abs(t - ref) <= bound)
+
+
+@pytest.mark.parametrize("n", [2, 257, 1000, 1409, 1500, 1536, 1537, 1700, 2600])
+@pytest.mark.parametrize("p,spread", [(1, 1.0), (8, 1.0), (9, 1.0), (32, 1.0), (20, 9.0)])
+def test_multi_vector_tiles_cover_every_pair(K_, n, p, spread):
+    """Two to eight vectors: row pairs of 256 rows shared out over the CTAs anywhere, partial sums per CTA;
+    bound as above, and repeated products are bit-identical."""
+    rng = np.random.default_rng(n + p)
+    X = rng.standard_normal((n, p))
+    X[0] *= spread
+    gamma = 1.0 / p
+    K = O.gram(X, X, "rbf", gamma)
+    Xc = (X - X.mean(0)) * np.sqrt(gamma / np.log(2.0))
+    nr = np.linalg.norm(Xc, axis=1)
+    with K_.Problem(X, np.zeros(n), "rbf", gamma, gram_store=0, rank0=2) as prob:
+        for m in (2, 3, 5, 8):
+            V = rng.standard_normal((n, m))
+            U = prob.kmatvec(V, K_.PREC_FP32)
+            ref = K @ V
+            far = (K * (np.add.outer(nr ** 2, nr ** 2) * (np.log(2.0) * 2.0 ** -19))) @ np.abs(V)
+            assert np.all(np.abs(U - ref) <= 1e-5 * np.max(np.abs(ref)) + far)
+            np.testing.assert_array_equal(U, prob.kmatvec(V, K_.PREC_FP32))
