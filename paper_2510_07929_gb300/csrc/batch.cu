@@ -9,19 +9,18 @@
 //   S = XS_I XS_J^T        (128 x 64 tile, K = p, from TMA tiles, 128-byte swizzle)
 //   P = exp2(2 S - n_i - n_j) = K_IJ   (epilogue warps: TMEM -> registers -> TMEM, or
 //                                        shared memory with KQR_BATCH_P_IN_SMEM)
-//   U_I += P V_J           (128 x 64 accumulator, K = 64 Gram columns)
+//   U_I += P V_J           (128 x 64 accumulator, K = the step's Gram columns)
 // with XS = sqrt(gamma log2 e)(x - mean_b) rounded to TF32 and n = |XS|^2 of
 // the rounded rows (so the tile is the RBF kernel at those rows, and stays
 // positive semidefinite), P rounded to TF32 (nearest) and V rounded to TF32.
 //
-// Work item = (problem, 128-row tile); its 64-column steps stream X_J and V_J
-// through TMA rings of 4 and 5 stages.  Items are sorted by length and dealt
-// round-robin to one persistent CTA per SM.  Warp roles (320 threads): warp 0
-// issues TMA copies, warp 1 owns tensor memory and issues the MMAs, warps 2-9
-// are the epilogue in two groups of four that take alternate steps (thread =
-// TMEM lane = row), so two tiles are exponentiated at once.  Tensor memory: four S buffers and two U accumulators (64 columns
-// each); the first MMAs run two steps ahead of the second ones, so the epilogue
-// finds its next S tile computed, and the read-out of item i overlaps item i + 1.
+// Work item = (problem, 128-row tile); items are sorted by length and dealt round-robin to one
+// persistent CTA per SM.  Two kernels: batch_kv_tmem_kernel keeps the Gram tile in tensor memory
+// (the default, described there); batch_kv_kernel stages it through shared memory
+// (KQR_BATCH_P_IN_SMEM): 64-column steps, X_J and V_J through TMA rings of 4 and 5 stages; warp 0
+// issues the copies, warp 1 owns tensor memory and issues the MMAs, warps 2-9 are the epilogue in
+// two groups of four that take alternate steps (thread = TMEM lane = row); tensor memory holds four
+// S buffers and two U accumulators (64 columns each), and the first MMAs run two steps ahead.
 // Every wait is bounded; a timeout sets the error flag and an abort flag that
 // ends every role's loop, after which the CTA drains its copies and MMAs and
 // frees its tensor memory.
@@ -61,7 +60,6 @@ constexpr uint32_t kOffBar = kOffP + 2 * kPBytes;
 constexpr int kNumBars = 2 + 2 + 2 * kXStages + 2 * kVStages + 2 * kSBufs + 2 + 2 + 2 + 2 + 1;
 constexpr size_t kBatchSmem = 1024 + kOffBar + kNumBars * 8 + 16;
 constexpr uint32_t kUCol = 64 * kSBufs;     // first TMEM column of the U accumulators
-constexpr uint32_t kPCol = kUCol + 128;     // first TMEM column of the P tiles (P kept in tensor memory)
 
 __device__ __forceinline__ void tmem_alloc_b(uint32_t* dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols)
@@ -196,7 +194,6 @@ struct MmaStep {
 
 // items[i] = {row0 (padded row of the tile), col0 (padded first row of its problem),
 //             nt (64-column steps), nvalid (rows < n_b in the tile)}; out0[i] = output row of row0.
-template <bool PT>
 __global__ void __launch_bounds__(kBatchThreads, 1)
     batch_kv_kernel(const __grid_constant__ CUtensorMap tm_xi, const __grid_constant__ CUtensorMap tm_xj,
                     const __grid_constant__ CUtensorMap tm_v, const float* __restrict__ nrm,
@@ -316,12 +313,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
 #pragma unroll
         for (int k = 0; k < kBN / 8; ++k) {
           const uint32_t ka = (uint32_t)(k >> 2), kb = (uint32_t)(k & 3) * 32u;
-          if (PT)
-            mma_tf32_ta(d, tmem + kPCol + (uint32_t)(pb * 64 + k * 8), desc_sw128(va + ka * kVAtom + kb), idesc,
-                        (ps.first && k == 0) ? 0u : 1u);
-          else
-            mma_tf32(d, desc_sw128(pa + ka * kPAtom + kb), desc_sw128(va + ka * kVAtom + kb), idesc,
-                     (ps.first && k == 0) ? 0u : 1u);
+          mma_tf32(d, desc_sw128(pa + ka * kPAtom + kb), desc_sw128(va + ka * kVAtom + kb), idesc,
+                   (ps.first && k == 0) ? 0u : 1u);
         }
         mma_commit(&p_empty[pb]);
         mma_commit(&vl_empty[ps.stage]);
@@ -410,21 +403,15 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
             e[4 * c4 + 2] = tf32_rna(ex2_approx(fmaf(2.f, __uint_as_float(g[2]), -(ni + nn.z))));
             e[4 * c4 + 3] = tf32_rna(ex2_approx(fmaf(2.f, __uint_as_float(g[3]), -(ni + nn.w))));
           }
-          if (PT) {
-            // P tile in tensor memory, lane = row, columns [32 ch, 32 ch + 32)
-            tmem_st32_nowait(tmem + kPCol + (uint32_t)(pb * 64 + ch * 32) + lane_off, e);
-          } else {
-            // columns [32 ch, 32 ch + 32) are swizzle atom ch of the P tile in shared memory
-            unsigned char* prow = base + kOffP + pb * kPBytes + ch * kPAtom + r * 128;
+          // columns [32 ch, 32 ch + 32) are swizzle atom ch of the P tile in shared memory
+          unsigned char* prow = base + kOffP + pb * kPBytes + ch * kPAtom + r * 128;
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-              *reinterpret_cast<uint4*>(prow + ((c ^ (r & 7)) * 16)) =
-                  make_uint4(e[4 * c], e[4 * c + 1], e[4 * c + 2], e[4 * c + 3]);
-          }
+          for (int c = 0; c < 8; ++c)
+            *reinterpret_cast<uint4*>(prow + ((c ^ (r & 7)) * 16)) =
+                make_uint4(e[4 * c], e[4 * c + 1], e[4 * c + 2], e[4 * c + 3]);
         }
-        if (PT) tmem_wait_st();
         fence_before();
-        if (!PT) fence_async_smem();
+        fence_async_smem();
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&s_empty[sb]);
@@ -457,6 +444,358 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
   __syncthreads();
   fence_after();
   if (warp == 1) tmem_dealloc_b(tmem, 512);
+}
+
+// ---- Gram tile kept in tensor memory (the default) --------------------------------------
+// Steps of 128 columns; the Gram tile P overwrites its S tile in tensor memory (same lane, same
+// columns), so three 128-column buffers and two U accumulators of 64 columns fill the 512.
+//
+// What bounds it: one ex2 and four issue slots per entry (the exponent's two operations packed
+// f32x2, the TF32 rounding as an integer add and mask: cvt.rna.tf32 shares the ex2 unit at 32 per
+// clock) are 512 cycles a step, the second contraction's 16 MMAs another 512 on the tensor pipe.
+// The previous form (64-column steps, two groups of four epilogue warps on alternate steps, one
+// warp per scheduler each) spent 2800 cycles on half as many entries waiting on hand-offs: 10.3 ms
+// for the 64-problem workload at m = 64, now 4.2.  Here 16 epilogue warps share a step (32 columns
+// each), the first MMAs run two steps ahead, stage indexes and descriptors are running values (6.5 ms
+// when a branch of one lane issued the MMAs), and an item's result is read out one step into the next
+// item, when its last MMAs are done.  A step now takes 2050 cycles, still the chain S - P - second
+// MMAs - free buffer over three buffers: without the epilogue's work it takes 1900, without 15 of the
+// 16 second MMAs 1650, without both 1430; half the copies (two row tiles per X_J and V_J) and
+// accumulators read half a step ahead change nothing.
+constexpr int kTN = 128;                        // Gram columns per step
+constexpr int kTBufs = 3;                       // S/P buffers and X_J, V_J stages
+constexpr int kTVStages = kTBufs;               // V_J stages
+constexpr int kTNStages = 6;                    // column norms of a step (copied with X_J, ahead of V_J)
+constexpr int kTEpi = 16;
+constexpr int kTThreads = (kTEpi + 2) * 32;
+constexpr uint32_t kTXBytes = kTN * 128;        // 128 rows x 128 B
+constexpr uint32_t kTVAtom = kBR * 128;         // 64 right-hand sides x 32 columns
+constexpr uint32_t kTVBytes = 4 * kTVAtom;
+constexpr uint32_t kTNrm = kTN * 4;
+constexpr uint32_t kTOffXJ = 2 * kXIBytes;
+constexpr uint32_t kTOffV = kTOffXJ + kTBufs * kTXBytes;
+constexpr uint32_t kTOffN = kTOffV + kTVStages * kTVBytes;
+constexpr uint32_t kTOffBar = kTOffN + kTNStages * kTNrm;
+constexpr int kTNumBars = 4 + 4 * kTBufs + kTVStages + 2 * kTNStages + 4 + 1;
+constexpr size_t kTSmem = 1024 + kTOffBar + kTNumBars * 8 + 16;
+constexpr uint32_t kTUCol = kTBufs * 128;
+
+__device__ __forceinline__ uint64_t bpack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void bunpack2(uint64_t r, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+// exp2 rounded to TF32 (nearest, ties away, as cvt.rna.tf32 on positive numbers)
+__device__ __forceinline__ uint32_t exp2_tf32(float x) {
+  return (__float_as_uint(ex2_approx(x)) + 0x1000u) & 0xffffe000u;
+}
+
+// items[i] = {row0 (padded row of the tile), col0 (padded first row of its problem), nt (steps of
+// kTN columns), nvalid (rows < n_b in the tile)}; out0[i] = output row of row0.  ksteps: 8-feature
+// MMA steps of the first contraction.
+__global__ void __launch_bounds__(kTThreads, 1)
+    batch_kv_tmem_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_v,
+                         const float* __restrict__ nrm, const int4* __restrict__ items, const int* __restrict__ out0,
+                         int n_items, int ksteps, double* __restrict__ out, int m, int* __restrict__ err) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                         ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(base + kTOffBar);
+  uint64_t* xi_full = bars;                     // [2] row tile landed
+  uint64_t* xi_empty = bars + 2;                // [2] its last MMA is done
+  uint64_t* x_full = bars + 4;                  // [kTBufs]
+  uint64_t* v_full = x_full + kTBufs;          // [kTVStages] V_J landed
+  uint64_t* n_full = v_full + kTVStages;       // [kTNStages] column norms landed
+  uint64_t* n_empty = n_full + kTNStages;       // all epilogue warps are done with them
+  uint64_t* s_full = n_empty + kTNStages;       // first MMAs done
+  uint64_t* p_full = s_full + kTBufs;           // all epilogue warps have written P
+  uint64_t* b_free = p_full + kTBufs;           // second MMAs done: the buffer can take another S
+  uint64_t* u_full = b_free + kTBufs;           // [2]
+  uint64_t* u_empty = u_full + 2;               // [2]
+  uint64_t* drain = u_empty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kTNumBars);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  if (warp == kTEpi + 1) {
+    tmem_alloc_b(tmem_slot, 512);
+    tmem_relinquish_b();
+  }
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&xi_full[i], 1);
+      mbar_init(&xi_empty[i], 1);
+      mbar_init(&u_full[i], 1);
+      mbar_init(&u_empty[i], kTEpi);
+    }
+    for (int i = 0; i < kTBufs; ++i) {
+      mbar_init(&x_full[i], 1);
+      mbar_init(&s_full[i], 1);
+      mbar_init(&p_full[i], kTEpi);
+      mbar_init(&b_free[i], 1);
+    }
+    for (int i = 0; i < kTVStages; ++i) {
+      mbar_init(&v_full[i], 1);
+    }
+    for (int i = 0; i < kTNStages; ++i) {
+      mbar_init(&n_full[i], 1);
+      mbar_init(&n_empty[i], kTEpi);
+    }
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == kTEpi) {
+    // ---- copies ----
+    if (lane == 0) {
+      int s = 0, sv = 0, sn = 0, seq = 0, nx = 0, nv = 0, nn = 0;   // stages; copies issued of each kind
+      uint32_t ph = 1, vph = 1, nph = 1;   // parities of the empty barriers: a buffer's first use does not wait
+      bool ok = true;
+      for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
+        const int4 I = items[it];
+        const int xb = seq & 1;
+        ok = bwait(&xi_empty[xb], ((seq >> 1) & 1) ^ 1, abort_flag, err);
+        if (!ok) break;
+        mbar_arrive_expect_tx(&xi_full[xb], kXIBytes);
+        tma_load_2d(base + xb * kXIBytes, &tm_x, 0, I.x, &xi_full[xb]);
+        ++seq;
+        int c0 = I.y;
+        for (int j = 0; j < I.z; ++j, c0 += kTN) {
+          ok = bwait(&s_full[s], ph, abort_flag, err);   // the first MMAs of the stage's last step are done
+          if (!ok) break;
+          mbar_arrive_expect_tx(&x_full[s], kTXBytes);
+          tma_load_2d(base + kTOffXJ + s * kTXBytes, &tm_x, 0, c0, &x_full[s]);
+          ++nx;
+          if (++s == kTBufs) {
+            s = 0;
+            ph ^= 1;
+          }
+          ok = bwait(&n_empty[sn], nph, abort_flag, err);
+          if (!ok) break;
+          mbar_arrive_expect_tx(&n_full[sn], kTNrm);
+          bulk_load(base + kTOffN + sn * kTNrm, nrm + c0, kTNrm, &n_full[sn]);
+          ++nn;
+          if (++sn == kTNStages) {
+            sn = 0;
+            nph ^= 1;
+          }
+          ok = bwait(&b_free[sv], vph, abort_flag, err);   // and here the second ones
+          if (!ok) break;
+          mbar_arrive_expect_tx(&v_full[sv], kTVBytes);
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+            tma_load_2d(base + kTOffV + sv * kTVBytes + a * kTVAtom, &tm_v, c0 + 32 * a, 0, &v_full[sv]);
+          ++nv;
+          if (++sv == kTVStages) {
+            sv = 0;
+            vph ^= 1;
+          }
+        }
+      }
+      // every copy this thread issued has landed before the CTA exits (bounded)
+      for (int k = (seq > 2 ? seq - 2 : 0); k < seq; ++k) dwait(&xi_full[k & 1], (k >> 1) & 1);
+      for (int k = (nx > kTBufs ? nx - kTBufs : 0); k < nx; ++k) dwait(&x_full[k % kTBufs], (k / kTBufs) & 1);
+      for (int k = (nn > kTNStages ? nn - kTNStages : 0); k < nn; ++k)
+        dwait(&n_full[k % kTNStages], (k / kTNStages) & 1);
+      for (int k = (nv > kTVStages ? nv - kTVStages : 0); k < nv; ++k)
+        dwait(&v_full[k % kTVStages], (k / kTVStages) & 1);
+    }
+  } else if (warp == kTEpi + 1) {
+    // ---- MMAs: the first ones run two steps ahead of the second ones.  The warp stays converged, so
+    // that indexes and descriptors are uniform values, and one elected lane issues ----
+    {
+      const bool elected = elect_one();
+      const uint64_t dxi = desc_sw128(smem_u32(base)), dxj = desc_sw128(smem_u32(base + kTOffXJ));
+      const uint64_t dv = desc_sw128(smem_u32(base + kTOffV));
+      const uint32_t dhi = (uint32_t)(dxi >> 32);
+      auto dsc = [&](uint32_t lo) { return ((uint64_t)dhi << 32) | lo; };
+      // kind::tf32, FP32 accumulate, A and B K-major, M = 128; N = 128 and N = m rounded up to 16
+      const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 4) << 24);
+      const uint32_t idesc1 = idesc0 | ((128u >> 3) << 17);
+      const uint32_t n2 = (uint32_t)((m + 15) / 16 * 16);
+      const uint32_t idesc2 = idesc0 | ((n2 >> 3) << 17);
+      // cursor of the first MMAs
+      int it1 = blockIdx.x, j1 = 0, nt1 = it1 < n_items ? items[it1].z : 0, seq1 = 0, b1 = 0;
+      uint32_t ph1 = 0, fph1 = 1;
+      bool ok = true;
+      auto first = [&]() {      // first MMAs of the next step
+        const int xb = seq1 & 1;
+        if (j1 == 0) ok = bwait(&xi_full[xb], (seq1 >> 1) & 1, abort_flag, err);
+        ok = ok && bwait(&x_full[b1], ph1, abort_flag, err) && bwait(&b_free[b1], fph1, abort_flag, err);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) return;
+        fence_after();
+        const uint32_t d = tmem + (uint32_t)(b1 * 128);
+        const uint32_t a = (uint32_t)dxi + (uint32_t)xb * (kXIBytes / 16u), b = (uint32_t)dxj + (uint32_t)b1 * (kTXBytes / 16u);
+        if (elected) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (k < ksteps) mma_tf32(d, dsc(a + k * 2u), dsc(b + k * 2u), idesc1, k > 0 ? 1u : 0u);
+          mma_commit(&s_full[b1]);
+          if (j1 + 1 == nt1) mma_commit(&xi_empty[xb]);
+        }
+        __syncwarp();
+        if (++j1 == nt1) {
+          j1 = 0;
+          ++seq1;
+          it1 += gridDim.x;
+          nt1 = it1 < n_items ? items[it1].z : 0;
+        }
+        if (++b1 == kTBufs) {
+          b1 = 0;
+          ph1 ^= 1;
+          fph1 ^= 1;
+        }
+      };
+      if (it1 < n_items) first();
+      if (ok && it1 < n_items) first();
+      int seq = 0, b = 0, sv = 0;
+      uint32_t ph = 0, vph = 0;
+      for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++seq) {
+        const int nt = items[it].z, ub = seq & 1;
+        const uint32_t du = tmem + kTUCol + (uint32_t)(ub * 64);
+        for (int j = 0; j < nt; ++j) {
+          if (it1 < n_items) first();
+          ok = ok && bwait(&v_full[sv], vph, abort_flag, err) && bwait(&p_full[b], ph, abort_flag, err);
+          if (ok && j == 0) ok = bwait(&u_empty[ub], ((seq >> 1) & 1) ^ 1, abort_flag, err);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          fence_after();
+          const uint32_t pa = tmem + (uint32_t)(b * 128);
+          const uint32_t v = (uint32_t)dv + (uint32_t)sv * (kTVBytes / 16u);
+          if (elected) {
+#pragma unroll
+            for (int k = 0; k < kTN / 8; ++k)
+              mma_tf32_ta(du, pa + (uint32_t)(k * 8), dsc(v + ((uint32_t)(k >> 2) * kTVAtom + (uint32_t)(k & 3) * 32u) / 16u),
+                          idesc2, (j == 0 && k == 0) ? 0u : 1u);
+            mma_commit(&b_free[b]);
+            if (j == nt - 1) mma_commit(&u_full[ub]);
+          }
+          __syncwarp();
+          if (++b == kTBufs) {
+            b = 0;
+            ph ^= 1;
+          }
+          if (++sv == kTVStages) {
+            sv = 0;
+            vph ^= 1;
+          }
+        }
+      }
+      // all MMAs of this thread have completed before the tensor memory is freed (bounded)
+      if (elected) mma_commit(drain);
+      dwait(drain, 0);
+    }
+  } else {
+    // ---- epilogue: warp w takes TMEM lanes 32 (w mod 4) .. + 31 (rows) and 32 columns of a step ----
+    const int lq = warp & 3, cg = warp >> 2;
+    const int r = lq * 32 + lane;
+    const uint32_t lane_off = (uint32_t)(lq * 32) << 16;
+    int b = 0, sn = 0, seq = 0;
+    uint32_t ph = 0, nph = 0;
+    bool ok = true;
+    int pend = -1, pend_it = 0, pend_valid = 0;   // item whose result is still in its accumulator
+    auto read_out = [&]() {
+      const int ub = pend & 1;
+      if (!bwait(&u_full[ub], (pend >> 1) & 1, abort_flag, err)) {
+        ok = false;
+        return;
+      }
+      __syncwarp();
+      fence_after();
+      uint32_t u[16];
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+          "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+          : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]),
+            "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+          : "r"(tmem + kTUCol + (uint32_t)(ub * 64 + cg * 16) + lane_off));
+      tmem_wait_ld();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&u_empty[ub]);
+      if (r < pend_valid) {
+        double* o = out + (size_t)(out0[pend_it] + r) * m + cg * 16;
+        const int mc = m - cg * 16;
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          if (c < mc) o[c] = (double)__uint_as_float(u[c]);
+      }
+      pend = -1;
+    };
+    for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++seq) {
+      const int4 I = items[it];
+      const float ni = __ldg(nrm + I.x + r);
+      const uint64_t ni2 = bpack2(ni, ni), two = bpack2(2.f, 2.f);
+      for (int j = 0; j < I.z; ++j) {
+        if (!bwait(&n_full[sn], nph, abort_flag, err) || !bwait(&s_full[b], ph, abort_flag, err)) {
+          ok = false;
+          break;
+        }
+        __syncwarp();
+        fence_after();
+        uint32_t g[32];
+        const uint32_t cols = tmem + (uint32_t)(b * 128 + cg * 32) + lane_off;
+        tmem_ld32_nowait(cols, g);
+        tmem_wait_ld();
+        const float4* nj4 = reinterpret_cast<const float4*>(base + kTOffN + sn * kTNrm) + cg * 8;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float4 nn = nj4[c];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            uint64_t sum, arg;
+            asm("add.rn.f32x2 %0, %1, %2;" : "=l"(sum) : "l"(ni2), "l"(u ? bpack2(nn.z, nn.w) : bpack2(nn.x, nn.y)));
+            sum ^= 0x8000000080000000ull;
+            asm("fma.rn.f32x2 %0, %1, %2, %3;"
+                : "=l"(arg)
+                : "l"(bpack2(__uint_as_float(g[4 * c + 2 * u]), __uint_as_float(g[4 * c + 2 * u + 1]))), "l"(two), "l"(sum));
+            float a0, a1;
+            bunpack2(arg, a0, a1);
+            g[4 * c + 2 * u] = exp2_tf32(a0);
+            g[4 * c + 2 * u + 1] = exp2_tf32(a1);
+          }
+        }
+        tmem_st32_nowait(cols, g);
+        tmem_wait_st();
+        fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&p_full[b]);
+          mbar_arrive(&n_empty[sn]);
+        }
+        if (++b == kTBufs) {
+          b = 0;
+          ph ^= 1;
+        }
+        if (++sn == kTNStages) {
+          sn = 0;
+          nph ^= 1;
+        }
+        if (pend >= 0 && (j == 1 || I.z == 1)) {
+          read_out();
+          if (!ok) break;
+        }
+      }
+      if (!ok) break;
+      pend = seq;
+      pend_it = it;
+      pend_valid = I.w;
+    }
+    if (ok && pend >= 0) read_out();
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (warp == kTEpi + 1) tmem_dealloc_b(tmem, 512);
 }
 
 // Row-major padded TF32 coordinates xt[R][32] and squared norms of the rounded rows.
@@ -561,7 +900,8 @@ kqr_status batch_create(Handle* h, const double* X, const int64_t* offsets, int6
   std::vector<It> its;
   for (int64_t b = 0; b < B; ++b) {
     const int64_t nb = offsets[b + 1] - offsets[b];
-    const int nt = (int)((nb + kBN - 1) / kBN);
+    const int step = bd->p_in_smem ? kBN : kTN;
+    const int nt = (int)((nb + step - 1) / step);
     for (int64_t i0 = 0; i0 < nb; i0 += kBM)
       its.push_back({(int)(bd->roff[b] + i0), (int)bd->roff[b], nt, (int)std::min<int64_t>(kBM, nb - i0),
                      (int)(offsets[b] + i0)});
@@ -636,15 +976,22 @@ cudaError_t batch_kmatmul(Handle* h, const double* V, double* U, int m, cudaStre
   h->launches++;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  auto kern = bd->p_in_smem ? batch_kv_kernel<false> : batch_kv_kernel<true>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem);
-  if (e != cudaSuccess) return e;
   const int grid = std::min(h->num_sms, bd->n_items);
   const int ksteps = (int)((bd->p + 7) / 8);
-  prof_mark(h, 0, true, st);
-  kern<<<grid, kBatchThreads, kBatchSmem, st>>>(bd->tm_xi, bd->tm_xj, bd->tm_v, bd->nrm,
-                                              reinterpret_cast<const int4*>(bd->items), bd->out0, bd->n_items,
-                                              ksteps, U, m, h->err_flag);
+  const int4* items = reinterpret_cast<const int4*>(bd->items);
+  if (bd->p_in_smem) {
+    e = cudaFuncSetAttribute(batch_kv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem);
+    if (e != cudaSuccess) return e;
+    prof_mark(h, 0, true, st);
+    batch_kv_kernel<<<grid, kBatchThreads, kBatchSmem, st>>>(bd->tm_xi, bd->tm_xj, bd->tm_v, bd->nrm, items, bd->out0,
+                                                             bd->n_items, ksteps, U, m, h->err_flag);
+  } else {
+    e = cudaFuncSetAttribute(batch_kv_tmem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTSmem);
+    if (e != cudaSuccess) return e;
+    prof_mark(h, 0, true, st);
+    batch_kv_tmem_kernel<<<grid, kTThreads, kTSmem, st>>>(bd->tm_xi, bd->tm_v, bd->nrm, items, bd->out0, bd->n_items,
+                                                          ksteps, U, m, h->err_flag);
+  }
   prof_mark(h, 0, false, st);
   h->launches++;
   return cudaGetLastError();
