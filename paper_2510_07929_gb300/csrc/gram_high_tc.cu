@@ -23,7 +23,7 @@
 // 40 instructions per MMA among 16 busy warps and made the MMAs the bound).  For one vector each
 // off-diagonal tile serves its rows and its columns (n(n+1)/2 entries); for several, an entry is formed
 // once per pass over K and added to every vector's row sums.  Measured: one vector, n = 50000, p = 20:
-// 4.33 ms (issue slots 66 % used), before 20.9 ms; eight vectors, n = 10007, p = 8: 0.62 ms, before
+// 3.79 ms, before 20.9 ms; eight vectors, n = 10007, p = 8: 0.62 ms, before
 // 4.38 ms.  Before: int64 sums of squared differences on the CUDA cores (6 operations per entry and
 // feature, all n^2 entries, columns one after another).
 //
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_free + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = M == 1 ? warp_index() : tid >> 5, lane = tid & 31;
   const int4 unit = units[blockIdx.x];
   const int ti = unit.x, jt0 = unit.y, nt = unit.z - unit.y;
 
@@ -250,10 +250,20 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == kEpiWarps) {
-    if (lane == 0) {
+    // Copies and MMAs.  M = 1: the warp stays converged, so that indexes and descriptors are uniform
+    // values, and one elected lane issues (n = 50000: 3.79 ms, 4.32 with a branch of one lane); with
+    // several vectors one lane does it all, which measured faster (M = 8, n = 10007: 0.62 against 0.64).
+    constexpr bool kConverged = M == 1;
+    if (kConverged || lane == 0) {
+      const bool elected = !kConverged || elect_one();
+      auto agree = [](bool ok) { return kConverged ? (bool)__all_sync(0xffffffffu, ok) : ok; };
+      auto join = []() {
+        if (kConverged) __syncwarp();
+      };
       auto load_j = [&](int q) {
         const int s = q % kStages;
         const int col0 = (jt0 + q) * kJCols;
+        if (!elected) return;
         mbar_arrive_expect_tx(&full_j[s], j_bytes + kJCols * 16u + kJCols * M * 8u);
         for (int a = 0; a < katoms; ++a)
           tma_load_2d(base + off_j + s * j_bytes + a * kJAtom, &tm_j, a * 32, col0, &full_j[s]);
@@ -265,28 +275,36 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
       const uint64_t i_desc = ht_desc(sbase), j_desc = ht_desc(sbase + off_j);
       int loaded = 0, issued = 0;
       bool ok = true;
-      mbar_arrive_expect_tx(full_i, i_bytes);
-      for (int a = 0; a < katoms; ++a) tma_load_2d(base + a * kIAtom, &tm_i, a * 32, ti * 128, full_i);
+      if (elected) {
+        mbar_arrive_expect_tx(full_i, i_bytes);
+        for (int a = 0; a < katoms; ++a) tma_load_2d(base + a * kIAtom, &tm_i, a * 32, ti * 128, full_i);
+      }
       for (; loaded < nt && loaded < kStages; ++loaded) load_j(loaded);
       for (int q = 0; q < nt && ok; ++q) {
         const int s = q % kStages, b = q & 1;
         if (q == 0) ok = mbar_wait_bounded(full_i, 0, err);
         if (ok) ok = mbar_wait_bounded(&full_j[s], (uint32_t)((q / kStages) & 1), err);
         if (ok && q >= 2) ok = *abort_flag == 0 && mbar_wait_bounded(&tmem_free[b], (uint32_t)(((q >> 1) - 1) & 1), err);
+        ok = agree(ok);
         if (!ok) break;
         ht_fence_after();
-        ht_issue_tile<KS>(tmem + (uint32_t)(b * 256), (uint32_t)i_desc, (uint32_t)j_desc + s * (j_bytes / 16u),
-                          (uint32_t)(i_desc >> 32), idesc);
-        ht_commit(&mma_done[b]);
+        if (elected) {
+          ht_issue_tile<KS>(tmem + (uint32_t)(b * 256), (uint32_t)i_desc, (uint32_t)j_desc + s * (j_bytes / 16u),
+                            (uint32_t)(i_desc >> 32), idesc);
+          ht_commit(&mma_done[b]);
+        }
+        join();
         issued = q + 1;
         // the stage that held tile q - 2 takes tile q + 1: waiting for a later stage here would hold the
         // next tile's MMAs back until the epilogue of tile q - 1 is over
         if (q >= 2 && loaded < nt) {
           ok = *abort_flag == 0 && mbar_wait_bounded(&stage_free[(q - 2) % kStages], (uint32_t)(((q - 2) / kStages) & 1), err);
+          ok = agree(ok);
           if (ok) {
             load_j(loaded);
             ++loaded;
           }
+          join();
         }
       }
       if (!ok) {
