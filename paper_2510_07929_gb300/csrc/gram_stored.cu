@@ -132,11 +132,26 @@ __global__ void __launch_bounds__(256) kstore_fill_kernel(const float* __restric
   }
 }
 
+// What the one-launch product needs besides the tiles.
+struct KsWhole {
+  const double* V = nullptr;
+  double* out = nullptr;
+  int64_t n = 0;
+  unsigned int* counter = nullptr;
+};
+
 // Symmetric streaming product over the stored tiles; sched[b] = (t0, t1, I0, J0)
 // is CTA b's tile range and the (I, J) of its first tile.
+//
+// WHOLE: the plain product in one launch, for the sizes of kKsWholeRows.  The vector is read as FP64
+// and rounded on the way; the CTA that finishes last turns the sums into the result and leaves them
+// zero for the next product (acc is then a buffer of its own, zeroed once).  A few microseconds of
+// work are bound by launches: n = 2000 takes 3.3 us a product back to back, in three launches
+// (convert, multiply, finish) 6.6.
+template <bool WHOLE>
 __global__ void __launch_bounds__(kKsThreads, 1)
     kstore_gemv_kernel(const float* __restrict__ K, const float* __restrict__ v32, float* __restrict__ acc,
-                       const int4* __restrict__ sched, int T, int* __restrict__ err) {
+                       const int4* __restrict__ sched, int T, const KsWhole whole, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char ks_raw[];
   float* stages = reinterpret_cast<float*>(ks_raw);                              // kKsStages x 4096
   float* colred = stages + kKsStages * kKsChunkFloats;                           // [2][8][128]
@@ -194,7 +209,10 @@ __global__ void __launch_bounds__(kKsThreads, 1)
   bool aborted = false;
   auto load_vi = [&](int Irow) {
 #pragma unroll
-    for (int r = 0; r < 16; ++r) vi[r] = __ldg(v32 + (size_t)Irow * kTile + (r >> 2) * kKsChunkRows + 4 * warp + (r & 3));
+    for (int r = 0; r < 16; ++r) {
+      const int64_t i = (int64_t)Irow * kTile + (r >> 2) * kKsChunkRows + 4 * warp + (r & 3);
+      vi[r] = WHOLE ? (i < whole.n ? (float)__ldg(whole.V + i) : 0.f) : __ldg(v32 + i);
+    }
   };
   const int ntiles = t1 - t0;
   if (ntiles > 0) load_vi(I);
@@ -203,7 +221,15 @@ __global__ void __launch_bounds__(kKsThreads, 1)
     for (int r = 0; r < 16; ++r) rp[r] = 0.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) col[j] = 0.f;
-    vj = __ldg(reinterpret_cast<const float4*>(v32 + (size_t)J * kTile) + lane);
+    if (WHOLE) {
+      const int64_t j = (int64_t)J * kTile + 4 * lane;
+      vj.x = j < whole.n ? (float)__ldg(whole.V + j) : 0.f;
+      vj.y = j + 1 < whole.n ? (float)__ldg(whole.V + j + 1) : 0.f;
+      vj.z = j + 2 < whole.n ? (float)__ldg(whole.V + j + 2) : 0.f;
+      vj.w = j + 3 < whole.n ? (float)__ldg(whole.V + j + 3) : 0.f;
+    } else {
+      vj = __ldg(reinterpret_cast<const float4*>(v32 + (size_t)J * kTile) + lane);
+    }
 #pragma unroll
     for (int q = 0; q < kKsChunksPerTile; ++q) {
       const int c = tl * kKsChunksPerTile + q;
@@ -288,8 +314,33 @@ __global__ void __launch_bounds__(kKsThreads, 1)
     I = nI;
     J = nJ;
   }
+  if (!WHOLE) return;
+
+  // ---- the CTA that finishes last: every other CTA's sums are there
+  __shared__ bool last_cta;
+  __threadfence();
+  consumer_sync();
+  if (threadIdx.x == 0) last_cta = atomicAdd(whole.counter, 1u) == gridDim.x - 1;
+  consumer_sync();
+  if (!last_cta) return;
+  __threadfence();
+  const int rows = T * kTile;
+  // four rows a thread and pass: the tail is a chain of latencies
+  for (int i = 4 * threadIdx.x; i < rows; i += 4 * kKsConsumerWarps * 32) {
+    const float4 a4 = __ldcg(reinterpret_cast<const float4*>(acc + i));
+    const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+    *reinterpret_cast<float4*>(acc + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k < whole.n) whole.out[i + k] = (double)a[k];
+  }
+  if (threadIdx.x == 0) *whole.counter = 0u;
 }
 
+// Up to this many rows a plain product is one launch (n = 5000: 3.3 us back to back against 6.5).  The
+// products of CG are not: their last step has the operator's terms and a dot product, which one CTA
+// takes longer over than a launch of its own (a system of n = 2000: 2.87 against 2.62 ms).
+constexpr int64_t kKsWholeRows = 5120;
 constexpr size_t kStoreL2Bytes = (size_t)64 << 20;   // stored tiles up to this size stay in L2
 
 size_t kstore_bytes(int64_t ldn) {
@@ -360,13 +411,25 @@ kqr_status kstore_setup(Handle* h) {
   }
   h->launches++;
   if (e == cudaSuccess) e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kstore_gemv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kstore_gemv_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)kstore_smem());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kstore_gemv_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)kstore_smem());
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     dev_free(h, K);
     dev_free(h, dsched);
     return cuda_fail(h, e, "stored K fill");
+  }
+  if (h->ldn <= kKsWholeRows) {
+    // sums of the one-launch product, zero between products (without them it takes three launches)
+    h->kstore_acc = (float*)dev_alloc(h, h->ldn * sizeof(float));
+    if (h->kstore_acc && (cudaMemsetAsync(h->kstore_acc, 0, h->ldn * sizeof(float), st) != cudaSuccess ||
+                          cudaStreamSynchronize(st) != cudaSuccess)) {
+      dev_free(h, h->kstore_acc);
+      h->kstore_acc = nullptr;
+    }
+    cudaGetLastError();
   }
   h->kstore = K;
   h->kstore_bytes = bytes;
@@ -378,6 +441,8 @@ kqr_status kstore_setup(Handle* h) {
 void kstore_free(Handle* h) {
   dev_free(h, h->kstore);
   dev_free(h, h->kstore_sched);
+  dev_free(h, h->kstore_acc);
+  h->kstore_acc = nullptr;
   h->kstore = nullptr;
   h->kstore_sched = nullptr;
   h->kstore_bytes = 0;
@@ -385,16 +450,29 @@ void kstore_free(Handle* h) {
 
 cudaError_t gram_stored(Handle* h, const double* V, double* U, const GramEpilogue* ep, cudaStream_t st) {
   cudaError_t e;
+  GramEpilogue none;
+  const GramEpilogue& g = ep ? *ep : none;
+  if (h->kstore_acc && !ep && (U + h->n <= V || V + h->n <= U)) {   // it reads V to the end
+    KsWhole w;
+    w.V = V;
+    w.out = U;
+    w.n = h->n;
+    w.counter = h->red_counter;
+    prof_mark(h, 2, true, st);
+    kstore_gemv_kernel<true><<<h->kstore_grid, kKsThreads, kstore_smem(), st>>>(
+        h->kstore, nullptr, h->kstore_acc, h->kstore_sched, (int)(h->ldn / kTile), w, h->err_flag);
+    prof_mark(h, 2, false, st);
+    h->launches++;
+    return cudaGetLastError();
+  }
   float* v32;
   double* sums;
   if ((e = sym_buffers(h, &v32, &sums)) != cudaSuccess) return e;
   float* acc = reinterpret_cast<float*>(sums);
-  GramEpilogue none;
-  const GramEpilogue& g = ep ? *ep : none;
   if (!g.prepped && (e = sym_prep(h, V, v32, sums, const_cast<double*>(g.sum_p), st)) != cudaSuccess) return e;
   prof_mark(h, 2, true, st);
-  kstore_gemv_kernel<<<h->kstore_grid, kKsThreads, kstore_smem(), st>>>(h->kstore, v32, acc, h->kstore_sched,
-                                                                       (int)(h->ldn / kTile), h->err_flag);
+  kstore_gemv_kernel<false><<<h->kstore_grid, kKsThreads, kstore_smem(), st>>>(
+      h->kstore, v32, acc, h->kstore_sched, (int)(h->ldn / kTile), KsWhole{}, h->err_flag);
   prof_mark(h, 2, false, st);
   h->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

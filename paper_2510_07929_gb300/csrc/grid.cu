@@ -287,6 +287,7 @@ static Handle* column_clone(Handle* base, GridRdv* g, kqr_status* st) {
   c->part_cap = 0;
   c->v32 = nullptr;
   c->v32_cap = 0;
+  c->kstore_acc = nullptr;  // the base handle keeps it
   c->stream = nullptr;
   c->scal_host = nullptr;
   c->opt.cg_tf32 = 0;       // the grid runs FP32 or FP64-class CG products only

@@ -211,6 +211,7 @@ struct Handle {
   float* kstore = nullptr;
   size_t kstore_bytes = 0;
   int4* kstore_sched = nullptr;       // per-CTA (first tile, end tile, I, J) of the product
+  float* kstore_acc = nullptr;        // sums of the one-launch product (its own buffer: zero between products)
   int kstore_grid = 0;
 };
 
