@@ -592,7 +592,7 @@ constexpr int kSymCols = 32;                       // columns of tile I per warp
 static_assert(kSymEpi * 32 * kSymCols == kTile * kTile, "the warps cover a tile");
 constexpr int kSymThreads = (kSymEpi + 2) * 32;    // + copy warp + MMA warp
 constexpr int kSymBufs = 4;                        // TMEM accumulators of 128 columns
-constexpr int kSymMaxStages = 4;
+constexpr int kSymMaxStages = 8;
 
 __device__ __forceinline__ uint64_t pack2(float a, float b) {
   uint64_t r;
@@ -917,7 +917,7 @@ __global__ void __launch_bounds__(kSymThreads, 1)
   if (warp == kSymEpi) tmem_dealloc(tmem, 128 * kSymBufs);
 }
 
-// Row-tile buffers and J stages: 2 + 4 (tiles of 16 KB), 2 + 3 (32 KB), 1 + 2 (64 KB).
+// Row-tile buffers and J stages: 2 + 8 (tiles of 16 KB; 4: 0.33 ms), 2 + 3 (32 KB), 1 + 2 (64 KB).
 static void tc_sym_stages(size_t tile_bytes, int* nibuf, int* nstage) {
   *nibuf = tile_bytes <= 32 * 1024 ? 2 : 1;
   *nstage = tile_bytes <= 16 * 1024 ? kSymMaxStages : (tile_bytes <= 32 * 1024 ? 3 : 2);
