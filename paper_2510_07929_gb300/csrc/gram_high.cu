@@ -131,11 +131,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
           const int dH = ha[a] - hb[b];
-          A[a][b] += abs(dH);
+          A[a][b] = (int)__sad(ha[a], hb[b], (unsigned)A[a][b]);
           const float dl = la[a] - lb[b];
           const int dlb = __float_as_int(dl);
           // key < 0 exactly when the true difference is negative: dH <= -1, or dH == 0 and dl < 0.
-          const int key = (dH << 1) + (dlb >> 31);
+          const int key = dH - (int)((unsigned)dlb >> 31);
           Lo[a][b] += __int_as_float(dlb ^ (key & (int)0x80000000));
         }
     }

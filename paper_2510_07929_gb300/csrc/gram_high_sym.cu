@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     s_hi[a] = s_lo[a] = 0.f;
   }
   const float scaleG = __int_as_float((127 - G) << 23);
-  const int mone = -one, two = one + one;
+  const int mone = -one;
   const int shift_f = G - kTBs;
   const int mask_f = (1 << kTBs) - 1;
   const int mask_r = (1 << shift_f) - 1;
@@ -162,18 +162,20 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float la[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
       const int hb[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
       const float lb[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-      // Integer adds are written as multiply-adds by the run-time constant `one`
-      // (= 1) so that they issue on the FMA pipe, which the float part leaves
-      // mostly idle, instead of the integer ALU pipe (the bottleneck otherwise).
+      // Per feature and entry: one sum of absolute differences for the integer part (21.0 -> 18.9 ms at
+      // n = 50001, p = 50, against abs and a multiply-add), the integer difference as a multiply-add by a
+      // run-time -1 (on the FMA pipe, which the float part leaves mostly idle), and the float part
+      // with the sign of the whole difference, which is that of dH - (dl < 0): negative for dH <= -1, and
+      // for dH = 0 if dl is (17.3 ms, against 2 dH - (dl < 0) as a multiply-add).
 #pragma unroll
       for (int a = 0; a < 8; ++a)
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
           const int dH = hb[b] * mone + ha[a];
-          A[a][b] = abs(dH) * one + A[a][b];
+          A[a][b] = (int)__sad(ha[a], hb[b], (unsigned)A[a][b]);
           const float dl = la[a] - lb[b];
           const int dlb = __float_as_int(dl);
-          const int key = dH * two + (dlb >> 31);
+          const int key = dH - (int)((unsigned)dlb >> 31);
           Lo[a][b] += __int_as_float(dlb ^ (key & (int)0x80000000));
         }
     }
