@@ -12,6 +12,7 @@
 // shared memory (double-buffered by tile parity) and added to the output with
 // FP32 atomics, as are the unit's row sums at the end; the order of those
 // additions is not fixed, so results vary in the last bits between runs.
+#include <cmath>
 #include <vector>
 
 #include "kqr_internal.h"
@@ -20,12 +21,71 @@
 
 namespace kqr {
 
-enum { SYM_RBF = 0, SYM_LAP = 1 };
+enum { SYM_RBF = 0, SYM_LAP = 1, SYM_LAP_MIX = 2 };
+
+// ---- Laplacian distances on two pipes (SYM_LAP_MIX) --------------------------------------
+// A feature's |x_i - x_j| costs two FP32 operations (a difference and an addition), 128 lanes a clock
+// and SM, or one 64-lane integer sum of absolute differences of the fixed-point coordinates hq =
+// round(xs 2^G) of the FP64-class layout.  The first p_int features go to the integer pipe, the others
+// to the FP32 one (differences as packed f32x2, which halves their issue slots); half of the warps of
+// every scheduler take the integer features first and the other half last, so that both pipes work.
+// A thread's 64 sums change type between the two: integer sums are below 2^30 (the choice of G), FP32
+// sums are rounded to the 2^-G grid.  The integer unit turned out to share much of the FP32 lanes' time
+// (busy 53 and 42 % together): n = 200000, p = 50 takes 50.9 ms, 61.5 with all features in FP32.
+__device__ __forceinline__ uint64_t lap_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+__device__ __forceinline__ void lap_int(const int32_t* HI, const int32_t* HJ, int n, int ty, int tx,
+                                        unsigned (&A)[8][8]) {
+#pragma unroll 2
+  for (int k = 0; k < n; ++k) {
+    const int4 a0 = *reinterpret_cast<const int4*>(HI + k * kTile + ty * 8);
+    const int4 a1 = *reinterpret_cast<const int4*>(HI + k * kTile + ty * 8 + 4);
+    const int4 b0 = *reinterpret_cast<const int4*>(HJ + k * kTile + tx * 8);
+    const int4 b1 = *reinterpret_cast<const int4*>(HJ + k * kTile + tx * 8 + 4);
+    const int ha[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+    const int hb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int b = 0; b < 8; ++b) A[a][b] = __sad(ha[a], hb[b], A[a][b]);
+  }
+}
+
+__device__ __forceinline__ void lap_f32(const float* XI, const float* XJ, int n, int ty, int tx, float (&d)[8][8]) {
+  const uint64_t mone = lap_pack(-1.f, -1.f);
+#pragma unroll 2
+  for (int k = 0; k < n; ++k) {
+    const float4 a0 = *reinterpret_cast<const float4*>(XI + k * kTile + ty * 8);
+    const float4 a1 = *reinterpret_cast<const float4*>(XI + k * kTile + ty * 8 + 4);
+    const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(XJ + k * kTile + tx * 8);
+    const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(XJ + k * kTile + tx * 8 + 4);
+    const float xa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+    const uint64_t xb[4] = {b0.x, b0.y, b1.x, b1.y};
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const uint64_t aa = lap_pack(xa[a], xa[a]);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        uint64_t t;
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(xb[b]), "l"(mone), "l"(aa));
+        float t0, t1;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(t0), "=f"(t1) : "l"(t));
+        d[a][2 * b] += fabsf(t0);
+        d[a][2 * b + 1] += fabsf(t1);
+      }
+    }
+  }
+}
 
 template <int KIND>
 __global__ void __launch_bounds__(kThreads, 2)
     gram_f32_sym_kernel(const __grid_constant__ CUtensorMap tm, const float* __restrict__ nrm,
                         const float* __restrict__ v32, const int4* __restrict__ units, float* __restrict__ acc, int p,
+                        const __grid_constant__ CUtensorMap tm_int, int p_int, float grid, float grid_inv,
                         int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* XI = reinterpret_cast<float*>(smem_raw);
@@ -50,11 +110,19 @@ __global__ void __launch_bounds__(kThreads, 2)
     fence_mbar_init();
   }
   __syncthreads();
+  // one tile: p rows of 128 coordinates; SYM_LAP_MIX: the p_int fixed-point rows, then the FP32 ones
+  auto load_tile = [&](float* dst, int c0, uint64_t* bar) {
+    mbar_arrive_expect_tx(bar, bytes);
+    if (KIND == SYM_LAP_MIX) {
+      tma_load_2d(dst, &tm_int, c0, 0, bar);
+      tma_load_2d(dst + p_int * kTile, &tm, c0, p_int, bar);
+    } else {
+      tma_load_2d(dst, &tm, c0, 0, bar);
+    }
+  };
   if (tid == 0) {
-    mbar_arrive_expect_tx(&bars[0], bytes);
-    tma_load_2d(XI, &tm, row0, 0, &bars[0]);
-    mbar_arrive_expect_tx(&bars[1], bytes);
-    tma_load_2d(XJ0, &tm, jt0 * kTile, 0, &bars[1]);
+    load_tile(XI, row0, &bars[0]);
+    load_tile(XJ0, jt0 * kTile, &bars[1]);
   }
   float va[8], ni[8];
 #pragma unroll
@@ -73,8 +141,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     float* XJ = s ? XJ1 : XJ0;
     if (tid == 0 && t + 1 < jt1) {
       const int ns = (q + 1) & 1;
-      mbar_arrive_expect_tx(&bars[1 + ns], bytes);
-      tma_load_2d(ns ? XJ1 : XJ0, &tm, (t + 1) * kTile, 0, &bars[1 + ns]);
+      load_tile(ns ? XJ1 : XJ0, (t + 1) * kTile, &bars[1 + ns]);
     }
     const int col0 = t * kTile + tx * 8;
     float vb[8], nj[8];
@@ -86,27 +153,60 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) return;
 
     float d[8][8];
+    if (KIND == SYM_LAP_MIX) {
+      const int32_t* HI = reinterpret_cast<const int32_t*>(XI);
+      const int32_t* HJ = reinterpret_cast<const int32_t*>(XJ);
+      unsigned A[8][8];
+      if (warp & 4) {
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+        for (int a = 0; a < 8; ++a)
 #pragma unroll
-      for (int b = 0; b < 8; ++b) d[a][b] = 0.f;
-#pragma unroll 2
-    for (int k = 0; k < p; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(XI + k * kTile + ty * 8);
-      const float4 a1 = *reinterpret_cast<const float4*>(XI + k * kTile + ty * 8 + 4);
-      const float4 b0 = *reinterpret_cast<const float4*>(XJ + k * kTile + tx * 8);
-      const float4 b1 = *reinterpret_cast<const float4*>(XJ + k * kTile + tx * 8 + 4);
-      const float xa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float xb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+          for (int b = 0; b < 8; ++b) d[a][b] = 0.f;
+        lap_f32(XI + p_int * kTile, XJ + p_int * kTile, p - p_int, ty, tx, d);
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+          for (int b = 0; b < 8; ++b) A[a][b] = __float2uint_rn(d[a][b] * grid_inv);
+        lap_int(HI, HJ, p_int, ty, tx, A);
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+          for (int b = 0; b < 8; ++b) d[a][b] = __uint2float_rn(A[a][b]) * grid;
+      } else {
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+          for (int b = 0; b < 8; ++b) A[a][b] = 0u;
+        lap_int(HI, HJ, p_int, ty, tx, A);
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+          for (int b = 0; b < 8; ++b) d[a][b] = __uint2float_rn(A[a][b]) * grid;
+        lap_f32(XI + p_int * kTile, XJ + p_int * kTile, p - p_int, ty, tx, d);
+      }
+    } else {
 #pragma unroll
       for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
-          if (KIND == SYM_LAP)
-            d[a][b] += fabsf(xa[a] - xb[b]);
-          else
-            d[a][b] = fmaf(xa[a], xb[b], d[a][b]);
-        }
+        for (int b = 0; b < 8; ++b) d[a][b] = 0.f;
+#pragma unroll 2
+      for (int k = 0; k < p; ++k) {
+        const float4 a0 = *reinterpret_cast<const float4*>(XI + k * kTile + ty * 8);
+        const float4 a1 = *reinterpret_cast<const float4*>(XI + k * kTile + ty * 8 + 4);
+        const float4 b0 = *reinterpret_cast<const float4*>(XJ + k * kTile + tx * 8);
+        const float4 b1 = *reinterpret_cast<const float4*>(XJ + k * kTile + tx * 8 + 4);
+        const float xa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float xb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+          for (int b = 0; b < 8; ++b) {
+            if (KIND == SYM_LAP)
+              d[a][b] += fabsf(xa[a] - xb[b]);
+            else
+              d[a][b] = fmaf(xa[a], xb[b], d[a][b]);
+          }
+      }
     }
     float cs[8];
 #pragma unroll
@@ -115,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     for (int a = 0; a < 8; ++a)
 #pragma unroll
       for (int b = 0; b < 8; ++b) {
-        const float arg = (KIND == SYM_LAP) ? -d[a][b] : fmaf(2.f, d[a][b], -(ni[a] + nj[b]));
+        const float arg = (KIND != SYM_RBF) ? -d[a][b] : fmaf(2.f, d[a][b], -(ni[a] + nj[b]));
         const float e = ex2_approx(arg);
         racc[a] = fmaf(e, vb[b], racc[a]);
         cs[b] = fmaf(e, va[a], cs[b]);
@@ -231,17 +331,14 @@ cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilog
   float* acc = reinterpret_cast<float*>(sums);
   const size_t smem = sym_smem_bytes((int)h->p);
   prof_mark(h, 0, true, st);
-  if (h->kind == KQR_LAPLACIAN) {
-    e = cudaFuncSetAttribute(gram_f32_sym_kernel<SYM_LAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    gram_f32_sym_kernel<SYM_LAP><<<h->sym_nunits, kThreads, smem, st>>>(h->tm_xs32, h->nrm32, v32, h->sym_units, acc,
-                                                                        (int)h->p, h->err_flag);
-  } else {
-    e = cudaFuncSetAttribute(gram_f32_sym_kernel<SYM_RBF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    gram_f32_sym_kernel<SYM_RBF><<<h->sym_nunits, kThreads, smem, st>>>(h->tm_xs32, h->nrm32, v32, h->sym_units, acc,
-                                                                        (int)h->p, h->err_flag);
-  }
+  const bool mix = h->kind == KQR_LAPLACIAN && h->lap_int > 0;
+  auto kern = mix ? gram_f32_sym_kernel<SYM_LAP_MIX>
+                  : (h->kind == KQR_LAPLACIAN ? gram_f32_sym_kernel<SYM_LAP> : gram_f32_sym_kernel<SYM_RBF>);
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<h->sym_nunits, kThreads, smem, st>>>(mix ? h->tm_lap_f32 : h->tm_xs32, h->nrm32, v32, h->sym_units, acc,
+                                              (int)h->p, h->tm_lap_int, h->lap_int, std::ldexp(1.f, -h->grid_G),
+                                              std::ldexp(1.f, h->grid_G), h->err_flag);
   prof_mark(h, 0, false, st);
   h->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

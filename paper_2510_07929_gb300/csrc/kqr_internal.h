@@ -107,6 +107,9 @@ struct Handle {
   float* hl = nullptr;
   int grid_G = 0;
   CUtensorMap tm_hq{}, tm_hl{};
+  // FP32-class Laplacian tiles: features [0, lap_int) from hq, the others from xs32 (0: all from xs32).
+  CUtensorMap tm_lap_int{}, tm_lap_f32{};
+  int lap_int = 0;
   float2* exp_table = nullptr;        // 2^-(k / 2^kExpTableBits) as (hi, lo) floats
   // Centred FP64 copy, feature-major [p][ldn] (RBF high-precision product and K columns).
   double* xc64 = nullptr;
