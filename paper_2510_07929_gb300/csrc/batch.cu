@@ -455,19 +455,17 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
 // clock) are 512 cycles a step, the second contraction's 16 MMAs another 512 on the tensor pipe.
 // The previous form (64-column steps, two groups of four epilogue warps on alternate steps, one
 // warp per scheduler each) spent 2800 cycles on half as many entries waiting on hand-offs: 10.3 ms
-// for the 64-problem workload at m = 64, now 4.2.  Here 16 epilogue warps share a step (32 columns
-// each), the first MMAs run two steps ahead, stage indexes and descriptors are running values (6.5 ms
-// when a branch of one lane issued the MMAs), and an item's result is read out one step into the next
-// item, when its last MMAs are done.  A step now takes 2050 cycles, still the chain S - P - second
-// MMAs - free buffer over three buffers: without the epilogue's work it takes 1900, without 15 of the
-// 16 second MMAs 1650, without both 1430; half the copies (two row tiles per X_J and V_J) and
-// accumulators read half a step ahead change nothing.
+// for the 64-problem workload at m = 64, now 3.35.  Here 16 epilogue warps share a step (32 columns
+// each); copies, first MMAs and second MMAs are issued by a warp each, converged, with running stage
+// indexes and descriptors (6.5 ms from a branch of one lane; 4.16 ms with one warp for all MMAs, which
+// waited for a buffer to come free for the first ones while the second ones' operands were ready); and
+// an item's result is read out one step into the next item, when its last MMAs are done.
 constexpr int kTN = 128;                        // Gram columns per step
 constexpr int kTBufs = 3;                       // S/P buffers and X_J, V_J stages
 constexpr int kTVStages = kTBufs;               // V_J stages
 constexpr int kTNStages = 6;                    // column norms of a step (copied with X_J, ahead of V_J)
 constexpr int kTEpi = 16;
-constexpr int kTThreads = (kTEpi + 2) * 32;
+constexpr int kTThreads = (kTEpi + 3) * 32;    // + copies, first MMAs, second MMAs
 constexpr uint32_t kTXBytes = kTN * 128;        // 128 rows x 128 B
 constexpr uint32_t kTVAtom = kBR * 128;         // 64 right-hand sides x 32 columns
 constexpr uint32_t kTVBytes = 4 * kTVAtom;
@@ -476,7 +474,7 @@ constexpr uint32_t kTOffXJ = 2 * kXIBytes;
 constexpr uint32_t kTOffV = kTOffXJ + kTBufs * kTXBytes;
 constexpr uint32_t kTOffN = kTOffV + kTVStages * kTVBytes;
 constexpr uint32_t kTOffBar = kTOffN + kTNStages * kTNrm;
-constexpr int kTNumBars = 4 + 4 * kTBufs + kTVStages + 2 * kTNStages + 4 + 1;
+constexpr int kTNumBars = 4 + 4 * kTBufs + kTVStages + 2 * kTNStages + 4 + 2;
 constexpr size_t kTSmem = 1024 + kTOffBar + kTNumBars * 8 + 16;
 constexpr uint32_t kTUCol = kTBufs * 128;
 
@@ -515,7 +513,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   uint64_t* b_free = p_full + kTBufs;           // second MMAs done: the buffer can take another S
   uint64_t* u_full = b_free + kTBufs;           // [2]
   uint64_t* u_empty = u_full + 2;               // [2]
-  uint64_t* drain = u_empty + 2;
+  uint64_t* drain = u_empty + 2;                // [2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kTNumBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -544,7 +542,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
       mbar_init(&n_full[i], 1);
       mbar_init(&n_empty[i], kTEpi);
     }
-    mbar_init(drain, 1);
+    mbar_init(&drain[0], 1);
+    mbar_init(&drain[1], 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -609,32 +608,28 @@ __global__ void __launch_bounds__(kTThreads, 1)
         dwait(&v_full[k % kTVStages], (k / kTVStages) & 1);
     }
   } else if (warp == kTEpi + 1) {
-    // ---- MMAs: the first ones run two steps ahead of the second ones.  The warp stays converged, so
-    // that indexes and descriptors are uniform values, and one elected lane issues ----
+    // ---- first MMAs, S = X_I X_J^T.  The warp stays converged, so that indexes and descriptors are
+    // uniform values, and one elected lane issues ----
     {
       const bool elected = elect_one();
       const uint64_t dxi = desc_sw128(smem_u32(base)), dxj = desc_sw128(smem_u32(base + kTOffXJ));
-      const uint64_t dv = desc_sw128(smem_u32(base + kTOffV));
       const uint32_t dhi = (uint32_t)(dxi >> 32);
       auto dsc = [&](uint32_t lo) { return ((uint64_t)dhi << 32) | lo; };
-      // kind::tf32, FP32 accumulate, A and B K-major, M = 128; N = 128 and N = m rounded up to 16
-      const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 4) << 24);
-      const uint32_t idesc1 = idesc0 | ((128u >> 3) << 17);
-      const uint32_t n2 = (uint32_t)((m + 15) / 16 * 16);
-      const uint32_t idesc2 = idesc0 | ((n2 >> 3) << 17);
-      // cursor of the first MMAs
+      // kind::tf32, FP32 accumulate, A and B K-major, M = 128, N = 128
+      const uint32_t idesc1 = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
       int it1 = blockIdx.x, j1 = 0, nt1 = it1 < n_items ? items[it1].z : 0, seq1 = 0, b1 = 0;
       uint32_t ph1 = 0, fph1 = 1;
       bool ok = true;
-      auto first = [&]() {      // first MMAs of the next step
+      while (it1 < n_items) {
         const int xb = seq1 & 1;
         if (j1 == 0) ok = bwait(&xi_full[xb], (seq1 >> 1) & 1, abort_flag, err);
         ok = ok && bwait(&x_full[b1], ph1, abort_flag, err) && bwait(&b_free[b1], fph1, abort_flag, err);
         ok = __all_sync(0xffffffffu, ok);
-        if (!ok) return;
+        if (!ok) break;
         fence_after();
         const uint32_t d = tmem + (uint32_t)(b1 * 128);
-        const uint32_t a = (uint32_t)dxi + (uint32_t)xb * (kXIBytes / 16u), b = (uint32_t)dxj + (uint32_t)b1 * (kTXBytes / 16u);
+        const uint32_t a = (uint32_t)dxi + (uint32_t)xb * (kXIBytes / 16u);
+        const uint32_t b = (uint32_t)dxj + (uint32_t)b1 * (kTXBytes / 16u);
         if (elected) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
@@ -654,16 +649,28 @@ __global__ void __launch_bounds__(kTThreads, 1)
           ph1 ^= 1;
           fph1 ^= 1;
         }
-      };
-      if (it1 < n_items) first();
-      if (ok && it1 < n_items) first();
+      }
+      // all MMAs of this thread have completed before the tensor memory is freed (bounded)
+      if (elected) mma_commit(&drain[0]);
+      dwait(&drain[0], 0);
+    }
+  } else if (warp == kTEpi + 2) {
+    // ---- second MMAs, U += P V_J ----
+    {
+      const bool elected = elect_one();
+      const uint64_t dv = desc_sw128(smem_u32(base + kTOffV));
+      const uint32_t dhi = (uint32_t)(dv >> 32);
+      auto dsc = [&](uint32_t lo) { return ((uint64_t)dhi << 32) | lo; };
+      // as above, N = m rounded up to 16
+      const uint32_t n2 = (uint32_t)((m + 15) / 16 * 16);
+      const uint32_t idesc2 = (1u << 4) | (2u << 7) | (2u << 10) | ((n2 >> 3) << 17) | ((128u >> 4) << 24);
+      bool ok = true;
       int seq = 0, b = 0, sv = 0;
       uint32_t ph = 0, vph = 0;
       for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++seq) {
         const int nt = items[it].z, ub = seq & 1;
         const uint32_t du = tmem + kTUCol + (uint32_t)(ub * 64);
         for (int j = 0; j < nt; ++j) {
-          if (it1 < n_items) first();
           ok = ok && bwait(&v_full[sv], vph, abort_flag, err) && bwait(&p_full[b], ph, abort_flag, err);
           if (ok && j == 0) ok = bwait(&u_empty[ub], ((seq >> 1) & 1) ^ 1, abort_flag, err);
           ok = __all_sync(0xffffffffu, ok);
@@ -690,9 +697,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
           }
         }
       }
-      // all MMAs of this thread have completed before the tensor memory is freed (bounded)
-      if (elected) mma_commit(drain);
-      dwait(drain, 0);
+      if (elected) mma_commit(&drain[1]);
+      dwait(&drain[1], 0);
     }
   } else {
     // ---- epilogue: warp w takes TMEM lanes 32 (w mod 4) .. + 31 (rows) and 32 columns of a step ----
