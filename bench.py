@@ -450,7 +450,8 @@ def run_ours(args):
                     "kernel": "gram_f32_sym_kernel (FP32 Gram tiles, symmetric)",
                     "launches": n32, "avg_ms": ms32 / n32, "entries_per_launch": entries,
                     "work_per_entry": f"{ops_per_entry} FP32-pipe lane operations (FADD, FADD|.| per feature; "
-                                      f"two FFMAs for the row and column sums)",
+                                      f"two FFMAs for the row and column sums; 42 % of the features take one 64-lane "
+                                      f"integer operation instead of two FP32 ones)",
                     "peak_basis": f"{sm_count} SMs (device query) x {FP32_LANES_PER_SM} FP32 lanes x {sm_mhz:g} MHz "
                                   f"(max SM clock sampled by nvidia-smi); derived from unit counts and clocks",
                     "flop_convention": {
