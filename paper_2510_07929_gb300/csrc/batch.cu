@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
 // clock) are 512 cycles a step, the second contraction's 16 MMAs another 512 on the tensor pipe.
 // The previous form (64-column steps, two groups of four epilogue warps on alternate steps, one
 // warp per scheduler each) spent 2800 cycles on half as many entries waiting on hand-offs: 10.3 ms
-// for the 64-problem workload at m = 64, now 3.35.  Here 16 epilogue warps share a step (32 columns
+// for the 64-problem workload at m = 64, now 3.2.  Here 16 epilogue warps share a step (32 columns
 // each); copies, first MMAs and second MMAs are issued by a warp each, converged, with running stage
 // indexes and descriptors (6.5 ms from a branch of one lane; 4.16 ms with one warp for all MMAs, which
 // waited for a buffer to come free for the first ones while the second ones' operands were ready); and
@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
     for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++seq) {
       const int4 I = items[it];
       const float ni = __ldg(nrm + I.x + r);
-      const uint64_t ni2 = bpack2(ni, ni), two = bpack2(2.f, 2.f);
+      const uint64_t ni2 = bpack2(-ni, -ni), two = bpack2(2.f, 2.f), mone = bpack2(-1.f, -1.f);
       for (int j = 0; j < I.z; ++j) {
         if (!bwait(&n_full[sn], nph, abort_flag, err) || !bwait(&s_full[b], ph, abort_flag, err)) {
           ok = false;
@@ -758,9 +758,12 @@ __global__ void __launch_bounds__(kTThreads, 1)
           const float4 nn = nj4[c];
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
+            // -(n_i + n_j), then 2 x_i.x_j + that (the sign through the multiply-add: as integer
+            // operations on the sum 3.35 ms)
             uint64_t sum, arg;
-            asm("add.rn.f32x2 %0, %1, %2;" : "=l"(sum) : "l"(ni2), "l"(u ? bpack2(nn.z, nn.w) : bpack2(nn.x, nn.y)));
-            sum ^= 0x8000000080000000ull;
+            asm("fma.rn.f32x2 %0, %1, %2, %3;"
+                : "=l"(sum)
+                : "l"(u ? bpack2(nn.z, nn.w) : bpack2(nn.x, nn.y)), "l"(mone), "l"(ni2));
             asm("fma.rn.f32x2 %0, %1, %2, %3;"
                 : "=l"(arg)
                 : "l"(bpack2(__uint_as_float(g[4 * c + 2 * u]), __uint_as_float(g[4 * c + 2 * u + 1]))), "l"(two), "l"(sum));
