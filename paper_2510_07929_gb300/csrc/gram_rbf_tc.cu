@@ -774,6 +774,7 @@ __global__ void __launch_bounds__(kSymThreads, 1)
               }
             }
           }
+          if (w.left == 1) umma_commit(&i_free[ib]);   // the row ends: committed before the last waits below
           umma_commit(&mma_done[b]);
           umma_commit(&stage_free[s]);
         }
@@ -790,8 +791,6 @@ __global__ void __launch_bounds__(kSymThreads, 1)
         }
         fresh = w.next();
         if (fresh && q + 1 < nt) {
-          if (elected) umma_commit(&i_free[ib]);
-          __syncwarp();
           bi += s16;
           if (++ib == nibuf) {
             ib = 0;
