@@ -33,7 +33,6 @@
 // point constants.  Row sums stay in registers over the unit; column sums are reduced across the
 // warp's 32 rows and added with FP64 atomics.  Every wait is bounded; on a timeout the CTA records
 // the error, waits (bounded) for its own copies and MMAs and frees its tensor memory.
-#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -41,6 +40,7 @@
 
 #include <cuda_bf16.h>
 
+#include "ht_units.h"
 #include "kqr_internal.h"
 #include "ptx.cuh"
 
@@ -553,36 +553,18 @@ static cudaError_t ht_prepare(Handle* h) {
   return cudaSuccess;
 }
 
-// Work units.  Symmetric (one vector): (I, run of 64-column tiles from the diagonal on), about 8 per
-// SM but no shorter than 16 tiles while an SM gets that many (a unit's set-up, table and tile I, costs
-// about one tile), longest first.  Rows only: (I, split) with about 8 units per SM; the split's row sums go to
-// its own partial, added in a fixed order.
+// The work list of the one-vector (sym) or of the several-vector products, made at its first use.
 static cudaError_t ht_units(Handle* h, bool sym) {
-  const int k = sym ? 0 : 1;
-  if (h->ht_units[k]) return cudaSuccess;
-  const int T = (int)(h->ldn / kTile), TJ = 2 * T;
-  std::vector<int4> u;
-  if (sym) {
-    int64_t tiles = 0;
-    for (int I = 0; I < T; ++I) tiles += TJ - 2 * I;
-    const int C = (int)std::max<int64_t>(1, (tiles + (int64_t)8 * h->num_sms - 1) / ((int64_t)8 * h->num_sms));
-    const int C1 = (int)std::max<int64_t>(C, std::min<int64_t>(16, (tiles + h->num_sms - 1) / h->num_sms));
-    for (int I = 0; I < T; ++I)
-      for (int j = 2 * I; j < TJ; j += C1) u.push_back(make_int4(I, j, std::min(TJ, j + C1), 0));
-    std::stable_sort(u.begin(), u.end(), [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
-    h->ht_parts = 1;
-  } else {
-    const int64_t want = ((int64_t)8 * h->num_sms + T - 1) / T;
-    const int per = (int)std::max<int64_t>(std::min<int64_t>(8, (int64_t)((TJ * (int64_t)T + h->num_sms - 1) / h->num_sms)),
-                                           (TJ + want - 1) / want);
-    h->ht_parts = (TJ + per - 1) / per;
-    for (int s = 0; s < h->ht_parts; ++s)
-      for (int I = 0; I < T; ++I) u.push_back(make_int4(I, s * per, std::min(TJ, (s + 1) * per), s));
-  }
-  h->ht_units[k] = (int4*)dev_alloc(h, u.size() * sizeof(int4));
-  if (!h->ht_units[k]) return cudaErrorMemoryAllocation;
-  h->ht_nunits[k] = (int)u.size();
-  return cudaMemcpy(h->ht_units[k], u.data(), u.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  Handle::HtWork& w = h->ht_work[sym ? 0 : 1];
+  if (w.units) return cudaSuccess;
+  const int T = (int)(h->ldn / kTile);
+  const HtList l = sym ? ht_list_symmetric(T, h->num_sms) : ht_list_rows(T, h->num_sms);
+  static_assert(sizeof(HtUnit) == sizeof(int4), "the kernel reads a unit as an int4");
+  w.units = (int4*)dev_alloc(h, l.units.size() * sizeof(int4));
+  if (!w.units) return cudaErrorMemoryAllocation;
+  w.n = (int)l.units.size();
+  w.parts = l.parts;
+  return cudaMemcpy(w.units, l.units.data(), l.units.size() * sizeof(int4), cudaMemcpyHostToDevice);
 }
 
 static size_t ht_smem(int katoms, int M) {
@@ -598,10 +580,10 @@ static cudaError_t ht_launch(Handle* h, const float2* vhl, double* out, cudaStre
   if (e != cudaSuccess) return e;
   const double c = kLn2 * std::ldexp(1.0, -33);
   const float c1 = (float)c, c2 = (float)(c - (double)c1);
-  const int k = SYM ? 0 : 1;
+  const Handle::HtWork& w = h->ht_work[SYM ? 0 : 1];
   prof_mark(h, 1, true, st);
-  kern<<<h->ht_nunits[k], kThreadsHt, smem, st>>>(h->tm_ht_i, h->tm_ht_j, h->ht_cst, vhl, h->ht_table, h->ht_units[k],
-                                                  out, h->ldn, c1, c2, h->err_flag);
+  kern<<<w.n, kThreadsHt, smem, st>>>(h->tm_ht_i, h->tm_ht_j, h->ht_cst, vhl, h->ht_table, w.units, out, h->ldn, c1, c2,
+                                      h->err_flag);
   prof_mark(h, 1, false, st);
   h->launches++;
   return cudaGetLastError();
@@ -631,12 +613,13 @@ cudaError_t gram_high_tc(Handle* h, const double* V, double* U, int m, cudaStrea
   const int M = m <= 1 ? 1 : (m <= 2 ? 2 : (m <= 4 ? 4 : 8));
   cudaError_t e = ht_units(h, sym);
   if (e != cudaSuccess) return e;
+  const int parts = h->ht_work[sym ? 0 : 1].parts;
   const size_t vbytes = (size_t)h->ldn * M * sizeof(float2) + (sym ? (size_t)h->ldn * sizeof(double) : 0);
   if ((e = ht_buffer(h, &h->v32, &h->v32_cap, vbytes)) != cudaSuccess) return e;
   float2* vhl = reinterpret_cast<float2*>(h->v32);
   double* acc = reinterpret_cast<double*>(vhl + h->ldn * M);
   if (!sym) {
-    if ((e = ht_buffer(h, &h->part, &h->part_cap, (size_t)h->ht_parts * h->ldn * M * sizeof(double))) != cudaSuccess)
+    if ((e = ht_buffer(h, &h->part, &h->part_cap, (size_t)parts * h->ldn * M * sizeof(double))) != cudaSuccess)
       return e;
     acc = reinterpret_cast<double*>(h->part);
   }
@@ -650,7 +633,7 @@ cudaError_t gram_high_tc(Handle* h, const double* V, double* U, int m, cudaStrea
     default: e = ht_launch<8, false>(h, vhl, acc, st); break;
   }
   if (e != cudaSuccess) return e;
-  ht_finish_kernel<<<grid_for(h->n * m), 256, 0, st>>>(acc, sym ? 1 : h->ht_parts, h->ldn, M, m, h->n, U);
+  ht_finish_kernel<<<grid_for(h->n * m), 256, 0, st>>>(acc, parts, h->ldn, M, m, h->n, U);
   h->launches++;
   return cudaGetLastError();
 }
@@ -659,8 +642,7 @@ void high_tc_free(Handle* h) {
   dev_free(h, h->ht_dig);
   dev_free(h, h->ht_cst);
   dev_free(h, h->ht_table);
-  dev_free(h, h->ht_units[0]);
-  dev_free(h, h->ht_units[1]);
+  for (Handle::HtWork& w : h->ht_work) dev_free(h, w.units);
 }
 
 }  // namespace kqr

@@ -147,15 +147,16 @@ struct Handle {
   int tc16_katoms = 0;
   CUtensorMap tm_tc_a16{}, tm_tc_b16{};
 
-  // FP64-class RBF products on tensor cores (gram_high_tc.cu): digits, point constants, table,
-  // work units (0: symmetric, 1: rows only) and the partial sums the latter need.
+  // FP64-class RBF products on tensor cores (gram_high_tc.cu): digits, point constants, table and
+  // the work lists (0: symmetric, 1: rows only), each with the number of partial sums it writes.
   int ht_state = 0;
   void* ht_dig = nullptr;
   int4* ht_cst = nullptr;
   float2* ht_table = nullptr;
-  int ht_parts = 0;
-  int4* ht_units[2] = {nullptr, nullptr};
-  int ht_nunits[2] = {0, 0};
+  struct HtWork {
+    int4* units = nullptr;
+    int n = 0, parts = 0;
+  } ht_work[2];
   CUtensorMap tm_ht_i{}, tm_ht_j{};
 
   // Symmetric Gram product: work-unit table (row tile, first and end column tile).
