@@ -180,6 +180,18 @@ __device__ __forceinline__ bool bwait(uint64_t* bar, uint32_t parity, volatile i
   return false;
 }
 
+// bwait for a whole converged warp whose lanes act together on the outcome (warp-wide operations on
+// tensor memory): a vote at every poll, so that no lane leaves with another answer than the others.
+__device__ __forceinline__ bool bwait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err) {
+  for (uint32_t i = 0; i < (1u << 22); ++i) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((i & 255u) == 255u && __any_sync(0xffffffffu, *abort_flag)) return false;
+  }
+  *abort_flag = 1;
+  atomicExch(err, 1);
+  return false;
+}
+
 // Drain wait: bounded, ignores the abort flag.
 __device__ __forceinline__ void dwait(uint64_t* bar, uint32_t parity) {
   for (uint32_t i = 0; i < (1u << 22); ++i)
@@ -377,12 +389,10 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
       for (int j = 0; j < I.z; ++j, ++q) {
         if ((q & 1) != grp) continue;
         const int sb = q % kSBufs, vs = q % kVStages, pb = q & 1;
-        if (!bwait(&s_full[sb], (q / kSBufs) & 1, abort_flag, err) ||
-            !bwait(&vl_full[vs], (q / kVStages) & 1, abort_flag, err) ||
-            !bwait(&p_empty[pb], ((q >> 1) & 1) ^ 1, abort_flag, err)) {
-          ok = false;
-          break;
-        }
+        ok = bwait_warp(&s_full[sb], (q / kSBufs) & 1, abort_flag, err) &&
+             bwait_warp(&vl_full[vs], (q / kVStages) & 1, abort_flag, err) &&
+             bwait_warp(&p_empty[pb], ((q >> 1) & 1) ^ 1, abort_flag, err);
+        if (!ok) break;
         fence_after();
         // the step's column norms arrived with V_J (the stage stays until this step's second MMA)
         const float4* nj4 = reinterpret_cast<const float4*>(base + kOffV + vs * kVStride + kVBytes);
@@ -421,7 +431,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
       if (!ok) break;
       if ((q_last & 1) != grp) continue;        // the other group reads this item's result
       const int ub = seq & 1;
-      if (!bwait(&u_full[ub], (seq >> 1) & 1, abort_flag, err)) break;
+      if (!bwait_warp(&u_full[ub], (seq >> 1) & 1, abort_flag, err)) break;
       fence_after();
 #pragma unroll 1
       for (int ch = 0; ch < 2; ++ch) {
@@ -711,11 +721,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
     int pend = -1, pend_it = 0, pend_valid = 0;   // item whose result is still in its accumulator
     auto read_out = [&]() {
       const int ub = pend & 1;
-      if (!bwait(&u_full[ub], (pend >> 1) & 1, abort_flag, err)) {
-        ok = false;
-        return;
-      }
-      __syncwarp();
+      ok = bwait_warp(&u_full[ub], (pend >> 1) & 1, abort_flag, err);
+      if (!ok) return;
       fence_after();
       uint32_t u[16];
       asm volatile(
@@ -742,11 +749,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
       const float ni = __ldg(nrm + I.x + r);
       const uint64_t ni2 = bpack2(-ni, -ni), two = bpack2(2.f, 2.f), mone = bpack2(-1.f, -1.f);
       for (int j = 0; j < I.z; ++j) {
-        if (!bwait(&n_full[sn], nph, abort_flag, err) || !bwait(&s_full[b], ph, abort_flag, err)) {
-          ok = false;
-          break;
-        }
-        __syncwarp();
+        ok = bwait_warp(&n_full[sn], nph, abort_flag, err) && bwait_warp(&s_full[b], ph, abort_flag, err);
+        if (!ok) break;
         fence_after();
         uint32_t g[32];
         const uint32_t cols = tmem + (uint32_t)(b * 128 + cg * 32) + lane_off;

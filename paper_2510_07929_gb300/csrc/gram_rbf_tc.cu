@@ -238,7 +238,8 @@ __global__ void __launch_bounds__(256, 1)
     if (q >= 1) {
       const int pq = q - 1;
       const int b = pq & 1;
-      if (mbar_wait_bounded(&bars[3 + b], (uint32_t)((pq >> 1) & 1), err)) {
+      // the lanes agree on the outcome: the loads from tensor memory are operations of the whole warp
+      if (__all_sync(0xffffffffu, mbar_wait_bounded(&bars[3 + b], (uint32_t)((pq >> 1) & 1), err))) {
         tc_fence_after();
         const uint32_t tbase = tmem + (uint32_t)(b * 128 + half * 64) + ((uint32_t)((warp & 3) * 32) << 16);
         const float* nj = s_nrm + b * 128 + half * 64;
