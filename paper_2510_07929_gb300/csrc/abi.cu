@@ -22,6 +22,18 @@ void dev_free(Handle* h, void* p) {
   else cudaFree(p);
 }
 
+cudaError_t dev_upload(Handle* h, const void* src, size_t bytes, cudaStream_t st, void** out) {
+  *out = dev_alloc(h, bytes);
+  if (!*out) return cudaErrorMemoryAllocation;
+  cudaError_t e = cudaMemcpyAsync(*out, src, bytes, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    dev_free(h, *out);
+    *out = nullptr;
+  }
+  return e;
+}
+
 kqr_status fail(Handle* h, kqr_status s, const std::string& msg) {
   if (h) h->err = msg;
   return s;

@@ -301,7 +301,7 @@ static size_t sym_smem_bytes(int p) {
 
 // Work-unit table: for each row tile I, column tiles [J0, J1) with I <= J0,
 // chunks of C tiles, C chosen for ~64 units per resident CTA.
-cudaError_t sym_units_ensure(Handle* h) {
+cudaError_t sym_units_ensure(Handle* h, cudaStream_t st) {
   const int T = (int)(h->ldn / kTile);
   if (h->sym_units && h->sym_T == T) return cudaSuccess;
   const int64_t pairs = (int64_t)T * (T + 1) / 2;
@@ -312,15 +312,13 @@ cudaError_t sym_units_ensure(Handle* h) {
   for (int I = 0; I < T; ++I)
     for (int J0 = I; J0 < T; J0 += C) u.push_back(make_int4(I, J0, J0 + C < T ? J0 + C : T, 0));
   dev_free(h, h->sym_units);
-  h->sym_units = (int4*)dev_alloc(h, u.size() * sizeof(int4));
-  if (!h->sym_units) return cudaErrorMemoryAllocation;
   h->sym_nunits = (int)u.size();
   h->sym_T = T;
-  return cudaMemcpy(h->sym_units, u.data(), u.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  return dev_upload(h, u.data(), u.size() * sizeof(int4), st, reinterpret_cast<void**>(&h->sym_units));
 }
 
 cudaError_t gram_f32_sym(Handle* h, const double* V, double* U, const GramEpilogue* ep, cudaStream_t st) {
-  cudaError_t e = sym_units_ensure(h);
+  cudaError_t e = sym_units_ensure(h, st);
   if (e != cudaSuccess) return e;
   float* v32;
   double* sums;

@@ -13,7 +13,7 @@
 
 namespace kqr {
 
-cudaError_t sym_units_ensure(Handle* h);
+cudaError_t sym_units_ensure(Handle* h, cudaStream_t st);
 
 constexpr int kTBs = kExpTableBits;
 constexpr float kLn2HiS = 0.693147182464599609375f;
@@ -243,7 +243,7 @@ static size_t high_sym_smem(int p) {
 }
 
 cudaError_t gram_high_sym(Handle* h, const double* V, double* U, cudaStream_t st) {
-  cudaError_t e = sym_units_ensure(h);
+  cudaError_t e = sym_units_ensure(h, st);
   if (e != cudaSuccess) return e;
   const size_t need = (size_t)h->ldn * (sizeof(float2) + sizeof(double));
   if (h->v32_cap < need) {

@@ -554,17 +554,15 @@ static cudaError_t ht_prepare(Handle* h) {
 }
 
 // The work list of the one-vector (sym) or of the several-vector products, made at its first use.
-static cudaError_t ht_units(Handle* h, bool sym) {
+static cudaError_t ht_units(Handle* h, bool sym, cudaStream_t st) {
   Handle::HtWork& w = h->ht_work[sym ? 0 : 1];
   if (w.units) return cudaSuccess;
   const int T = (int)(h->ldn / kTile);
   const HtList l = sym ? ht_list_symmetric(T, h->num_sms) : ht_list_rows(T, h->num_sms);
   static_assert(sizeof(HtUnit) == sizeof(int4), "the kernel reads a unit as an int4");
-  w.units = (int4*)dev_alloc(h, l.units.size() * sizeof(int4));
-  if (!w.units) return cudaErrorMemoryAllocation;
   w.n = (int)l.units.size();
   w.parts = l.parts;
-  return cudaMemcpy(w.units, l.units.data(), l.units.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  return dev_upload(h, l.units.data(), l.units.size() * sizeof(int4), st, reinterpret_cast<void**>(&w.units));
 }
 
 static size_t ht_smem(int katoms, int M) {
@@ -611,7 +609,7 @@ cudaError_t high_tc_ready(Handle* h, bool* ready) {
 cudaError_t gram_high_tc(Handle* h, const double* V, double* U, int m, cudaStream_t st) {
   const bool sym = m == 1;
   const int M = m <= 1 ? 1 : (m <= 2 ? 2 : (m <= 4 ? 4 : 8));
-  cudaError_t e = ht_units(h, sym);
+  cudaError_t e = ht_units(h, sym, st);
   if (e != cudaSuccess) return e;
   const int parts = h->ht_work[sym ? 0 : 1].parts;
   const size_t vbytes = (size_t)h->ldn * M * sizeof(float2) + (sym ? (size_t)h->ldn * sizeof(double) : 0);

@@ -38,6 +38,11 @@ struct GridRdv;
 // ---- device memory ---------------------------------------------------------
 void* dev_alloc(Handle* h, size_t bytes);
 void dev_free(Handle* h, void* p);
+// Copy of a host table in new device memory, made on the stream that will read it and waited for
+// before the host table can go: the handle's and the callers' streams do not wait for the default
+// stream, on which a plain cudaMemcpy of pageable memory may return with its copy still under way.
+// On failure *out is null.
+cudaError_t dev_upload(Handle* h, const void* src, size_t bytes, cudaStream_t st, void** out);
 
 // ---- Gram products (gram_f32.cu, gram_high.cu) ------------------------------
 // Epilogue applied when the per-split partial sums are combined:
