@@ -32,7 +32,8 @@
 // and MMAs.  Two accumulator sets of 256 columns fill tensor memory; three stages of J digits and
 // point constants.  Row sums stay in registers over the unit; column sums are reduced across the
 // warp's 32 rows and added with FP64 atomics.  Every wait is bounded; on a timeout the CTA records
-// the error, waits (bounded) for its own copies and MMAs and frees its tensor memory.
+// the error.  In any case it waits (bounded) for its own copies and MMAs before it frees its tensor
+// memory.
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -307,14 +308,14 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
           join();
         }
       }
-      if (!ok) {
-        // a wait gave up: let this CTA's own copies and MMAs finish (bounded)
-        *abort_flag = 1;
-        mbar_wait_bounded(full_i, 0, err);
-        for (int q = loaded > kStages ? loaded - kStages : 0; q < loaded; ++q)
-          mbar_wait_bounded(&full_j[q % kStages], (uint32_t)((q / kStages) & 1), err);
-        if (issued > 0) mbar_wait_bounded(&mma_done[(issued - 1) & 1], (uint32_t)(((issued - 1) >> 1) & 1), err);
-      }
+      if (!ok) *abort_flag = 1;
+      // The CTA does not free its tensor memory or exit with a copy or an MMA of its own in flight, also
+      // when it was an epilogue warp that gave up, after the last tile was issued (bounded waits, done
+      // already when nothing went wrong).
+      mbar_wait_bounded(full_i, 0, err);
+      for (int q = loaded > kStages ? loaded - kStages : 0; q < loaded; ++q)
+        mbar_wait_bounded(&full_j[q % kStages], (uint32_t)((q / kStages) & 1), err);
+      if (issued > 0) mbar_wait_bounded(&mma_done[(issued - 1) & 1], (uint32_t)(((issued - 1) >> 1) & 1), err);
     }
   } else {
     const int lq = warp & 3, cg = warp >> 2;
