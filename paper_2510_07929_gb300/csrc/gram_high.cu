@@ -520,7 +520,7 @@ static size_t lap_high_smem(int p) {
 cudaError_t gram_high(Handle* h, const double* V, double* U, int m, cudaStream_t st) {
   if (m == 1 && h->kind == KQR_LAPLACIAN && h->opt.symmetric_gram) return gram_high_sym(h, V, U, st);
   bool tc = false;
-  cudaError_t te = high_tc_ready(h, &tc);
+  cudaError_t te = high_tc_ready(h, m, st, &tc);
   if (te != cudaSuccess) return te;
   if (tc) return gram_high_tc(h, V, U, m, st);
   const int row_tiles = (int)(h->ldn / kTile), col_tiles = row_tiles;

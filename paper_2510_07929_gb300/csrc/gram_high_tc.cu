@@ -501,7 +501,8 @@ __global__ void ht_finish_kernel(const double* __restrict__ part, int parts, int
 bool make_tmap_2d_f32_sw128(CUtensorMap* tm, void* base, int64_t inner, int64_t outer, int64_t row_bytes,
                             int box_inner, int box_outer);
 
-// Once per problem; h->ht_state: 0 not prepared, 1 ready, -1 this problem keeps the CUDA-core kernels.
+// Once per problem; h->ht_state: 0 not prepared, 1 ready, -1 this problem keeps the CUDA-core kernels
+// (norms too large, or no memory for the digits: 256 or 512 bytes a row that those kernels do without).
 static cudaError_t ht_prepare(Handle* h) {
   if (h->ht_state) return cudaSuccess;
   const int kf = h->p <= 16 ? 16 : 32;
@@ -547,6 +548,10 @@ static cudaError_t ht_prepare(Handle* h) {
     h->ht_dig = nullptr;
     h->ht_cst = nullptr;
     h->ht_table = nullptr;
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      e = cudaSuccess;
+    }
     if (e == cudaSuccess) h->ht_state = -1;
     return e;
   }
@@ -596,32 +601,44 @@ static cudaError_t ht_buffer(Handle* h, float** buf, size_t* cap, size_t bytes) 
   return *buf ? cudaSuccess : cudaErrorMemoryAllocation;
 }
 
-// Whether the tensor-core product serves this problem: RBF, p <= 32, norms below 28 (kernel values
-// against the data's mean above 2^-28), and options.symmetric_gram and rbf_tensor_cores on.  Anything
-// else keeps the CUDA-core kernels of gram_high.cu.
-cudaError_t high_tc_ready(Handle* h, bool* ready) {
+// Scratch of the product of m vectors: the FP32 pairs of V (and, for one vector, the sums) in v32, the
+// partial sums of several in part.
+static cudaError_t ht_scratch(Handle* h, int m, int M, cudaStream_t st) {
+  const bool sym = m == 1;
+  cudaError_t e = ht_units(h, sym, st);
+  if (e != cudaSuccess) return e;
+  const size_t vbytes = (size_t)h->ldn * M * sizeof(float2) + (sym ? (size_t)h->ldn * sizeof(double) : 0);
+  if ((e = ht_buffer(h, &h->v32, &h->v32_cap, vbytes)) != cudaSuccess || sym) return e;
+  return ht_buffer(h, &h->part, &h->part_cap, (size_t)h->ht_work[1].parts * h->ldn * M * sizeof(double));
+}
+
+static int ht_columns(int m) { return m <= 1 ? 1 : (m <= 2 ? 2 : (m <= 4 ? 4 : 8)); }
+
+// Whether the tensor-core product of m vectors serves this problem: RBF, p <= 32, norms below 28
+// (kernel values against the data's mean above 2^-28), options.symmetric_gram and rbf_tensor_cores on,
+// and memory for its layout and scratch, which are made here.  Anything else keeps the CUDA-core
+// kernels of gram_high.cu, which need less memory.
+cudaError_t high_tc_ready(Handle* h, int m, cudaStream_t st, bool* ready) {
   *ready = false;
   if (h->kind != KQR_RBF || h->p > 32 || !h->opt.symmetric_gram || !h->opt.rbf_tensor_cores) return cudaSuccess;
-  const cudaError_t e = ht_prepare(h);
-  *ready = e == cudaSuccess && h->ht_state > 0;
+  cudaError_t e = ht_prepare(h);
+  if (e != cudaSuccess || h->ht_state < 0) return e;
+  e = ht_scratch(h, m, ht_columns(m), st);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return cudaSuccess;
+  }
+  *ready = e == cudaSuccess;
   return e;
 }
 
+// After high_tc_ready(h, m, ...) said so.
 cudaError_t gram_high_tc(Handle* h, const double* V, double* U, int m, cudaStream_t st) {
   const bool sym = m == 1;
-  const int M = m <= 1 ? 1 : (m <= 2 ? 2 : (m <= 4 ? 4 : 8));
-  cudaError_t e = ht_units(h, sym, st);
-  if (e != cudaSuccess) return e;
-  const int parts = h->ht_work[sym ? 0 : 1].parts;
-  const size_t vbytes = (size_t)h->ldn * M * sizeof(float2) + (sym ? (size_t)h->ldn * sizeof(double) : 0);
-  if ((e = ht_buffer(h, &h->v32, &h->v32_cap, vbytes)) != cudaSuccess) return e;
+  const int M = ht_columns(m), parts = h->ht_work[sym ? 0 : 1].parts;
+  cudaError_t e;
   float2* vhl = reinterpret_cast<float2*>(h->v32);
-  double* acc = reinterpret_cast<double*>(vhl + h->ldn * M);
-  if (!sym) {
-    if ((e = ht_buffer(h, &h->part, &h->part_cap, (size_t)parts * h->ldn * M * sizeof(double))) != cudaSuccess)
-      return e;
-    acc = reinterpret_cast<double*>(h->part);
-  }
+  double* acc = sym ? reinterpret_cast<double*>(vhl + h->ldn * M) : reinterpret_cast<double*>(h->part);
   ht_split_kernel<<<grid_for(h->ldn * M), 256, 0, st>>>(V, vhl, sym ? acc : nullptr, h->n, h->ldn, m, M);
   h->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -78,8 +78,9 @@ cudaError_t sym_finish(Handle* h, const void* acc, bool f64, double* U, const Gr
 cudaError_t gram_high(Handle* h, const double* V, double* U, int m, cudaStream_t st);
 // Laplacian m = 1 FP64-class product with each off-diagonal tile formed once (gram_high_sym.cu).
 cudaError_t gram_high_sym(Handle* h, const double* V, double* U, cudaStream_t st);
-// RBF FP64-class products with the cross term on tcgen05 (gram_high_tc.cu).
-cudaError_t high_tc_ready(Handle* h, bool* ready);
+// RBF FP64-class products with the cross term on tcgen05 (gram_high_tc.cu): whether they serve m
+// vectors of this problem (their buffers are made on the way), and the product itself.
+cudaError_t high_tc_ready(Handle* h, int m, cudaStream_t st, bool* ready);
 cudaError_t gram_high_tc(Handle* h, const double* V, double* U, int m, cudaStream_t st);
 void high_tc_free(Handle* h);
 // Stored-K product (gram_stored.cu): kstore_setup fills the packed upper-triangle tiles
