@@ -212,6 +212,7 @@ static kqr_status adjoint_cg(Handle* h, const double* L, const double* Lpre, dou
   a.Lpre = Lpre;
   a.gam = gam;
   a.x = x;
+  a.unit_first = false;
   for (;;) {
     for (int j = 0; j < kAdjointBlock; ++j) {
       AK(gram_high(h, vec(h, V_P), vec(h, V_KP), 1, st));

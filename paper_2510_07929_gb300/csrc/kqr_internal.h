@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/kqr.h"
+#include "cg_rule.h"
 
 namespace kqr {
 
@@ -305,8 +306,6 @@ kqr_status kkt(Handle* h, const double* alpha, const double* v, double beta, con
 // other terms, the device-resident step lengths and stopping test, the preconditioner and
 // the direction update (solver.cu).  Used by the grid's shared CG engine (grid.cu), which
 // runs the products of several columns together and this chain on each column's stream.
-// CG status (S_CGST): running, met tol, stopped at a non-positive curvature, non-finite, maxit.
-enum CgState { CG_RUN = 0, CG_MET = 1, CG_TRUNC = 2, CG_NONFINITE = 3, CG_MAXIT = 4 };
 struct CgArgs {
   const double* L = nullptr;
   const double* Lpre = nullptr;
@@ -314,6 +313,7 @@ struct CgArgs {
   double* x = nullptr;
   double* Kx = nullptr;
   double noise_coef = 0.0;
+  bool unit_first = true;   // a first curvature at the rounding level: step 1 along the direction, or 0 (cg_rule.h)
 };
 cudaError_t cg_after_product(Handle* h, const CgArgs& a, cudaStream_t st);
 // Start of a CG on the residual in vec(h, V_R) with ||r||^2 in S_RR: preconditioned direction, its sum and

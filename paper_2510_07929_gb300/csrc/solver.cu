@@ -88,7 +88,7 @@ static cudaError_t cg_operator(Handle* h, double* Ap, const double* Kp, const do
 // 0 running, 1 met tol, 2 stopped at a non-positive curvature, 3 non-finite, 4 maxit.
 // One CG step after p^T A p is known: the step length a = rz / pAp (rz in S_RZN), or the
 // truncation step when the curvature is at or below the product's rounding level
-// (noise_coef: that level per unit ||p||^2, 2^-22 sqrt(n) for FP32 entries and sums);
+// (noise_coef: that level per unit ||p||^2, 2^-22 sqrt(n) for FP32 entries and sums; cg_rule.h);
 // x += a p, Kx += a Kp, r -= a Ap; then, in the CTA that finishes last, ||r||^2, the
 // iteration count, rz copied to S_RZ for the next direction, and the status
 // (0 running, 1 met tol, 2 rounding-level curvature, 3 non-finite, 4 maxit).  A stopped CG
@@ -96,30 +96,15 @@ static cudaError_t cg_operator(Handle* h, double* Ap, const double* Kp, const do
 // The new residual is also left split for the Woodbury apply (w; scaled by the exponent of the
 // previous ||r||, which every CTA reads before the last one overwrites it), so that the apply
 // needs no pass of its own.
-__global__ void __launch_bounds__(256) cg_step_kernel(double* __restrict__ s, double noise_coef, double* __restrict__ x,
-                                                      double* __restrict__ Kx, double* __restrict__ r,
+__global__ void __launch_bounds__(256) cg_step_kernel(double* __restrict__ s, double noise_coef, int unit_first,
+                                                      double* __restrict__ x, double* __restrict__ Kx, double* __restrict__ r,
                                                       const double* __restrict__ p, const double* __restrict__ Kp,
                                                       const double* __restrict__ Ap, int64_t n, WbSplit w,
                                                       double* __restrict__ part, unsigned int* __restrict__ counter) {
   if ((int)s[S_CGST] != CG_RUN) return;
-  const double pAp = s[S_PAP];
-  double a;
-  int pend;
-  if (!isfinite(pAp)) {
-    a = 0.0;
-    pend = CG_NONFINITE;
-  } else if (!(pAp > 4.0 * noise_coef * s[S_PP])) {
-    // The operator is positive definite; a curvature at or below the product's
-    // rounding level is rounding in directions whose eigenvalues lie below its
-    // accuracy (a numerically low-rank K), and dividing by it would blow the step
-    // up.  Truncate: keep x, or at the first step take the preconditioned residual
-    // itself (a Newton step with the preconditioner as the Hessian model).
-    a = s[S_CGITS] == 0.0 ? 1.0 : 0.0;
-    pend = CG_TRUNC;
-  } else {
-    a = s[S_RZN] / pAp;
-    pend = CG_RUN;
-  }
+  const CgStep step =
+      cg_step_rule(s[S_PAP], 4.0 * noise_coef * s[S_PP], s[S_RZN], s[S_CGITS] == 0.0, unit_first != 0);
+  const double a = step.a;
   const int e = norm_exponent(s[S_RR], false);
   const double sr = pow2(-e);
   const double sw = w.us ? pow2(-max_exponent(*reinterpret_cast<const unsigned long long*>(s + S_WMAX))) : 0.0;
@@ -145,7 +130,7 @@ __global__ void __launch_bounds__(256) cg_step_kernel(double* __restrict__ s, do
   s[S_A] = a;
   s[S_RZ] = s[S_RZN];
   if (a != 0.0) s[S_CGITS] += 1.0;
-  int st = pend;
+  int st = step.state;
   if (st == CG_RUN) {
     if (!isfinite(rr)) st = CG_NONFINITE;
     else if (rr <= s[S_TOL2]) st = CG_MET;
@@ -184,10 +169,10 @@ __global__ void __launch_bounds__(256) cg_dir_kernel(double* __restrict__ s, dou
   }
 }
 
-static cudaError_t cg_step(Handle* h, double noise_coef, double* x, double* Kx, double* r, const double* p,
+static cudaError_t cg_step(Handle* h, double noise_coef, bool unit_first, double* x, double* Kx, double* r, const double* p,
                            const double* Kp, const double* Ap, cudaStream_t st) {
-  cg_step_kernel<<<grid_for(h->n, 256, 304), 256, 0, st>>>(h->scal, noise_coef, x, Kx, r, p, Kp, Ap, h->n,
-                                                           precond_split(h), h->red_part, h->red_counter);
+  cg_step_kernel<<<grid_for(h->n, 256, 304), 256, 0, st>>>(h->scal, noise_coef, unit_first ? 1 : 0, x, Kx, r, p, Kp, Ap,
+                                                           h->n, precond_split(h), h->red_part, h->red_counter);
   h->launches++;
   return cudaGetLastError();
 }
@@ -225,7 +210,7 @@ cudaError_t cg_after_product(Handle* h, const CgArgs& a, cudaStream_t st) {
   double* Kp = vec(h, V_KP);
   cudaError_t e = cg_operator(h, Ap, Kp, p, a.L, st);
   if (e != cudaSuccess) return e;
-  if ((e = cg_step(h, a.noise_coef, a.x, a.Kx, r, p, Kp, Ap, st)) != cudaSuccess) return e;
+  if ((e = cg_step(h, a.noise_coef, a.unit_first, a.x, a.Kx, r, p, Kp, Ap, st)) != cudaSuccess) return e;
   if ((e = precond_apply(h, a.Lpre, r, zz, s + S_RZN, st, s + S_RR, true)) != cudaSuccess) return e;
   return cg_dir(h, p, zz, nullptr, nullptr, st);
 }
@@ -311,7 +296,7 @@ kqr_status pcg(Handle* h, const double* L, const double* Lpre, double gam, const
       } else if (lowprec) e = gram_rbf_tc(h, p, Ap, 1, false, &ep, st);
       else e = gram_f32(h, p, Ap, 1, &ep, st);
       if (e != cudaSuccess) break;
-      if ((e = cg_step(h, noise_coef, x, Kx, r, p, Kp, Ap, st)) != cudaSuccess) break;
+      if ((e = cg_step(h, noise_coef, true, x, Kx, r, p, Kp, Ap, st)) != cudaSuccess) break;
       if ((e = precond_apply(h, Lpre, r, zz, s + S_RZN, st, s + S_RR, true)) != cudaSuccess) break;
       e = cg_dir(h, p, zz, v32, acc, st);
     }
