@@ -135,7 +135,8 @@ typedef struct kqr_options {
   int32_t phase1_only;           /* 1: stop after Phase I (for tests of Alg. 1) */
   int32_t symmetric_gram;        /* 1: single-vector products (FP32, FP64-class Laplacian, FP64-class RBF with p <= 32) form each off-diagonal tile once and
                                     use it for both K_IJ v_J and K_IJ^T v_I (n(n+1)/2 entries; summation
-                                    order not fixed); 0: every entry formed (deterministic) */
+                                    order not fixed, except the FP64-class RBF product's, whose sums do not
+                                    depend on the order); 0: every entry formed (deterministic) */
   int32_t rbf_tensor_cores;      /* 1: RBF FP32 products on tcgen05 (three TF32 terms); 0: FP32 CUDA cores */
   int32_t cg_tf32;               /* RBF only, 1: CG products in TF32 on tcgen05 (one term), each linear solve
                                     iteratively refined against FP32 residuals to the same tolerance */

@@ -23,7 +23,7 @@
 // 40 instructions per MMA among 16 busy warps and made the MMAs the bound).  For one vector each
 // off-diagonal tile serves its rows and its columns (n(n+1)/2 entries); for several, an entry is formed
 // once per pass over K and added to every vector's row sums.  Measured: one vector, n = 50000, p = 20:
-// 3.79 ms, before 20.9 ms; eight vectors, n = 10007, p = 8: 0.62 ms, before
+// 3.86 ms (3.80 with plain atomics, whose results differed from run to run), before 20.9 ms; eight vectors, n = 10007, p = 8: 0.62 ms, before
 // 4.38 ms.  Before: int64 sums of squared differences on the CUDA cores (6 operations per entry and
 // feature, all n^2 entries, columns one after another).
 //
@@ -31,7 +31,8 @@
 // tile I, columns 16 (w / 4) .. + 15 of the 64-column tile J), lane 0 of warp 16 issues TMA copies
 // and MMAs.  Two accumulator sets of 256 columns fill tensor memory; three stages of J digits and
 // point constants.  Row sums stay in registers over the unit; column sums are reduced across the
-// warp's 32 rows and added with FP64 atomics.  Every wait is bounded; on a timeout the CTA records
+// warp's 32 rows.  For one vector both go to the result by atomics whose sums do not depend on their
+// order (OrderFree below), so that the product is the same in every run.  Every wait is bounded; on a timeout the CTA records
 // the error.  In any case it waits (bounded) for its own copies and MMAs before it frees its tensor
 // memory.
 #include <cmath>
@@ -145,6 +146,14 @@ __device__ __forceinline__ void ht_add(float& sh, float& sl, float yh, float yl)
   sh = s;
   sl = __fadd_rn(sl, __fadd_rn(er, yl));
 }
+// The same with the lows added to one another first: swapping the operands gives the same bits.
+__device__ __forceinline__ void ht_add_even(float& sh, float& sl, float yh, float yl) {
+  const float s = __fadd_rn(sh, yh);
+  const float bb = __fsub_rn(s, sh);
+  const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(yh, bb));
+  sh = s;
+  sl = __fadd_rn(__fadd_rn(sl, yl), er);
+}
 // (ph, pl) = (kh + kl) (vh + vl)
 __device__ __forceinline__ void ht_mul(float kh, float kl, float vh, float vl, float& ph, float& pl) {
   ph = __fmul_rn(kh, vh);
@@ -161,10 +170,11 @@ struct EntryConst {
   float c1, c2;        // ln2 2^-33 as hi + lo
 };
 
-// The entry from its four cross-term sums; ci, cj: point constants (see ht_prep_kernel).
+// The entry from its four cross-term sums, times the power of two with the bits `one`; ci, cj: point
+// constants (see ht_prep_kernel).
 __device__ __forceinline__ void ht_entry(float ga, float gb, float gc, float gd, int ni, int nj, int fi, int fj,
-                                         float li, float lj, EntryConst ec, const unsigned char* tab, float& kh,
-                                         float& kl) {
+                                         float li, float lj, EntryConst ec, int one, const unsigned char* tab,
+                                         float& kh, float& kl) {
   const int ta = __float2int_rn(ga);                       // 2 x cross term, units of 2^-19
   const int tb = __float2int_rn(gb * 16384.f);             // 2 x cross term, units of 2^-33
   const float u = __fadd_rn(gc, kMagicC);                  // gc rounded to a cross term of 2^-34
@@ -174,7 +184,7 @@ __device__ __forceinline__ void ht_entry(float ga, float gb, float gc, float gd,
   const int T = (ni + nj - ta) + (J >> 14);                // units of 2^-19
   const float rem = __fsub_rn(__int_as_float((((T & 127) << 14) + 0x4B000000) | (J & 0x3fff)), 8388608.f);
   const float2 t = *reinterpret_cast<const float2*>(tab + ((T >> 4) & 0x7ff8));
-  const float sc = __int_as_float(0x3F800000 - (T & (int)0xfff80000) * 16);
+  const float sc = __int_as_float(one - (T & (int)0xfff80000) * 16);
   // 2^-(rem 2^-33) e^-w = 1 - y, y = x + ...
   const float x = __fmul_rn(rem, ec.c1);
   float e = fmaf(rem, ec.c1, -x);
@@ -192,17 +202,74 @@ __device__ __forceinline__ void ht_entry(float ga, float gb, float gc, float gd,
   kl = __fmul_rn(l, sc);
 }
 
+// Sums that come out the same whatever the order of their atomics.  An addend a is cut on fixed grids:
+// h1, a multiple of g1 = 2^(e0 - 52), h2 of g2, ..., each plane collecting its own.  2^e0 bounds
+// sum_j |K_ij v_j| (from n max |v|), so every partial sum of the h1 is a multiple of g1 below 2^53 g1:
+// exact, hence without an order.  What the first cut leaves of an addend is below g1; with 2^(la - 1) of
+// them the sums of the rest stay below 2^(e2 - 1), e2 = e0 - 52 + la, and the second grid is
+// g2 = 2^(e2 - 52); the later cuts leave half a step, so the grids then lie 53 - la bits apart.
+// Entries go down to 2^-112, addends carry 48 bits: four planes lose nothing that the addends carry.
+//
+// The first cut clears mantissa bits (FP64 operations have a latency of 65 cycles, and a warp would
+// wait for two more).  An addend of 2^e2 and more ends on the second grid by itself, its last bit being
+// at least 2^(e2 - 52): two atomics, one FP64 subtraction.  Smaller ones, by a vote of the warp, are cut
+// further.
+//
+// The entries are formed times 2^k, k such that max |v| 2^k comes to 2^60 (0 <= k <= 120), which costs
+// nothing (it is part of the entry's exponent) and keeps entry times vector inside the FP32 range down
+// to the smallest entries; the finishing kernel takes the factor out.
+// Layout: planes 0 and 1 of element i at [2 i], [2 i + 1], planes 2 and 3 the same way 2 ldn further.
+constexpr int kPlanes = 4;
+struct OrderFree {
+  int e0, e2, k, la;
+  __device__ __forceinline__ OrderFree(unsigned long long vmax, int log2n, int la_) : la(la_) {
+    const int field = (int)(vmax >> 52);
+    const int ex = field > 0 ? field - 1022 : 0;         // max |v| < 2^ex (below 2^-1022 it is zero in FP32)
+    k = min(120, max(0, 60 - ex));
+    e0 = ex + k + log2n + 1;
+    e2 = e0 - 52 + la;
+  }
+  // a rounded towards zero to a multiple of g1
+  __device__ __forceinline__ double first(double a) const {
+    const int t = min(63, max(0, e0 + 1023 - ((__double2hiint(a) >> 20) & 0x7ff)));
+    return __longlong_as_double(__double_as_longlong(a) & (t > 52 ? 0ll : -1ll << t));
+  }
+  // a is zero or not below 2^e2
+  __device__ __forceinline__ bool two_planes(double a) const {
+    const int hi = __double2hiint(a) & 0x7fffffff;
+    return hi == 0 || hi >= (e2 + 1023) << 20;
+  }
+  static __device__ __forceinline__ double power(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+  // a rounded to the grid of m = 1.5 2^e; r: the rest, exact
+  static __device__ __forceinline__ double cut(double a, double m, double& r) {
+    const double h = __dsub_rn(__dadd_rn(a, m), m);
+    r = __dsub_rn(a, h);
+    return h;
+  }
+  // the second to fourth plane of what the first cut left; p: the element of the second
+  static __device__ __noinline__ void rest(double* p, int64_t ldn, double r1, int e2, int la) {
+    double r2, r3, r4;
+    const double m2 = 1.5 * power(e2), step = power(la - 53);
+    atomicAdd(p, cut(r1, m2, r2));
+    atomicAdd(p + 2 * ldn - 1, cut(r2, m2 * step, r3));
+    atomicAdd(p + 2 * ldn, cut(r3, m2 * step * step, r4));
+  }
+};
+
 }  // namespace
 
 // units[b] = {row tile I, first and end 64-column tile, partial index}.  SYM (M = 1): each unit's
-// tiles start at or right of the diagonal, results into out[ldn] with atomics; else row sums over
-// the unit's columns into out[partial][ldn][M].
+// tiles start at or right of the diagonal, results into the kPlanes planes of out with atomics
+// (vmax[0]: bits of max |v|, vmax[1] receives those of 2^-k; log2n, la: base-2 logarithms, rounded up, of
+// n and of twice the addends of an element); else row sums over the unit's columns into
+// out[partial][ldn][M].
 template <int M, bool SYM, int KS>
 __global__ void __launch_bounds__(kThreadsHt, 1)
     gram_rbf_high_tc_kernel(const __grid_constant__ CUtensorMap tm_i, const __grid_constant__ CUtensorMap tm_j,
                             const int4* __restrict__ cst, const float2* __restrict__ vhl,
                             const float2* __restrict__ table, const int4* __restrict__ units, double* __restrict__ out,
-                            int64_t ldn, float c1, float c2, int* __restrict__ err) {
+                            int64_t ldn, float c1, float c2, unsigned long long* __restrict__ vmax, int log2n, int la,
+                            int* __restrict__ err) {
   constexpr int katoms = KS == 1 ? 2 : 4;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -252,7 +319,7 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
 
   if (warp == kEpiWarps) {
     // Copies and MMAs.  M = 1: the warp stays converged, so that indexes and descriptors are uniform
-    // values, and one elected lane issues (n = 50000: 3.79 ms, 4.32 with a branch of one lane); with
+    // values, and one elected lane issues (n = 50000: 3.79 ms then, 4.32 with a branch of one lane); with
     // several vectors one lane does it all, which measured faster (M = 8, n = 10007: 0.62 against 0.64).
     constexpr bool kConverged = M == 1;
     if (kConverged || lane == 0) {
@@ -325,6 +392,9 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
     float2 vi = make_float2(0.f, 0.f);
     if (SYM) vi = vhl[i];
     const EntryConst ec{c1, c2};
+    const OrderFree sums(SYM ? *vmax : 0ull, log2n, la);
+    const int one = SYM ? 0x3F800000 + (sums.k << 23) : 0x3F800000;
+    if (SYM && blockIdx.x == 0 && tid == 0) vmax[1] = (unsigned long long)(1023 - sums.k) << 52;
     float sh[M], sl[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) sh[m] = sl[m] = 0.f;
@@ -344,6 +414,7 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
       const int j0 = (jt0 + q) * kJCols + cg * 16;
       auto halves = [&](auto diag_tag) {
         constexpr bool DIAG = decltype(diag_tag)::value;
+        float c0h = 0.f, c0l = 0.f;   // column sums of the first half
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
           uint32_t g[4][8];
@@ -362,7 +433,7 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
             const int4 k = cj[h * 8 + c];
             float kh, kl;
             ht_entry(__uint_as_float(g[0][c]), __uint_as_float(g[1][c]), __uint_as_float(g[2][c]),
-                     __uint_as_float(g[3][c]), ci.x, k.x, ci.y, k.y, li, __int_as_float(k.z), ec, tab, kh, kl);
+                     __uint_as_float(g[3][c]), ci.x, k.x, ci.y, k.y, li, __int_as_float(k.z), ec, one, tab, kh, kl);
             if (DIAG && j0 + h * 8 + c < i) kh = kl = 0.f;   // the entry belongs to its mirror image
 #pragma unroll
             for (int m = 0; m < M; ++m) {
@@ -400,13 +471,25 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
                 ht_add(ch[c], cl[c], gh, gl);
               }
             }
-#pragma unroll
-            for (int o = 2; o >= 1; o >>= 1) {
-              const float gh = __shfl_xor_sync(0xffffffffu, ch[0], o);
-              const float gl = __shfl_xor_sync(0xffffffffu, cl[0], o);
-              ht_add(ch[0], cl[0], gh, gl);
+            // The first half waits for the second: lane bit 1 selects the half, bit 0 the plane, so that 16
+            // columns go out in one operation of 32 lanes.  Both lanes of a pair end with the same bits.
+            if (h == 0) {
+              c0h = ch[0];
+              c0l = cl[0];
+            } else {
+              const bool up = (lane & 2) != 0;
+              const float gh = __shfl_xor_sync(0xffffffffu, up ? c0h : ch[0], 2);
+              const float gl = __shfl_xor_sync(0xffffffffu, up ? c0l : cl[0], 2);
+              float sh2 = up ? ch[0] : c0h, sl2 = up ? cl[0] : c0l;
+              ht_add(sh2, sl2, gh, gl);
+              ht_add_even(sh2, sl2, __shfl_xor_sync(0xffffffffu, sh2, 1), __shfl_xor_sync(0xffffffffu, sl2, 1));
+              const double a = (double)sh2 + (double)sl2;
+              const double h1 = sums.first(a), r1 = __dsub_rn(a, h1);
+              const bool rest = (lane & 1) != 0;
+              double* p = out + 2 * (j0 + (up ? 8 : 0) + (lane >> 2)) + (lane & 1);
+              if (__all_sync(0xffffffffu, sums.two_planes(a)) || !rest) atomicAdd(p, rest ? r1 : h1);
+              else OrderFree::rest(p, ldn, r1, sums.e2, sums.la);
             }
-            if ((lane & 3) == 0) atomicAdd(out + j0 + h * 8 + (lane >> 2), (double)ch[0] + (double)cl[0]);
           }
         }
       };
@@ -424,8 +507,12 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
     if (*abort_flag == 0) {
       for (int e = tid; e < 128 * M; e += kEpiWarps * 32) {
         const double v = (red[e] + red[128 * M + e]) + (red[2 * 128 * M + e] + red[3 * 128 * M + e]);
-        if (SYM) atomicAdd(out + ti * 128 + e, v);
-        else out[((size_t)unit.w * ldn + ti * 128) * M + e] = v;
+        if (SYM) {
+          double* p = out + 2 * (ti * 128 + e);
+          const double h1 = sums.first(v);
+          atomicAdd(p, h1);
+          OrderFree::rest(p + 1, ldn, __dsub_rn(v, h1), sums.e2, sums.la);
+        } else out[((size_t)unit.w * ldn + ti * 128) * M + e] = v;
       }
     }
   }
@@ -473,28 +560,43 @@ __global__ void ht_prep_kernel(const double* __restrict__ xc, int64_t ldn, int p
   }
 }
 
-// V (n x m) -> (hi, lo) floats [ldn][M], zero padded; acc [ldn] zeroed (nullable).
-__global__ void ht_split_kernel(const double* __restrict__ V, float2* __restrict__ out, double* __restrict__ acc,
-                                int64_t n, int64_t ldn, int m, int M) {
+// V (n x m) -> (hi, lo) floats [ldn][M], zero padded.  One vector: the planes of the sums zeroed, and
+// the bits of max |v| into *vmax (zero before; NaN orders above all).
+__global__ void __launch_bounds__(256) ht_split_kernel(const double* __restrict__ V, float2* __restrict__ out,
+                                                       double* __restrict__ acc, int64_t n, int64_t ldn, int m, int M,
+                                                       unsigned long long* __restrict__ vmax) {
+  unsigned long long mx = 0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ldn * M; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / M;
     const int c = (int)(e % M);
     const double x = (i < n && c < m) ? V[i * m + c] : 0.0;
     const float hi = (float)x;
     out[e] = make_float2(hi, (float)(x - (double)hi));
-    if (acc && c == 0) acc[i] = 0.0;
+    if (acc) {
+#pragma unroll
+      for (int k = 0; k < kPlanes; ++k) acc[k * ldn + i] = 0.0;
+      mx = max(mx, (unsigned long long)__double_as_longlong(fabs(x)));
+    }
   }
+  if (!acc) return;
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0 && mx) atomicMax(vmax, mx);
 }
 
-// out[i][c] = sum over the partials (M = 1 and one partial: a copy).
+// out[i][c] = sum over the partials.  One vector (vmax not null): they are the planes, added from the
+// finest on, times vmax[1]; vmax[0] goes back to zero for the next product.
 __global__ void ht_finish_kernel(const double* __restrict__ part, int parts, int64_t ldn, int M, int m, int64_t n,
-                                 double* __restrict__ out) {
+                                 double* __restrict__ out, unsigned long long* __restrict__ vmax) {
+  if (vmax && blockIdx.x == 0 && threadIdx.x == 0) *vmax = 0ull;
+  const double unscale = vmax ? __longlong_as_double((long long)vmax[1]) : 1.0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * m; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / m;
     const int c = (int)(e % m);
     double s = 0.0;
-    for (int q = 0; q < parts; ++q) s += part[((size_t)q * ldn + i) * M + c];
-    out[e] = s;
+    if (vmax) s = ((part[2 * (ldn + i) + 1] + part[2 * (ldn + i)]) + part[2 * i + 1]) + part[2 * i];
+    else
+      for (int q = 0; q < parts; ++q) s += part[((size_t)q * ldn + i) * M + c];
+    out[e] = s * unscale;
   }
 }
 
@@ -576,6 +678,18 @@ static size_t ht_smem(int katoms, int M) {
          (1 + 2 * kStages + 4) * 8 + 16;
 }
 
+static unsigned long long* ht_vmax(Handle* h) { return reinterpret_cast<unsigned long long*>(h->scal + S_HTMAX); }
+
+static int log2_up(int64_t x) {
+  int k = 0;
+  while (((int64_t)1 << k) < x) ++k;
+  return k;
+}
+
+// Addends that an element of the one-vector sums gets at most: four warps' column sums from every row
+// tile above, and one from each unit of its own row tile (at most one per column tile).
+static int64_t ht_addends(const Handle* h) { return 6 * (h->ldn / kTile) + 8; }
+
 template <int M, bool SYM>
 static cudaError_t ht_launch(Handle* h, const float2* vhl, double* out, cudaStream_t st) {
   const size_t smem = ht_smem(h->p <= 16 ? 2 : 4, M);
@@ -587,7 +701,7 @@ static cudaError_t ht_launch(Handle* h, const float2* vhl, double* out, cudaStre
   const Handle::HtWork& w = h->ht_work[SYM ? 0 : 1];
   prof_mark(h, 1, true, st);
   kern<<<w.n, kThreadsHt, smem, st>>>(h->tm_ht_i, h->tm_ht_j, h->ht_cst, vhl, h->ht_table, w.units, out, h->ldn, c1, c2,
-                                      h->err_flag);
+                                      SYM ? ht_vmax(h) : nullptr, log2_up(h->n), log2_up(2 * ht_addends(h)), h->err_flag);
   prof_mark(h, 1, false, st);
   h->launches++;
   return cudaGetLastError();
@@ -607,7 +721,7 @@ static cudaError_t ht_scratch(Handle* h, int m, int M, cudaStream_t st) {
   const bool sym = m == 1;
   cudaError_t e = ht_units(h, sym, st);
   if (e != cudaSuccess) return e;
-  const size_t vbytes = (size_t)h->ldn * M * sizeof(float2) + (sym ? (size_t)h->ldn * sizeof(double) : 0);
+  const size_t vbytes = (size_t)h->ldn * M * sizeof(float2) + (sym ? (size_t)kPlanes * h->ldn * sizeof(double) : 0);
   if ((e = ht_buffer(h, &h->v32, &h->v32_cap, vbytes)) != cudaSuccess || sym) return e;
   return ht_buffer(h, &h->part, &h->part_cap, (size_t)h->ht_work[1].parts * h->ldn * M * sizeof(double));
 }
@@ -639,7 +753,8 @@ cudaError_t gram_high_tc(Handle* h, const double* V, double* U, int m, cudaStrea
   cudaError_t e;
   float2* vhl = reinterpret_cast<float2*>(h->v32);
   double* acc = sym ? reinterpret_cast<double*>(vhl + h->ldn * M) : reinterpret_cast<double*>(h->part);
-  ht_split_kernel<<<grid_for(h->ldn * M), 256, 0, st>>>(V, vhl, sym ? acc : nullptr, h->n, h->ldn, m, M);
+  ht_split_kernel<<<grid_for(h->ldn * M), 256, 0, st>>>(V, vhl, sym ? acc : nullptr, h->n, h->ldn, m, M,
+                                                         sym ? ht_vmax(h) : nullptr);
   h->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   switch (M) {
@@ -649,7 +764,7 @@ cudaError_t gram_high_tc(Handle* h, const double* V, double* U, int m, cudaStrea
     default: e = ht_launch<8, false>(h, vhl, acc, st); break;
   }
   if (e != cudaSuccess) return e;
-  ht_finish_kernel<<<grid_for(h->n * m), 256, 0, st>>>(acc, parts, h->ldn, M, m, h->n, U);
+  ht_finish_kernel<<<grid_for(h->n * m), 256, 0, st>>>(acc, parts, h->ldn, M, m, h->n, U, sym ? ht_vmax(h) : nullptr);
   h->launches++;
   return cudaGetLastError();
 }

@@ -337,6 +337,8 @@ enum Scal {
   S_RZN = 22, S_CGST = 23, S_CGITS = 24, S_TOL2 = 25, S_PEND = 26, S_MAXIT = 27, S_GAM = 28, S_PP = 29,
   // preconditioner: bits of max L^{-1}, exponent that scales the current r, max |r| where the caller gives no norm
   S_WMAX = 30, S_WEXP = 31, S_WMAXR = 32,
+  // FP64-class RBF product of one vector: bits of max |v| (zero between products), its results' unit
+  S_HTMAX = 33, S_HTUNIT = 34,
   S_COUNT = 40
 };
 
