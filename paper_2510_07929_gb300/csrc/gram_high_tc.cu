@@ -5,13 +5,15 @@
 // Each coordinate is an integer H = rint(xs 2^59), cut into seven balanced base-512 digits
 // d_6 .. d_0 (|d| <= 256, exact in bf16, stored as d 2^(9 s - 59) 2^10, so that the sums come out in
 // units the epilogue can convert without a multiplication).  The product of digits s and t has weight
-// 2^(9 (s + t) - 118) in the cross term, so the 28 digit pairs with s + t >= 6 give the
-// cross term to about 2^-53 (the dropped ones are below 2^-54).  They run as kind::f16 MMAs (bf16
+// 2^(9 (s + t) - 118) in the cross term.  The 28 digit pairs with s + t >= 6 are taken; the first level
+// dropped is at most 6 p 2^16 2^-73 = 2^-49.4 at p = 32 (digits all of magnitude 256 and of one sign;
+// about 2^-54 for digits without correlation).  They run as kind::f16 MMAs (bf16
 // A and B, FP32 accumulators in tensor memory), grouped by level l = s + t so that the sums the
 // exponent needs exactly are exact integers below 2^24 units:
 //   A = levels 12 + 11 (|sum| <= |xs_i||xs_j| < 28 = 2^23.8 units of 2^-19),
 //   B = level 10 and C = level 9 (at most 4 p 2^16 <= 2^23 units),
-//   D = levels 8 + 7 + 6 (below 2^-26: FP32 rounding leaves 2^-50).
+//   D = levels 8 + 7 + 6 (at most 5 p 2^16 2^-46 = 2^-22.7 and a little, so an FP32 rounding is up to
+//   2^-47; about 2^-26 and 2^-50 for digits without correlation).
 // The epilogue adds them to the norms (two int32 words and a float per point) in fixed point:
 // integer part, 12-bit table index (4096-entry double-float table of 2^-(k/4096)) and a remainder
 // below 2^-12, whose exponential needs one float polynomial; entry and sums are double-float.
