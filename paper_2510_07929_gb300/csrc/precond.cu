@@ -35,25 +35,39 @@ namespace kqr {
 // n = 20011, r = 1024, and a conversion of F besides.  Here a product is an FP32 factor (F
 // itself, exact) times a double-float (w U, or F of the set-up, as hi + lo): 11 FP32 pipe
 // operations with the TwoSum accumulation, 128 lanes per clock and SM instead of 2.  The
-// double-float sums run over kCgRows rows only and are then added to FP64 sums: their rounding
-// error grows with the square of the rows summed, and at 32 rows it is below that of the long
-// FP64 sum it replaces (64 rows: 6.6 instead of 7.2 ms, but a larger error).  w is scaled by the power of two that
-// brings its maximum to [1, 2), so that hi and lo stay inside the FP32 range.
+// double-float sums run over kCgRows rows only, renormalised every 4, and are then added to FP64 sums.
+// Their low part is a plain float sum, whose rounding grows with the rows of a group, where the rounding
+// of the FP64 sum that it replaces grows with all rows.  Against 64 bits the apply of such a core errs
+// as much as that of an FP64 core, or less, at n = 12000 .. 30000 (geometric means over systems of five
+// kinds of diagonal; groups of 32 rows not renormalised: up to 1.7 times as much); at n = 1000 it
+// erred two to three times as much.  So up to kCgCompRows rows the low part is summed with its rounding errors
+// kept (COMP, 23 operations a product instead of 11), which is at or below FP64's error at every size;
+// such a core is small.  w is scaled by the power of two that brings its maximum to [1, 2), so that hi
+// and lo stay inside the FP32 range.
 //
 // Tile: 64 x 64 entries per CTA of 128 threads, 4 x 8 per thread (32 independent chains; the
 // operands of a row are 20 shared-memory words for 352 FP32 operations).  The rows are cut into
 // chunks so that about two waves of CTAs exist at every (n, r): with a fixed chunk of 4096 rows
 // a rank-45 core at n = 2000 ran on 3 CTAs (707 us, now 26).  n = 20011, r = 1024: 21.1 ms
-// before, 7.2 ms now; the FP32 pipe alone would take 3.4 ms, the rest is the operand split and
-// the FP64 additions.
+// before, 8.5 ms now; the FP32 pipe alone would take 3.4 ms, the rest is the operand split and
+// the FP64 additions (7.2 ms with groups of 32 rows, whose error was larger).
 constexpr int kCT = 64;      // core tile
 constexpr int kCR = 16;      // rows per shared-memory step
-constexpr int kCgRows = 32;  // rows per double-float sum
+constexpr int kCgRows = 16;  // rows per double-float sum
 constexpr int kCgThreads = 128;
+constexpr int64_t kCgCompRows = 8192;   // rows up to which the low parts are compensated
+
+// s + e = a + b exactly, s = fl(a + b)
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
 
 // T: float (the FP32 factor, weights w; both triangles of G are written) or double (the set-up's FP64 factor, no weights).
-template <typename T>
-__global__ void __launch_bounds__(kCgThreads, 3)
+template <typename T, bool COMP>
+__global__ void __launch_bounds__(kCgThreads, COMP ? 2 : 3)
     core_gram_kernel(const T* __restrict__ F, int64_t ldf, int rr, int ncols, int64_t n, const double* __restrict__ w,
                      const unsigned long long* __restrict__ wmax, double* __restrict__ G, int ntile,
                      int64_t chunk) {
@@ -90,11 +104,14 @@ __global__ void __launch_bounds__(kCgThreads, 3)
   const int64_t i0 = (int64_t)blockIdx.y * chunk;
   const int64_t i1 = min(n, i0 + chunk);
   for (int64_t ig = i0; ig < i1; ig += kCgRows) {
-    float sh[4][8];
+    float sh[4][8], sll[COMP ? 4 : 1][COMP ? 8 : 1];   // sll: what the low sums' roundings left
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < 8; ++b) sh[a][b] = 0.f;
+      for (int b = 0; b < 8; ++b) {
+        sh[a][b] = 0.f;
+        if (COMP) sll[COMP ? a : 0][COMP ? b : 0] = 0.f;
+      }
     if (!kPair) {
       __syncthreads();
       if (tid < kCgRows) {
@@ -130,6 +147,16 @@ __global__ void __launch_bounds__(kCgThreads, 3)
       __syncthreads();
 #pragma unroll 2
       for (int k = 0; k < kCR; ++k) {
+        if (!COMP && k > 0 && k % 4 == 0) {   // renormalise, so that the low sums' roundings stay small
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+              const float v = __fadd_rn(sh[a][b], sl[a][b]);
+              sl[a][b] = __fsub_rn(sl[a][b], __fsub_rn(v, sh[a][b]));
+              sh[a][b] = v;
+            }
+        }
         const float4 a4 = *reinterpret_cast<const float4*>(&Ah[k][la]);
         const float4 h0 = *reinterpret_cast<const float4*>(&Bh[k][lb]);
         const float4 h1 = *reinterpret_cast<const float4*>(&Bh[k][32 + lb]);
@@ -150,13 +177,18 @@ __global__ void __launch_bounds__(kCgThreads, 3)
             const float p = __fmul_rn(xa[a], yh[b]);
             float e = fmaf(xa[a], yh[b], -p);
             e = fmaf(xa[a], yl[b], e);
-            if (kPair) e = fmaf(xl[a], yh[b], e);
-            // TwoSum
-            const float s = __fadd_rn(sh[a][b], p);
-            const float bb = __fsub_rn(s, sh[a][b]);
-            const float er = __fadd_rn(__fsub_rn(sh[a][b], __fsub_rn(s, bb)), __fsub_rn(p, bb));
-            sh[a][b] = s;
-            sl[a][b] = __fadd_rn(sl[a][b], __fadd_rn(er, e));
+            if (kPair) e = fmaf(xl[a], yh[b], fmaf(xl[a], yl[b], e));
+            float er;
+            sh[a][b] = two_sum(sh[a][b], p, er);
+            if (COMP) {
+              float g0, g1;
+              const float g = two_sum(er, e, g0);
+              sl[a][b] = two_sum(sl[a][b], g, g1);
+              float& c = sll[COMP ? a : 0][COMP ? b : 0];
+              c = __fadd_rn(c, __fadd_rn(g0, g1));
+            } else {
+              sl[a][b] = __fadd_rn(sl[a][b], __fadd_rn(er, e));
+            }
           }
       }
     }
@@ -167,6 +199,7 @@ __global__ void __launch_bounds__(kCgThreads, 3)
         // renormalise, so that one FP64 addition takes all but a remainder below half an ulp of it
         const float v = __fadd_rn(sh[a][b], sl[a][b]);
         sl[a][b] = __fsub_rn(sl[a][b], __fsub_rn(v, sh[a][b]));
+        if (COMP) sl[a][b] = __fadd_rn(sl[a][b], sll[COMP ? a : 0][COMP ? b : 0]);
         tot[a][b] += (double)v;
       }
   }
@@ -197,7 +230,8 @@ static cudaError_t core_gram(Handle* h, const T* F, int64_t ldf, int rr, bool on
   int64_t chunk = (h->n + want - 1) / want;
   chunk = (chunk + kCgRows - 1) / kCgRows * kCgRows;
   const int chunks = (int)((h->n + chunk - 1) / chunk);
-  core_gram_kernel<T><<<dim3(pairs, chunks), kCgThreads, 0, st>>>(F, ldf, rr, ncols, h->n, w, wmax, G, ntile, chunk);
+  auto kern = h->n <= kCgCompRows ? core_gram_kernel<T, true> : core_gram_kernel<T, false>;
+  kern<<<dim3(pairs, chunks), kCgThreads, 0, st>>>(F, ldf, rr, ncols, h->n, w, wmax, G, ntile, chunk);
   h->launches++;
   return cudaGetLastError();
 }
@@ -225,35 +259,36 @@ __global__ void recip_kernel(double* out, const double* L, int64_t n, unsigned l
 // What bounds it: reading F twice (80 MB each at n = 20011, r = 1024: from L2, beyond that from
 // HBM).  On the FP64 pipe the two passes cost 2 r n FMAs at 2 per clock and SM plus a conversion
 // of every F entry at the same rate, 160 and 334 us at that size with the latency of one thread
-// per row.  Here every product is FP32 x double-float (11 FP32-pipe operations, as in the core):
-// L^{-1} r and the core's result are split once into hi + lo, after scaling by powers of two
-// (the exponent of ||r|| and of max L^{-1}) that keep both parts inside the FP32 range for any r.
-// Sums run in double-float over at most 32 terms between renormalisations and are combined in
-// FP64.  Measured (n = 20011, r = 1024, cold caches): 37 and 68 us.
-// (sh, sl) += x (yh + yl), x FP32.
-__device__ __forceinline__ void df_mac(float& sh, float& sl, float x, float yh, float yl) {
-  const float p = __fmul_rn(x, yh);
-  const float e = fmaf(x, yl, fmaf(x, yh, -p));
-  const float s = __fadd_rn(sh, p);
-  const float bb = __fsub_rn(s, sh);
-  const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  sh = s;
-  sl = __fadd_rn(sl, __fadd_rn(er, e));
-}
-// (sh, sl) += (yh, yl), renormalised.
-__device__ __forceinline__ void df_add(float& sh, float& sl, float yh, float yl) {
-  const float s = __fadd_rn(sh, yh);
-  const float bb = __fsub_rn(s, sh);
-  const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(yh, bb));
-  const float l = __fadd_rn(__fadd_rn(sl, yl), er);
-  sh = __fadd_rn(s, l);
-  sl = __fsub_rn(l, __fsub_rn(sh, s));
-}
-__device__ __forceinline__ void df_renorm(float& sh, float& sl) {
-  const float v = __fadd_rn(sh, sl);
-  sl = __fsub_rn(sl, __fsub_rn(v, sh));
-  sh = v;
-}
+// per row.  Here every product is FP32 x double-float: L^{-1} r and the core's result are split once
+// into hi + lo, after scaling by powers of two (the exponent of ||r|| and of max L^{-1}) that keep both
+// parts inside the FP32 range for any r.  Sums are three floats (23 FP32-pipe operations a product: the
+// roundings of the low sums are summed too); as double-floats, 11 operations, the apply's error was two
+// to three times that of FP64 passes on well-conditioned systems (n = 1000 .. 20000, ranks from 200),
+// like this it is FP64's.  Measured (n = 20011, r = 1024): 42 and 37 us (passes in FP64: 160 and 334).
+// Sum of three floats, (h + l + ll) += x (yh + yl), x FP32.
+struct Sum3 {
+  float h = 0.f, l = 0.f, ll = 0.f;
+  __device__ __forceinline__ void mac(float x, float yh, float yl) {
+    const float p = __fmul_rn(x, yh);
+    const float e = fmaf(x, yl, fmaf(x, yh, -p));
+    float er, g0, g1;
+    h = two_sum(h, p, er);
+    const float g = two_sum(er, e, g0);
+    l = two_sum(l, g, g1);
+    ll = __fadd_rn(ll, __fadd_rn(g0, g1));
+  }
+  __device__ __forceinline__ void add(float yh, float yl, float yll) {
+    float er, e0, e1;
+    h = two_sum(h, yh, er);
+    l = two_sum(l, yl, e0);
+    l = two_sum(l, er, e1);
+    ll = __fadd_rn(__fadd_rn(ll, yll), __fadd_rn(e0, e1));
+  }
+  __device__ __forceinline__ void add_lane(int o) {
+    add(__shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o), __shfl_xor_sync(0xffffffffu, ll, o));
+  }
+  __device__ __forceinline__ double value() const { return (double)h + ((double)l + (double)ll); }
+};
 
 // bits of max |r|
 __global__ void absmax_kernel(const double* __restrict__ rv, int64_t n, unsigned long long* __restrict__ out) {
@@ -299,7 +334,7 @@ __global__ void __launch_bounds__(256) ut_kernel(const float* __restrict__ F, in
   __syncthreads();
   const int c0 = blockIdx.y * 32 + warp * 4;
   if (c0 > r) return;
-  float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
+  Sum3 sum[4];
   const float* Fc[4];
 #pragma unroll
   for (int c = 0; c < 4; ++c) Fc[c] = F + (size_t)min(c0 + c, r > 0 ? r - 1 : 0) * ldf + i0;
@@ -314,45 +349,29 @@ __global__ void __launch_bounds__(256) ut_kernel(const float* __restrict__ F, in
     const float4 ul = *reinterpret_cast<const float4*>(su + rows + k);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      df_mac(sh[c], sl[c], f[c].x, uh.x, ul.x);
-      df_mac(sh[c], sl[c], f[c].y, uh.y, ul.y);
-      df_mac(sh[c], sl[c], f[c].z, uh.z, ul.z);
-      df_mac(sh[c], sl[c], f[c].w, uh.w, ul.w);
+      sum[c].mac(f[c].x, uh.x, ul.x);
+      sum[c].mac(f[c].y, uh.y, ul.y);
+      sum[c].mac(f[c].z, uh.z, ul.z);
+      sum[c].mac(f[c].w, uh.w, ul.w);
     }
   }
   // reduce-scatter: lane bits 4 and 3 select the column, then the lanes of a column are added
-#pragma unroll
-  for (int c = 0; c < 4; ++c) df_renorm(sh[c], sl[c]);
   const bool u4 = (lane & 16) != 0, u3 = (lane & 8) != 0;
+  auto exchange = [](Sum3& keep, const Sum3& other, bool up, int o) {   // up lanes keep `other`, the rest `keep`
+    const Sum3 send = up ? keep : other;
+    if (up) keep = other;
+    keep.add(__shfl_xor_sync(0xffffffffu, send.h, o), __shfl_xor_sync(0xffffffffu, send.l, o),
+             __shfl_xor_sync(0xffffffffu, send.ll, o));
+  };
+  exchange(sum[0], sum[2], u4, 16);
+  exchange(sum[1], sum[3], u4, 16);
+  exchange(sum[0], sum[1], u3, 8);
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    const float gh = __shfl_xor_sync(0xffffffffu, u4 ? sh[c] : sh[c + 2], 16);
-    const float gl = __shfl_xor_sync(0xffffffffu, u4 ? sl[c] : sl[c + 2], 16);
-    if (u4) {
-      sh[c] = sh[c + 2];
-      sl[c] = sl[c + 2];
-    }
-    df_add(sh[c], sl[c], gh, gl);
-  }
-  {
-    const float gh = __shfl_xor_sync(0xffffffffu, u3 ? sh[0] : sh[1], 8);
-    const float gl = __shfl_xor_sync(0xffffffffu, u3 ? sl[0] : sl[1], 8);
-    if (u3) {
-      sh[0] = sh[1];
-      sl[0] = sl[1];
-    }
-    df_add(sh[0], sl[0], gh, gl);
-  }
-#pragma unroll
-  for (int o = 4; o >= 1; o >>= 1) {
-    const float gh = __shfl_xor_sync(0xffffffffu, sh[0], o);
-    const float gl = __shfl_xor_sync(0xffffffffu, sl[0], o);
-    df_add(sh[0], sl[0], gh, gl);
-  }
+  for (int o = 4; o >= 1; o >>= 1) sum[0].add_lane(o);
   const int col = c0 + (u4 ? 2 : 0) + (u3 ? 1 : 0);
   if ((lane & 7) == 0 && col <= r) {
     const int ew = max_exponent(*reinterpret_cast<const unsigned long long*>(scal + S_WMAX));
-    atomicAdd(&t[col], (((double)sh[0] + (double)sl[0]) * pow2((int)scal[S_WEXP])) * pow2(ew));
+    atomicAdd(&t[col], (sum[0].value() * pow2((int)scal[S_WEXP])) * pow2(ew));
   }
 }
 
@@ -387,7 +406,7 @@ __global__ void __launch_bounds__(256) woodbury_out_kernel(const float* __restri
                                                            unsigned int* __restrict__ counter,
                                                            double* __restrict__ rz) {
   extern __shared__ float2 ts[];   // r + 1
-  __shared__ float2 red[2][8][32];
+  __shared__ float red[2][8][3][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int c = threadIdx.x; c <= r; c += 256) ts[c] = t2s[c];
   __syncthreads();
@@ -404,28 +423,29 @@ __global__ void __launch_bounds__(256) woodbury_out_kernel(const float* __restri
       li = Linv[i];
       ri = rv[i];
     }
-    float sh = 0.f, sl = 0.f;
+    Sum3 sum;
     int c = c0;
     for (; c + 16 <= c1; c += 16) {
       float f[16];
 #pragma unroll
       for (int u = 0; u < 16; ++u) f[u] = __ldg(Fi + (size_t)(c + u) * ldf);
 #pragma unroll
-      for (int u = 0; u < 16; ++u) df_mac(sh, sl, f[u], ts[c + u].x, ts[c + u].y);
-      df_renorm(sh, sl);
+      for (int u = 0; u < 16; ++u) sum.mac(f[u], ts[c + u].x, ts[c + u].y);
     }
 #pragma unroll 4
-    for (; c < c1; ++c) df_mac(sh, sl, __ldg(Fi + (size_t)c * ldf), ts[c].x, ts[c].y);
-    df_renorm(sh, sl);
-    red[buf][warp][lane] = make_float2(sh, sl);
+    for (; c < c1; ++c) sum.mac(__ldg(Fi + (size_t)c * ldf), ts[c].x, ts[c].y);
+    red[buf][warp][0][lane] = sum.h;
+    red[buf][warp][1][lane] = sum.l;
+    red[buf][warp][2][lane] = sum.ll;
     __syncthreads();
     if (warp == 0) {
-      sh = ts[r].x;
-      sl = ts[r].y;
+      sum.h = ts[r].x;
+      sum.l = ts[r].y;
+      sum.ll = 0.f;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) df_add(sh, sl, red[buf][w][lane].x, red[buf][w][lane].y);
+      for (int w = 0; w < 8; ++w) sum.add(red[buf][w][0][lane], red[buf][w][1][lane], red[buf][w][2][lane]);
       if (i < n) {
-        const double o = li * (ri - ((double)sh + (double)sl) * unscale);
+        const double o = li * (ri - sum.value() * unscale);
         out[i] = o;
         dot = fma(ri, o, dot);
       }
