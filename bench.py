@@ -14,6 +14,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -28,13 +29,15 @@ sys.path.insert(0, ROOT)
 
 METRIC = "KQR solve sec to KKT≤1e-6 at n=200k; fused K·V TFLOP/s and % of roofline"
 FP32_LANES_PER_SM = 128          # FP32 FFMA/FADD lanes per SM (measured unit rate, see the design notes)
+INT_SAD_LANES_PER_SM = 64        # integer sums of absolute differences per SM and clock (microbenchmark)
 XU_LANES_PER_SM = 32             # MUFU ex2 per SM and clock (microbenchmark; ncu's XU-pipe counter agrees)
 TF32_PER_BF16 = 1.1 / 2.25       # nominal dense TF32 / bf16 tensor rate
 SM_COUNT_FALLBACK = 152          # used only when the device cannot be queried
 SM_MAX_MHZ_FALLBACK = 2070.0     # used only when nvidia-smi gives no maximum clock
 # DRAM bytes (read + write) per launch of gram_f32_sym_kernel on the n = 200000, p = 50
-# Laplacian workload, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum).
-SYM_LAPLACIAN_TRAFFIC = {(200000, 50): 42469632 + 8192}
+# Laplacian workload, from one ncu capture each (dram__bytes_read.sum + dram__bytes_write.sum) of the
+# form with all features in FP32 and of the one with 21 of them on the integer pipe.
+SYM_LAPLACIAN_TRAFFIC = {(200000, 50, 0): 42469632 + 8192, (200000, 50, 21): 42150000 + 32000}
 # Rows of the workload the oracle's full reference solve uses (dense FP64, Alg. 1
 # then Alg. 2/3): the full n = 200000 problem is far beyond it in a bench run.
 REF_SUBSAMPLE_ROWS = 2000
@@ -269,6 +272,49 @@ def rbf_tc_roofline(n: int, p: int, launches: int, ms: float, sm_count: int, sm_
                                   + ("" if bf16 else " (fallback 1.9 PFLOP/s bf16)")}}
 
 
+def lap_int_features(X, gamma: float) -> int:
+    """Features whose distances the symmetric FP32-class Laplacian tiles form on the integer pipe (the
+    library's rule: from 12 features on, 0.42 p of them, where the fixed-point grid 2^-G of the FP64-class
+    layout has p 2^-G <= 2^-20)."""
+    n, p = X.shape
+    if p < 12:
+        return 0
+    R = float(np.max(X.max(axis=0) - X.min(axis=0))) * gamma / math.log(2.0)
+    G = 33 if R <= 0 else min(33, math.floor(math.log2(((1 << 30) - 1.0) / (p * R))))
+    return math.floor(0.42 * p + 0.5) if p * 2.0 ** -G <= 2.0 ** -20 else 0
+
+
+def lap_roofline(n: int, p: int, p_int: int, launches: int, ms: float, sm_count: int, sm_mhz: float) -> dict:
+    """The symmetric FP32-class Laplacian tiles, pipe by pipe: per entry two FP32 lane operations for each of
+    the p - p_int features of the FP32 pipe and two for the row and column sums, and one 64-lane integer
+    operation for each of the p_int others; n(n+1)/2 entries per launch."""
+    entries = float(n) * float(n + 1) / 2.0
+    avg_s = ms / launches / 1e3
+    ops = 2 * (p - p_int) + 2
+    peak = sm_count * FP32_LANES_PER_SM * sm_mhz * 1e6 / 1e12             # Top/s
+    achieved = entries * ops / avg_s / 1e12
+    int_peak = sm_count * INT_SAD_LANES_PER_SM * sm_mhz * 1e6 / 1e12
+    int_achieved = entries * p_int / avg_s / 1e12
+    flops_per_entry = 3 * p + 4             # sub, abs, add per feature; scale, exp, multiply, add
+    flop_achieved = entries * flops_per_entry / avg_s / 1e12
+    return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Top/s", "frac": achieved / peak,
+            "traffic": SYM_LAPLACIAN_TRAFFIC.get((n, p, p_int)), "traffic_unit": "bytes per launch",
+            "kernel": "gram_f32_sym_kernel (FP32-class Laplacian tiles, symmetric)",
+            "launches": launches, "avg_ms": ms / launches, "entries_per_launch": entries,
+            "work_per_entry": f"{ops} FP32-pipe lane operations (FADD, FADD|.| per feature of {p - p_int}; two FFMAs "
+                              f"for the row and column sums) and {p_int} integer sums of absolute differences",
+            "integer_pipe": {"achieved": int_achieved, "peak": int_peak, "unit": "Top/s", "frac": int_achieved / int_peak},
+            "lanes_frac": achieved / peak + int_achieved / int_peak,
+            "lanes_note": "the two pipes share lanes: their fractions add up to the bound",
+            "peak_basis": f"{sm_count} SMs (device query) x {FP32_LANES_PER_SM} FP32 lanes ({INT_SAD_LANES_PER_SM} for the "
+                          f"integer operation) x {sm_mhz:g} MHz (max SM clock sampled by nvidia-smi); derived from unit "
+                          f"counts and clocks",
+            "flop_convention": {
+                "achieved": flop_achieved, "peak": 2.0 * peak, "unit": "TFLOP/s", "frac": flop_achieved / (2.0 * peak),
+                "flops_per_entry": flops_per_entry, "entries": "n(n+1)/2 formed per launch",
+                "peak_basis": "SMs x 128 lanes x 2 flops (FFMA) x clock"}}
+
+
 def bench_config(wl, args, world: int) -> dict:
     """The bench line's config, shared by both arms."""
     return {"workload": describe(wl, args), "n": wl.n, "p": wl.p, "kernel": wl.kind, "rank0": args.rank0,
@@ -437,27 +483,7 @@ def run_ours(args):
         fold = float(wl.gamma * np.log2(np.e) * np.max(np.sum(xc * xc, axis=1))) < 60.0
         roofline = rbf_tc_roofline(n, p, n32, ms32, sm_count, sm_mhz, f16=fold and 3 * p <= 128)
     elif n32 > 0:
-        avg_s = ms32 / n32 / 1e3
-        ops_per_entry = 2 * p + 2               # FADD + FADD|.| per feature; FFMA with v_j and with v_i
-        flops_per_entry = 3 * p + 4             # sub, abs, add per feature; scale, exp, multiply, add
-        peak = sm_count * FP32_LANES_PER_SM * sm_mhz * 1e6 / 1e12         # Top/s, FP32 pipe lane operations
-        achieved = entries * ops_per_entry / avg_s / 1e12
-        flop_peak = 2.0 * peak                                               # FFMA = 2 flops per lane and clock
-        flop_achieved = entries * flops_per_entry / avg_s / 1e12
-        traffic = SYM_LAPLACIAN_TRAFFIC.get((n, p))
-        roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Top/s", "frac": achieved / peak,
-                    "traffic": traffic, "traffic_unit": "bytes per launch",
-                    "kernel": "gram_f32_sym_kernel (FP32 Gram tiles, symmetric)",
-                    "launches": n32, "avg_ms": ms32 / n32, "entries_per_launch": entries,
-                    "work_per_entry": f"{ops_per_entry} FP32-pipe lane operations (FADD, FADD|.| per feature; "
-                                      f"two FFMAs for the row and column sums; 42 % of the features take one 64-lane "
-                                      f"integer operation instead of two FP32 ones)",
-                    "peak_basis": f"{sm_count} SMs (device query) x {FP32_LANES_PER_SM} FP32 lanes x {sm_mhz:g} MHz "
-                                  f"(max SM clock sampled by nvidia-smi); derived from unit counts and clocks",
-                    "flop_convention": {
-                        "achieved": flop_achieved, "peak": flop_peak, "unit": "TFLOP/s", "frac": flop_achieved / flop_peak,
-                        "flops_per_entry": flops_per_entry, "entries": "n(n+1)/2 formed per launch",
-                        "peak_basis": "SMs x 128 lanes x 2 flops (FFMA) x clock"}}
+        roofline = lap_roofline(n, p, lap_int_features(wl.X, wl.gamma), n32, ms32, sm_count, sm_mhz)
     hp = {"launches": nhp, "avg_ms": (mshp / nhp) if nhp else None}
 
     line = {"metric": METRIC, "value": value, "unit": "s", "n_gpus": world, "steps": args.steps,
