@@ -71,7 +71,10 @@ __global__ void __launch_bounds__(kThreads, (M <= 2) ? 2 : 1)
 #pragma unroll
     for (int c = 0; c < M; ++c) racc[a][c] = 0.f;
 
-  if (!mbar_wait_bounded(&bars[0], 0, err)) return;
+  if (!mbar_wait_bounded(&bars[0], 0, err)) {
+    if (tid == 0) tile_drain(bars, min(jt1 - jt0, 1), err);
+    return;
+  }
 
   for (int t = jt0; t < jt1; ++t) {
     const int q = t - jt0;
@@ -95,7 +98,10 @@ __global__ void __launch_bounds__(kThreads, (M <= 2) ? 2 : 1)
 #pragma unroll
       for (int b = 0; b < 8; ++b) nj[b] = __ldg(nrm + col0 + b);
     }
-    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) return;
+    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) {
+      if (tid == 0) tile_drain(bars, min(q + 2, jt1 - jt0), err);
+      return;
+    }
 
     float acc[8][8];
 #pragma unroll

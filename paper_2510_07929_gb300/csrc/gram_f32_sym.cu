@@ -133,7 +133,10 @@ __global__ void __launch_bounds__(kThreads, 2)
   float racc[8];
 #pragma unroll
   for (int a = 0; a < 8; ++a) racc[a] = 0.f;
-  if (!mbar_wait_bounded(&bars[0], 0, err)) return;
+  if (!mbar_wait_bounded(&bars[0], 0, err)) {
+    if (tid == 0) tile_drain(bars, 1, err);
+    return;
+  }
 
   for (int t = jt0; t < jt1; ++t) {
     const int q = t - jt0;
@@ -150,7 +153,10 @@ __global__ void __launch_bounds__(kThreads, 2)
       vb[b] = __ldg(v32 + col0 + b);
       nj[b] = (KIND == SYM_RBF) ? __ldg(nrm + col0 + b) : 0.f;
     }
-    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) return;
+    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) {
+      if (tid == 0) tile_drain(bars, min(q + 2, jt1 - jt0), err);
+      return;
+    }
 
     float d[8][8];
     if (KIND == SYM_LAP_MIX) {

@@ -81,7 +81,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int mask_f = (1 << kTB) - 1;
   const int mask_r = (1 << shift_f) - 1;
 
-  if (!mbar_wait_bounded(&bars[0], 0, err)) return;
+  if (!mbar_wait_bounded(&bars[0], 0, err)) {
+    if (tid == 0) tile_drain(bars, min(jt1 - jt0, 1), err);
+    return;
+  }
 
   for (int t = jt0; t < jt1; ++t) {
     const int q = t - jt0;
@@ -100,7 +103,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       vh[b] = w.x;
       vl[b] = w.y;
     }
-    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) return;
+    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) {
+      if (tid == 0) tile_drain(bars, min(q + 2, jt1 - jt0), err);
+      return;
+    }
     const int32_t* HJs = HJ[s];
     const float* LJs = LJ[s];
 
@@ -279,7 +285,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const float scaleA = __int_as_float((127 + 23 - 2 * G) << 23);  // 2^(23 - 2G)
   const float scaleB = __int_as_float((127 - 2 * G) << 23);       // 2^-2G
 
-  if (!mbar_wait_bounded(&bars[0], 0, err)) return;
+  if (!mbar_wait_bounded(&bars[0], 0, err)) {
+    if (tid == 0) tile_drain(bars, min(jt1 - jt0, 1), err);
+    return;
+  }
 
   for (int t = jt0; t < jt1; ++t) {
     const int q = t - jt0;
@@ -291,7 +300,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       tma_load_2d(LJ[ns], &tm_l, (t + 1) * kTile, 0, &bars[1 + ns]);
       tma_load_2d(XJ[ns], &tm_x, (t + 1) * kTile, 0, &bars[1 + ns]);
     }
-    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) return;
+    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) {
+      if (tid == 0) tile_drain(bars, min(q + 2, jt1 - jt0), err);
+      return;
+    }
     const int32_t* HJs = HJ[s];
     const float* LJs = LJ[s];
     const float* XJs = XJ[s];

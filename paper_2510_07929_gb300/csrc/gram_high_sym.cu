@@ -117,7 +117,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int shift_f = G - kTBs;
   const int mask_f = (1 << kTBs) - 1;
   const int mask_r = (1 << shift_f) - 1;
-  if (!mbar_wait_bounded(&bars[0], 0, err)) return;
+  if (!mbar_wait_bounded(&bars[0], 0, err)) {
+    if (tid == 0) tile_drain(bars, 1, err);
+    return;
+  }
 
   for (int t = jt0; t < jt1; ++t) {
     const int q = t - jt0;
@@ -136,7 +139,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       vbh[b] = w.x;
       vbl[b] = w.y;
     }
-    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) return;
+    if (!mbar_wait_bounded(&bars[1 + s], (uint32_t)((q >> 1) & 1), err)) {
+      if (tid == 0) tile_drain(bars, min(q + 2, jt1 - jt0), err);
+      return;
+    }
     const int32_t* HJs = HJ[s];
     const float* LJs = LJ[s];
 

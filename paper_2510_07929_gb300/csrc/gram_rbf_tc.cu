@@ -18,7 +18,8 @@
 // MMAs.  Column tiles are split over
 // gridDim.y; per-split row sums are added in FP64 by a second kernel.
 // Every mbarrier wait is bounded; on a timeout the CTA records the error,
-// stops issuing work and frees its tensor memory.
+// stops issuing work, waits (bounded) for its own copies and MMAs and frees
+// its tensor memory.
 #include <algorithm>
 #include <vector>
 
@@ -268,7 +269,15 @@ __global__ void __launch_bounds__(256, 1)
       tc_fence_before();
     }
     __syncthreads();
-    if (*abort_flag) break;
+    if (*abort_flag) {
+      // no copy and no MMA of this CTA in flight when its tensor memory is freed (bounded); without an
+      // abort every one of them has been waited for
+      if (tid == 0) {
+        tile_drain(bars, min(nt, max(2, q + 1)), err);
+        mma_drain(bars + 3, max(0, q - 1), min(q + 1, nt), err);
+      }
+      break;
+    }
     // Stage (q + 1) & 1 held tile q - 1, whose MMAs completed above: refill it with tile q + 1.
     if (tid == 0 && q >= 1 && q + 1 < nt) load_tile(XJh[(q + 1) & 1], XJl[(q + 1) & 1], (jt0 + q + 1) * 128, &bars[1 + ((q + 1) & 1)]);
   }

@@ -40,7 +40,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 
 // Bounded wait on an mbarrier phase.  Gives up after max_polls polls (each
 // try_wait itself suspends for a hardware-chosen interval), records
-// kErrWaitTimeout in *err and returns false; the caller then leaves the kernel.
+// kErrWaitTimeout in *err and returns false; the caller then stops its work and drains what is in flight.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int* err,
                                                   uint32_t max_polls = (1u << 22)) {
   for (uint32_t i = 0; i < max_polls; ++i)
@@ -58,6 +58,21 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, in
           "r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
+}
+
+// For CTAs that double-buffer column tiles, bars[0] for the row tile and bars[1 + (k & 1)] for column tile
+// k: thread 0 calls it on its way out after a wait that gave up, so that the row tile's copy and the
+// last two of the `issued` column tiles' have landed (bounded) before the CTA can end.  On the normal
+// way out it has waited for each of them.
+static __device__ __noinline__ void tile_drain(uint64_t* bars, int issued, int* err) {
+  mbar_wait_bounded(&bars[0], 0, err);
+  for (int k = issued > 2 ? issued - 2 : 0; k < issued; ++k)
+    mbar_wait_bounded(&bars[1 + (k & 1)], (uint32_t)((k >> 1) & 1), err);
+}
+
+// The same for the MMAs of tiles k0 .. k1 - 1, committed to done[k & 1].
+static __device__ __noinline__ void mma_drain(uint64_t* done, int k0, int k1, int* err) {
+  for (int k = k0; k < k1; ++k) mbar_wait_bounded(&done[k & 1], (uint32_t)((k >> 1) & 1), err);
 }
 
 // Index of this thread's warp, the same register value in all its lanes: branches on it are uniform.

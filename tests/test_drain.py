@@ -41,3 +41,27 @@ def test_the_last_mmas_are_waited_for_on_every_way_out(name, kernel, wait):
     blocks = enclosing(b, m[0].start())
     assert not any("ok" in h for h in blocks), blocks
     assert not any(h.startswith(("for", "while")) for h in blocks), blocks
+
+
+# Kernels that double-buffer column tiles: thread 0 leaves after a wait that gave up only once the copies it has issued
+# have landed: one column tile before the loop, tiles 0 .. q + 1 at the wait for tile q.
+TILE_KERNELS = [("gram_f32.cu", "gram_f32_kernel"), ("gram_f32_sym.cu", "gram_f32_sym_kernel"),
+                ("gram_high.cu", "gram_lap_high_kernel"), ("gram_high.cu", "gram_rbf_emu_kernel"),
+                ("gram_high_sym.cu", "gram_lap_high_sym_kernel")]
+
+
+@pytest.mark.parametrize("name,kernel", TILE_KERNELS)
+def test_tile_kernels_drain_before_they_leave(name, kernel):
+    b = body(code(name), kernel)
+    waits = [m.start() for m in re.finditer(r"\bmbar_wait_bounded\(", b)]
+    assert len(waits) == 2 and len(re.findall(r"\breturn\b", b)) == 2
+    for w, issued in zip(waits, (r"(?:1|min\(jt1 - jt0, 1\))", r"min\(q \+ 2, jt1 - jt0\)")):
+        assert re.match(r"mbar_wait_bounded\([^;{]*\) \{\s*if \(tid == 0\) tile_drain\(bars, " + issued +
+                        r", err\);\s*return;\s*\}", b[w:]), b[w:w + 200]
+
+
+def test_plain_tensor_core_kernel_drains_on_abort():
+    b = body(code("gram_rbf_tc.cu"), "gram_rbf_tc_kernel")
+    abort = b[b.index("if (*abort_flag) {"):]
+    abort = abort[:abort.index("break;")]
+    assert "tile_drain(bars, min(nt, max(2, q + 1)), err);" in abort and "mma_drain(bars + 3, max(0, q - 1), min(q + 1, nt), err);" in abort
