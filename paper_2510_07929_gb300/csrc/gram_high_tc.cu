@@ -512,8 +512,10 @@ __global__ void __launch_bounds__(kThreadsHt, 1)
         if (SYM) {
           double* p = out + 2 * (ti * 128 + e);
           const double h1 = sums.first(v);
+          const double r1 = __dsub_rn(v, h1);
           atomicAdd(p, h1);
-          OrderFree::rest(p + 1, ldn, __dsub_rn(v, h1), sums.e2, sums.la);
+          if (sums.two_planes(v)) atomicAdd(p + 1, r1);
+          else OrderFree::rest(p + 1, ldn, r1, sums.e2, sums.la);
         } else out[((size_t)unit.w * ldn + ti * 128) * M + e] = v;
       }
     }
