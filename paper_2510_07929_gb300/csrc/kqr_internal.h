@@ -268,7 +268,7 @@ cudaError_t fill_L(Handle* h, double* L, double base, const double* dres, int64_
 // Bounded wait on an mbarrier nothing arrives on (the wait-timeout path; kqr_test_bounded_wait).
 cudaError_t launch_wait_probe(Handle* h, uint32_t max_polls, cudaStream_t st);
 
-// ---- preconditioner (woodbury.cu, rpchol.cu) -------------------------------------
+// ---- preconditioner (precond.cu, spd_inverse.cu) -----------------------------------
 kqr_status precond_build(Handle* h, const double* Ldiag, double gam, cudaStream_t st);
 // As precond_build, but keeps the current core when it was built for the same gam
 // and max_i |Lpre_i - Lcore_i| / Lcore_i <= rtol (the preconditioner stays SPD; only
